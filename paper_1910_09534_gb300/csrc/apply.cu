@@ -28,19 +28,15 @@
 #include <cstring>
 #include <type_traits>
 
+#include "block_mat.cuh"
 #include "internal.h"
 
 namespace sycsim {
 namespace {
 
 template <int K>
-struct MatP {
-    float2 m[(1 << K) * (1 << K)];
-};
-
-struct MatPtr {
-    const float2 *p;
-};
+using MatP = BlockMat<K>;
+using MatPtr = BlockMat<6>;
 
 struct DirectGeom {
     float2 *psi;
@@ -578,36 +574,13 @@ BlockPath block_path(int nbits, int k, const int *tpos, int precision)
     return BlockPath::CudaCore;
 }
 
-bool staging_slot_free(sim_t *h, int nbits, int k, const int *tpos, int precision)
+// A block's matrix travels as kernel parameters (k <= 5) or, at k = 6, through device memory.
+size_t block_staged_bytes(int k) { return k == 6 ? sizeof(float2) * 4096 : 0; }
+
+bool staging_slot_free(sim_t *h, int k)
 {
     // an event never recorded counts as complete
-    if (block_path(nbits, k, tpos, precision) != BlockPath::CudaCore)
-        return cudaEventQuery(h->frag_ev[h->frag_next]) != cudaErrorNotReady;
-    if (k == 6) return cudaEventQuery(h->mat6_ev[h->mat6_next]) != cudaErrorNotReady;
-    return true;
-}
-
-// Operands of a block staged once in device memory (CUDA graphs): tensor-core B fragments, or
-// the matrix of a 6-qubit block on CUDA cores; nothing for narrower CUDA-core blocks, whose
-// matrix travels as kernel parameters.
-size_t block_staged_bytes(int nbits, int k, const int *tpos, int precision)
-{
-    switch (block_path(nbits, k, tpos, precision)) {
-    case BlockPath::Tcgen05: return tcgen05_staged_bytes(k);
-    case BlockPath::MmaSync: return tc_staged_bytes(k, precision);
-    default: return k == 6 ? sizeof(float2) * 4096 : 0;
-    }
-}
-
-void block_build_staged(int nbits, int k, const int *tpos, const float2 *mat, int precision, void *h_out)
-{
-    switch (block_path(nbits, k, tpos, precision)) {
-    case BlockPath::Tcgen05: tcgen05_build_staged(k, mat, precision == SIM_BF16X3, h_out); break;
-    case BlockPath::MmaSync: tc_build_staged(k, mat, precision, h_out); break;
-    default:
-        if (k == 6) std::memcpy(h_out, mat, sizeof(float2) * 4096);
-        break;
-    }
+    return block_staged_bytes(k) == 0 || cudaEventQuery(h->mat6_ev[h->mat6_next]) != cudaErrorNotReady;
 }
 
 int launch_block_staged(sim_t *h, float2 *psi, int nbits, int k, const int *tpos, const float2 *mat,
@@ -615,18 +588,15 @@ int launch_block_staged(sim_t *h, float2 *psi, int nbits, int k, const int *tpos
 {
     int rc;
     if (red_grid) *red_grid = 0;
+    const float2 *mat6 = k == 6 ? static_cast<const float2 *>(d_staged) : nullptr;
     switch (block_path(nbits, k, tpos, precision)) {
     case BlockPath::Tcgen05:
-        rc = tcgen05_launch_staged(h, psi, nbits, k, tpos, precision == SIM_BF16X3, d_staged, st, red, red_grid);
+        rc = launch_apply_tcgen05(h, psi, nbits, k, tpos, mat, mat6, precision == SIM_BF16X3, st, red, red_grid);
         break;
-    case BlockPath::MmaSync: rc = tc_launch_staged(psi, nbits, k, tpos, precision, d_staged, st); break;
-    default:
-        rc = launch_apply_fp32(h, psi, nbits, k, tpos, mat, k == 6 ? static_cast<const float2 *>(d_staged) : nullptr,
-                               st);
-        break;
+    case BlockPath::MmaSync: rc = launch_apply_tc(psi, nbits, k, tpos, mat, mat6, precision, st); break;
+    default: rc = launch_apply_fp32(h, psi, nbits, k, tpos, mat, mat6, st); break;
     }
-    if (rc != 0)
-        return fail(h, SIM_E_CUDA, "apply (staged): launch failed: %s", cudaGetErrorString(cudaGetLastError()));
+    if (rc != 0) return fail(h, SIM_E_CUDA, "apply: kernel launch failed: %s", cudaGetErrorString(cudaGetLastError()));
     return SIM_OK;
 }
 
@@ -634,46 +604,23 @@ int launch_block_staged(sim_t *h, float2 *psi, int nbits, int k, const int *tpos
 int enqueue_block_on(sim_t *h, float2 *psi, int nbits, int k, const int *tpos, const float2 *mat,
                      int precision, cudaStream_t st)
 {
-    const BlockPath path = block_path(nbits, k, tpos, precision);
-    if (path == BlockPath::Tcgen05) {
-        const int ps = prof_begin(h, SIM_PROF_APPLY, 16.0 * std::ldexp(1.0, nbits), st);
-        const int rc = launch_apply_tcgen05(h, psi, nbits, k, tpos, mat, precision == SIM_BF16X3, st);
-        prof_end(h, ps, st);
-        if (rc != 0)
-            return fail(h, SIM_E_CUDA, "apply (tcgen05): launch failed: %s",
-                        cudaGetErrorString(cudaGetLastError()));
-        return SIM_OK;
-    }
-    if (path == BlockPath::MmaSync) {
-        const int ps = prof_begin(h, SIM_PROF_APPLY, 16.0 * std::ldexp(1.0, nbits), st);
-        const int rc = launch_apply_tc(h, psi, nbits, k, tpos, mat, precision, st);
-        prof_end(h, ps, st);
-        if (rc != 0)
-            return fail(h, SIM_E_CUDA, "apply (tensor cores): launch failed: %s",
-                        cudaGetErrorString(cudaGetLastError()));
-        return SIM_OK;
-    }
-    const float2 *mat6 = nullptr;
-    int slot6 = -1;
-    if (k == 6) {
-        const int slot = slot6 = h->mat6_next;
+    const size_t bytes = block_staged_bytes(k);
+    float2 *staged = nullptr;
+    int slot = -1;
+    if (bytes) {
+        slot = h->mat6_next;
         h->mat6_next = (slot + 1) % sim_s::kMat6Slots;
         SIM_CUDA_TRY(h, cudaEventSynchronize(h->mat6_ev[slot]));  // host staging slot free
-        std::memcpy(h->h_mat6 + 4096 * slot, mat, sizeof(float2) * 4096);
-        float2 *dst = h->d_mat6 + 4096 * slot;
-        SIM_CUDA_TRY(h, cudaMemcpyAsync(dst, h->h_mat6 + 4096 * slot, sizeof(float2) * 4096,
-                                        cudaMemcpyHostToDevice, st));
-        mat6 = dst;
+        std::memcpy(h->h_mat6 + 4096 * slot, mat, bytes);
+        staged = h->d_mat6 + 4096 * slot;
+        SIM_CUDA_TRY(h, cudaMemcpyAsync(staged, h->h_mat6 + 4096 * slot, bytes, cudaMemcpyHostToDevice, st));
     }
     const int ps = prof_begin(h, SIM_PROF_APPLY, 16.0 * std::ldexp(1.0, nbits), st);
-    const int rc = launch_apply_fp32(h, psi, nbits, k, tpos, mat, mat6, st);
+    const int rc = launch_block_staged(h, psi, nbits, k, tpos, mat, precision, staged, st);
     prof_end(h, ps, st);
     // the matrix slot is free again once this kernel, which reads it, has run (on any stream)
-    if (slot6 >= 0) SIM_CUDA_TRY(h, cudaEventRecord(h->mat6_ev[slot6], st));
-    if (rc != 0)
-        return fail(h, SIM_E_CUDA, "apply: kernel launch failed: %s",
-                    cudaGetErrorString(cudaGetLastError()));
-    return SIM_OK;
+    if (slot >= 0) SIM_CUDA_TRY(h, cudaEventRecord(h->mat6_ev[slot], st));
+    return rc;
 }
 
 int enqueue_block(sim_t *h, int k, const int *tpos, const float2 *mat, int precision)

@@ -11,8 +11,8 @@
 //    is then the two complex values member 4s + t of groups g and g + 8: one 8-byte load each.
 //  * N (output reals) in tiles of 8 = 4 members: columns 2t, 2t+1 are Re, Im of member 4n + t,
 //    so a thread's accumulator pairs are whole output amplitudes: one 8-byte store each.
-// The B fragments (R^T, permuted as above, split hi/lo for the 3xTF32 mode) are arranged
-// fragment-major on the host and staged once per CTA in shared memory.
+// The B fragments (R^T, permuted as above, split hi/lo for the 3xTF32 mode) are built from the
+// FP32 matrix once per CTA, fragment-major in shared memory.
 //
 // Accumulation: chaining many MMAs through one FP32 accumulator was measured to shrink the
 // state's norm systematically (the tensor cores' internal accumulation is not round-to-nearest):
@@ -32,7 +32,9 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
+#include "block_mat.cuh"
 #include "internal.h"
 
 namespace sycsim {
@@ -43,7 +45,6 @@ struct MmaGeom {
     uint64_t n_mtiles;      // tiles of 16 groups: 2^(nbits - k - 4)
     int tpos[kMaxK];        // ascending target bits
     uint64_t moff[64];      // offset of member j
-    const uint32_t *bfrag;  // [split][kstep][ntile][lane][2] TF32 bit patterns
 };
 
 __device__ __forceinline__ uint32_t to_tf32(float x)
@@ -84,18 +85,50 @@ __device__ __forceinline__ uint64_t insert_zero_bits_t(uint64_t x, const int *po
 #endif
 constexpr int mma_min_blocks(int k) { return k <= 4 ? 2 : (k == 5 ? SYCSIM_MMA_MINB5 : 1); }
 
+// Round an FP32 value to TF32 (nearest, ties away from zero) with the dropped bits zero.
+__device__ __forceinline__ uint32_t round_tf32(float x)
+{
+    uint32_t u = __float_as_uint(x);
+    if ((u & 0x7f800000u) == 0x7f800000u) return u & 0xffffe000u;  // inf/nan: truncate
+    u += 0x1000u;                                                  // half of the dropped 13 bits
+    return u & 0xffffe000u;
+}
+
+// The B fragments of one block into shared memory (all threads): B[k][n] = R^T, permuted: k = (step
+// s, column c): member 4s + (c & 3), Re for c < 4, Im for c >= 4; n = (tile m, column c'): member
+// 4m + c'/2, Re for even c', Im for odd c'.  With the split, hi then lo.  Splitting on the device
+// keeps the host's share of a block to copying its matrix (built there it cost 15-200 us a block).
 template <int K, bool kSplit>
-__global__ void __launch_bounds__(256, mma_min_blocks(K)) k_apply_mma(MmaGeom g)
+__device__ __forceinline__ void build_frag_tf32(const float2 *mat, uint32_t *sb)
+{
+    constexpr int D = 1 << K, NT = D / 4, PAIRS = (D / 4) * NT * 32;
+    for (int i = threadIdx.x; i < PAIRS; i += blockDim.x) {
+        const int lane = i & 31, n = (i >> 5) & (NT - 1), s = (i >> 5) / NT;
+        const int gid = lane >> 2, t = lane & 3;
+        const float2 m = mat[(4 * n + (gid >> 1)) * D + 4 * s + t];
+        const bool out_im = gid & 1;
+        const float b0 = out_im ? m.y : m.x;   // Re x -> (Re y: Mr, Im y: Mi)
+        const float b1 = out_im ? m.x : -m.y;  // Im x -> (Re y: -Mi, Im y: Mr)
+        const uint32_t h0 = round_tf32(b0), h1 = round_tf32(b1);
+        *reinterpret_cast<uint2 *>(sb + 2 * i) = make_uint2(h0, h1);
+        if constexpr (kSplit)
+            *reinterpret_cast<uint2 *>(sb + 2 * PAIRS + 2 * i) =
+                make_uint2(round_tf32(b0 - __uint_as_float(h0)), round_tf32(b1 - __uint_as_float(h1)));
+    }
+    __syncthreads();
+}
+
+template <int K, bool kSplit>
+__global__ void __launch_bounds__(256, mma_min_blocks(K)) k_apply_mma(const __grid_constant__ MmaGeom g,
+                                                                      const __grid_constant__ BlockMat<K> M)
 {
     constexpr int D = 1 << K;
     constexpr int KS = D / 4;  // k-steps (4 input members each)
     constexpr int NT = D / 4;  // n-tiles (4 output members each)
     constexpr int NC = NT < SYCSIM_MMA_NC ? NT : SYCSIM_MMA_NC;  // n-tiles per output chunk
-    constexpr int NSPLIT = kSplit ? 2 : 1;
     constexpr int FRAG_WORDS = KS * NT * 64;
     extern __shared__ uint32_t sb[];
-    for (int i = threadIdx.x; i < NSPLIT * FRAG_WORDS; i += blockDim.x) sb[i] = g.bfrag[i];
-    __syncthreads();
+    build_frag_tf32<K, kSplit>(block_mat_ptr(M), sb);
 
     const int lane = threadIdx.x & 31, gid = lane >> 2, t = lane & 3;
     const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
@@ -176,8 +209,33 @@ __device__ __forceinline__ void split_half2(float re, float im, uint32_t &hi, ui
     lo = *reinterpret_cast<const uint32_t *>(&l);
 }
 
+// The B fragments (hi, lo) of one block into shared memory (all threads): k rows 2t, 2t+1 | 2t+8,
+// 2t+9; n column gid, as half2 (Re-input, Im-input) of input member 8s + t (word 0) and 8s + 4 + t
+// (word 1) for output member 4n + gid/2.
 template <int K>
-__global__ void __launch_bounds__(256, mma_min_blocks(K)) k_apply_mma_f16x3(MmaGeom g)
+__device__ __forceinline__ void build_frag_f16(const float2 *mat, uint32_t *sb)
+{
+    constexpr int D = 1 << K, NT = D / 4, PAIRS = (D / 8) * NT * 32;
+    for (int i = threadIdx.x; i < PAIRS; i += blockDim.x) {
+        const int lane = i & 31, n = (i >> 5) & (NT - 1), s = (i >> 5) / NT;
+        const int gid = lane >> 2, t = lane & 3;
+        const bool out_im = gid & 1;
+        uint32_t hi[2], lo[2];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const float2 m = mat[(4 * n + (gid >> 1)) * D + 8 * s + 4 * j + t];
+            // coefficients of Re x and Im x
+            split_half2(out_im ? m.y : m.x, out_im ? m.x : -m.y, hi[j], lo[j]);
+        }
+        *reinterpret_cast<uint2 *>(sb + 2 * i) = make_uint2(hi[0], hi[1]);
+        *reinterpret_cast<uint2 *>(sb + 2 * PAIRS + 2 * i) = make_uint2(lo[0], lo[1]);
+    }
+    __syncthreads();
+}
+
+template <int K>
+__global__ void __launch_bounds__(256, mma_min_blocks(K)) k_apply_mma_f16x3(const __grid_constant__ MmaGeom g,
+                                                                            const __grid_constant__ BlockMat<K> M)
 {
     constexpr int D = 1 << K;
     constexpr int KS = D / 8;  // k-steps (8 input members each)
@@ -185,8 +243,7 @@ __global__ void __launch_bounds__(256, mma_min_blocks(K)) k_apply_mma_f16x3(MmaG
     constexpr int NC = NT < SYCSIM_MMA_NC ? NT : SYCSIM_MMA_NC;
     constexpr int FRAG_WORDS = KS * NT * 64;
     extern __shared__ uint32_t sb[];
-    for (int i = threadIdx.x; i < 2 * FRAG_WORDS; i += blockDim.x) sb[i] = g.bfrag[i];
-    __syncthreads();
+    build_frag_f16<K>(block_mat_ptr(M), sb);
 
     const int lane = threadIdx.x & 31, gid = lane >> 2, t = lane & 3;
     const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
@@ -253,152 +310,16 @@ __global__ void __launch_bounds__(256, mma_min_blocks(K)) k_apply_mma_f16x3(MmaG
     }
 }
 
-uint32_t pack_half2(float lo, float hi)
-{
-    const __half a = __float2half_rn(lo), b = __float2half_rn(hi);
-    uint16_t ua, ub;
-    std::memcpy(&ua, &a, 2);
-    std::memcpy(&ub, &b, 2);
-    return (uint32_t)ua | ((uint32_t)ub << 16);
-}
-
 template <int K>
 constexpr size_t f16x3_bytes() { return sizeof(uint32_t) * 2 * ((1 << K) / 8) * ((1 << K) / 4) * 64; }
-
-// Host: the B fragments (hi, lo) of one block, as the kernel reads them.
-template <int K>
-void build_f16x3(const float2 *mat, uint32_t *h_frag)
-{
-    constexpr int D = 1 << K, KS = D / 8, NT = D / 4;
-    constexpr int FRAG_WORDS = KS * NT * 64;
-    // B fragment (k rows 2t, 2t+1 | 2t+8, 2t+9; n column gid) as half2 (Re-input, Im-input)
-    // of input member 8s + t (b0) and 8s + 4 + t (b1) for output member 4n + gid/2.
-    for (int s = 0; s < KS; s++)
-        for (int n = 0; n < NT; n++)
-            for (int lane = 0; lane < 32; lane++) {
-                const int gid = lane >> 2, t = lane & 3;
-                const int o = 4 * n + (gid >> 1);
-                const bool out_im = gid & 1;
-                const size_t idx = ((size_t)(s * NT + n) * 32 + lane) * 2;
-                for (int j = 0; j < 2; j++) {
-                    const float2 m = mat[o * D + 8 * s + 4 * j + t];
-                    const float re_in = out_im ? m.y : m.x;   // coefficient of Re x
-                    const float im_in = out_im ? m.x : -m.y;  // coefficient of Im x
-                    const uint32_t hi = pack_half2(re_in, im_in);
-                    __half hr, hm;
-                    const uint16_t lo16 = (uint16_t)(hi & 0xffffu), hi16 = (uint16_t)(hi >> 16);
-                    std::memcpy(&hr, &lo16, 2);
-                    std::memcpy(&hm, &hi16, 2);
-                    h_frag[idx + j] = hi;
-                    h_frag[FRAG_WORDS + idx + j] =
-                        pack_half2(re_in - __half2float(hr), im_in - __half2float(hm));
-                }
-            }
-}
-
-// Launch with the fragments already in device memory.
-template <int K>
-int launch_f16x3_staged(float2 *psi, int nbits, const int *tpos, const uint32_t *d_frag, cudaStream_t st)
-{
-    constexpr int D = 1 << K;
-    constexpr size_t bytes = f16x3_bytes<K>();
-    MmaGeom g{};
-    g.psi = psi;
-    g.n_mtiles = 1ull << (nbits - K - 4);
-    for (int i = 0; i < K; i++) g.tpos[i] = tpos[i];
-    for (int j = 0; j < D; j++) {
-        uint64_t o = 0;
-        for (int b = 0; b < K; b++)
-            if ((j >> b) & 1) o += 1ull << tpos[b];
-        g.moff[j] = o;
-    }
-    g.bfrag = d_frag;
-    auto kern = k_apply_mma_f16x3<K>;
-    static std::atomic<uint64_t> smem_done{0};
-    if (bytes > 48 * 1024 && !smem_opt_in(kern, (int)bytes, smem_done)) return -1;
-    static const LaunchCfg cfg = [&] {  // once per instantiation, thread-safe
-        LaunchCfg c;
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess) return c;
-        if (cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return c;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c.occ, kern, 256, bytes) != cudaSuccess || c.occ < 1)
-            c.occ = 1;
-        c.ok = true;
-        return c;
-    }();
-    if (!cfg.ok) return -1;
-    const uint64_t need = (g.n_mtiles + 7) / 8;
-    const uint64_t grid = std::min<uint64_t>(need, (uint64_t)cfg.sms * cfg.occ);
-    kern<<<(unsigned)grid, 256, bytes, st>>>(g);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
-}
-
-template <int K>
-int launch_f16x3_k(float2 *psi, int nbits, const int *tpos, const float2 *mat, cudaStream_t st,
-                   uint32_t *h_frag, uint32_t *d_frag, cudaEvent_t ev)
-{
-    build_f16x3<K>(mat, h_frag);
-    if (cudaMemcpyAsync(d_frag, h_frag, f16x3_bytes<K>(), cudaMemcpyHostToDevice, st) != cudaSuccess) return -1;
-    const int rc = launch_f16x3_staged<K>(psi, nbits, tpos, d_frag, st);
-    // the staging slot is free again once this kernel, which reads it, has run (on any stream)
-    if (cudaEventRecord(ev, st) != cudaSuccess) return -1;
-    return rc;
-}
-
-// Round an FP32 value to TF32 (nearest, ties away from zero, as cvt.rna), host side.
-uint32_t host_tf32(float x)
-{
-    uint32_t u;
-    std::memcpy(&u, &x, 4);
-    if ((u & 0x7f800000u) == 0x7f800000u) return u & 0xffffe000u;  // inf/nan: truncate
-    u += 0x1000u;                                                   // half of the dropped 13 bits
-    return u & 0xffffe000u;
-}
-
-float tf32_value(uint32_t u)
-{
-    float f;
-    std::memcpy(&f, &u, 4);
-    return f;
-}
 
 template <int K, bool kSplit>
 constexpr size_t mma_bytes() { return sizeof(uint32_t) * (kSplit ? 2 : 1) * ((1 << K) / 4) * ((1 << K) / 4) * 64; }
 
-// Host: the B fragments (TF32; with the split, hi then lo) of one block.
-template <int K, bool kSplit>
-void build_mma(const float2 *mat, uint32_t *h_frag)
-{
-    constexpr int D = 1 << K, KS = D / 4, NT = D / 4;
-    constexpr int FRAG_WORDS = KS * NT * 64;
-    // B[k][n] = R^T, permuted: k = (step s, column c): member 4s + (c & 3), Re for c < 4, Im for
-    // c >= 4; n = (tile m, column c'): member 4m + c'/2, Re for even c', Im for odd c'.
-    for (int s = 0; s < KS; s++)
-        for (int n = 0; n < NT; n++)
-            for (int lane = 0; lane < 32; lane++) {
-                const int gid = lane >> 2, t = lane & 3;
-                const int i = 4 * s + t;            // input member (b0: Re part, b1: Im part)
-                const int o = 4 * n + (gid >> 1);   // output member
-                const bool out_im = gid & 1;
-                const float2 m = mat[o * D + i];
-                const float b0 = out_im ? m.y : m.x;   // Re x -> (Re y: Mr, Im y: Mi)
-                const float b1 = out_im ? m.x : -m.y;  // Im x -> (Re y: -Mi, Im y: Mr)
-                const size_t idx = ((size_t)(s * NT + n) * 32 + lane) * 2;
-                const uint32_t h0 = host_tf32(b0), h1 = host_tf32(b1);
-                h_frag[idx] = h0;
-                h_frag[idx + 1] = h1;
-                if (kSplit) {
-                    h_frag[FRAG_WORDS + idx] = host_tf32(b0 - tf32_value(h0));
-                    h_frag[FRAG_WORDS + idx + 1] = host_tf32(b1 - tf32_value(h1));
-                }
-            }
-}
-
-template <int K, bool kSplit>
-int launch_mma_staged(float2 *psi, int nbits, const int *tpos, const uint32_t *d_frag, cudaStream_t st)
+template <int K, size_t kBytes, void (*kern)(const MmaGeom, const BlockMat<K>)>
+int launch_mma(float2 *psi, int nbits, const int *tpos, const BlockMat<K> &M, cudaStream_t st)
 {
     constexpr int D = 1 << K;
-    constexpr size_t bytes = mma_bytes<K, kSplit>();
     MmaGeom g{};
     g.psi = psi;
     g.n_mtiles = 1ull << (nbits - K - 4);
@@ -409,16 +330,14 @@ int launch_mma_staged(float2 *psi, int nbits, const int *tpos, const uint32_t *d
             if ((j >> b) & 1) o += 1ull << tpos[b];
         g.moff[j] = o;
     }
-    g.bfrag = d_frag;
-    auto kern = k_apply_mma<K, kSplit>;
     static std::atomic<uint64_t> smem_done{0};
-    if (bytes > 48 * 1024 && !smem_opt_in(kern, (int)bytes, smem_done)) return -1;
+    if (kBytes > 48 * 1024 && !smem_opt_in(kern, (int)kBytes, smem_done)) return -1;
     static const LaunchCfg cfg = [&] {  // once per instantiation, thread-safe
         LaunchCfg c;
         int dev = 0;
         if (cudaGetDevice(&dev) != cudaSuccess) return c;
         if (cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return c;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c.occ, kern, 256, bytes) != cudaSuccess || c.occ < 1)
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c.occ, kern, 256, kBytes) != cudaSuccess || c.occ < 1)
             c.occ = 1;
         c.ok = true;
         return c;
@@ -426,20 +345,8 @@ int launch_mma_staged(float2 *psi, int nbits, const int *tpos, const uint32_t *d
     if (!cfg.ok) return -1;
     const uint64_t need = (g.n_mtiles + 7) / 8;
     const uint64_t grid = std::min<uint64_t>(need, (uint64_t)cfg.sms * cfg.occ);
-    kern<<<(unsigned)grid, 256, bytes, st>>>(g);
+    kern<<<(unsigned)grid, 256, kBytes, st>>>(g, M);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
-}
-
-template <int K, bool kSplit>
-int launch_mma_k(float2 *psi, int nbits, const int *tpos, const float2 *mat, cudaStream_t st,
-                 uint32_t *h_frag, uint32_t *d_frag, cudaEvent_t ev)
-{
-    build_mma<K, kSplit>(mat, h_frag);
-    if (cudaMemcpyAsync(d_frag, h_frag, mma_bytes<K, kSplit>(), cudaMemcpyHostToDevice, st) != cudaSuccess) return -1;
-    const int rc = launch_mma_staged<K, kSplit>(psi, nbits, tpos, d_frag, st);
-    // the staging slot is free again once this kernel, which reads it, has run (on any stream)
-    if (cudaEventRecord(ev, st) != cudaSuccess) return -1;
-    return rc;
 }
 
 }  // namespace
@@ -454,73 +361,21 @@ bool tc_eligible(int nbits, int k, const int *) { return k >= 5 && k <= 6 && nbi
 // 4.27 ms), {0,2,6,8}: 2.59 ms (3.57), {1,6,7,12}: 2.60 ms (3.24).
 bool tc_eligible_low4(int nbits, int k) { return k == 4 && nbits >= k + 4; }
 
-size_t tc_staged_bytes(int k, int precision)
-{
-    const bool f16 = f16x3_mode(precision), split = precision == SIM_TF32X3;
-    switch (k) {
-    case 4: return f16 ? f16x3_bytes<4>() : (split ? mma_bytes<4, true>() : mma_bytes<4, false>());
-    case 5: return f16 ? f16x3_bytes<5>() : (split ? mma_bytes<5, true>() : mma_bytes<5, false>());
-    case 6: return f16 ? f16x3_bytes<6>() : (split ? mma_bytes<6, true>() : mma_bytes<6, false>());
-    default: return 0;
-    }
-}
-
-void tc_build_staged(int k, const float2 *mat, int precision, void *h_out)
-{
-    uint32_t *o = static_cast<uint32_t *>(h_out);
-    const bool f16 = f16x3_mode(precision), split = precision == SIM_TF32X3;
-    switch (k) {
-    case 4: f16 ? build_f16x3<4>(mat, o) : (split ? build_mma<4, true>(mat, o) : build_mma<4, false>(mat, o)); break;
-    case 5: f16 ? build_f16x3<5>(mat, o) : (split ? build_mma<5, true>(mat, o) : build_mma<5, false>(mat, o)); break;
-    case 6: f16 ? build_f16x3<6>(mat, o) : (split ? build_mma<6, true>(mat, o) : build_mma<6, false>(mat, o)); break;
-    default: break;
-    }
-}
-
-int tc_launch_staged(float2 *psi, int nbits, int k, const int *tpos, int precision, const void *d_staged,
-                     cudaStream_t st)
-{
-    const uint32_t *d = static_cast<const uint32_t *>(d_staged);
-    const bool f16 = f16x3_mode(precision), split = precision == SIM_TF32X3;
-    switch (k) {
-    case 4: return f16 ? launch_f16x3_staged<4>(psi, nbits, tpos, d, st)
-                       : (split ? launch_mma_staged<4, true>(psi, nbits, tpos, d, st)
-                                : launch_mma_staged<4, false>(psi, nbits, tpos, d, st));
-    case 5: return f16 ? launch_f16x3_staged<5>(psi, nbits, tpos, d, st)
-                       : (split ? launch_mma_staged<5, true>(psi, nbits, tpos, d, st)
-                                : launch_mma_staged<5, false>(psi, nbits, tpos, d, st));
-    case 6: return f16 ? launch_f16x3_staged<6>(psi, nbits, tpos, d, st)
-                       : (split ? launch_mma_staged<6, true>(psi, nbits, tpos, d, st)
-                                : launch_mma_staged<6, false>(psi, nbits, tpos, d, st));
-    default: return -1;
-    }
-}
-
-int launch_apply_tc(sim_t *h, float2 *psi, int nbits, int k, const int *tpos, const float2 *mat,
+int launch_apply_tc(float2 *psi, int nbits, int k, const int *tpos, const float2 *mat, const float2 *mat6_dev,
                     int precision, cudaStream_t st)
 {
-    const int slot = h->frag_next;
-    h->frag_next = (slot + 1) % sim_s::kFragSlots;
-    if (cudaEventSynchronize(h->frag_ev[slot]) != cudaSuccess) return -1;  // host staging free
-    uint32_t *hf = h->h_frag + sim_s::kFragWords * slot;
-    uint32_t *df = h->d_frag + sim_s::kFragWords * slot;
-    cudaEvent_t ev = h->frag_ev[slot];
-    if (f16x3_mode(precision)) {
-        switch (k) {
-        case 4: return launch_f16x3_k<4>(psi, nbits, tpos, mat, st, hf, df, ev);
-        case 5: return launch_f16x3_k<5>(psi, nbits, tpos, mat, st, hf, df, ev);
-        case 6: return launch_f16x3_k<6>(psi, nbits, tpos, mat, st, hf, df, ev);
-        default: return -1;
-        }
-    }
-    const bool split = precision == SIM_TF32X3;
+    auto go = [&](auto kc) {
+        constexpr int K = decltype(kc)::value;
+        const BlockMat<K> M = block_mat<K>(mat, mat6_dev);
+        if (f16x3_mode(precision)) return launch_mma<K, f16x3_bytes<K>(), k_apply_mma_f16x3<K>>(psi, nbits, tpos, M, st);
+        if (precision == SIM_TF32X3)
+            return launch_mma<K, mma_bytes<K, true>(), k_apply_mma<K, true>>(psi, nbits, tpos, M, st);
+        return launch_mma<K, mma_bytes<K, false>(), k_apply_mma<K, false>>(psi, nbits, tpos, M, st);
+    };
     switch (k) {
-    case 4: return split ? launch_mma_k<4, true>(psi, nbits, tpos, mat, st, hf, df, ev)
-                         : launch_mma_k<4, false>(psi, nbits, tpos, mat, st, hf, df, ev);
-    case 5: return split ? launch_mma_k<5, true>(psi, nbits, tpos, mat, st, hf, df, ev)
-                         : launch_mma_k<5, false>(psi, nbits, tpos, mat, st, hf, df, ev);
-    case 6: return split ? launch_mma_k<6, true>(psi, nbits, tpos, mat, st, hf, df, ev)
-                         : launch_mma_k<6, false>(psi, nbits, tpos, mat, st, hf, df, ev);
+    case 4: return go(std::integral_constant<int, 4>{});
+    case 5: return go(std::integral_constant<int, 5>{});
+    case 6: return go(std::integral_constant<int, 6>{});
     default: return -1;
     }
 }

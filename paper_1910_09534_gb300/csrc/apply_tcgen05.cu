@@ -35,7 +35,7 @@
 //    read.  Blocks with two or more targets below bit 4 are left to the other kernels.
 // K (input reals) is interleaved, column 2m + p is part p (Re, Im) of member m, so a row's
 // 16-byte chunk is four consecutive members; N likewise.  R^T (hi, lo; FP16, core-matrix layout)
-// is built on the host and staged in shared memory once per CTA.  Two TMEM accumulator sets let
+// is split from the FP32 matrix into shared memory once per CTA.  Two TMEM accumulator sets let
 // tile i + 1 be multiplied while tile i is drained.
 //
 // BF16x3 (SIM_BF16X3) is the same pipeline with BF16 pieces (8 significant bits each instead of
@@ -51,7 +51,9 @@
 
 #include <algorithm>
 #include <cstring>
+#include <type_traits>
 
+#include "block_mat.cuh"
 #include "internal.h"
 
 namespace sycsim {
@@ -84,7 +86,6 @@ struct Tc5Geom {
     uint32_t ridx[8];        // staging-index bit of row bit j (bit 7: sub-tile)
     uint64_t roff[8];        // address offset of row bit j
     uint64_t moff[64];       // address offset of member m
-    const uint32_t *bmat;    // R^T hi then lo, FP16 core-matrix layout, as 32-bit words
     int *err;                // set to 1 if a wait timed out
     double *red;             // if set: this CTA's (sum p, sum p^2) of the results at red[2 blockIdx.x]
 };
@@ -276,6 +277,58 @@ __device__ __forceinline__ void swap_u32(uint32_t &a, uint32_t &b)
 
 __device__ __forceinline__ uint32_t cm_off(int row, int k) { return (row >> 3) * 256 + ((k >> 3) & 1) * 128 + (row & 7) * 16 + (k & 7) * 2; }
 
+template <bool BF>
+__device__ __forceinline__ void split_pair(float re, float im, uint32_t &hi, uint32_t &lo)
+{
+    if constexpr (BF) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(re, im);
+        const float2 hf = __bfloat1622float2(h);
+        const __nv_bfloat162 l = __floats2bfloat162_rn(re - hf.x, im - hf.y);
+        hi = *reinterpret_cast<const uint32_t *>(&h);
+        lo = *reinterpret_cast<const uint32_t *>(&l);
+    } else {
+        const __half2 h = __floats2half2_rn(re, im);
+        const float2 hf = __half22float2(h);
+        const __half2 l = __floats2half2_rn(re - hf.x, im - hf.y);
+        hi = *reinterpret_cast<const uint32_t *>(&h);
+        lo = *reinterpret_cast<const uint32_t *>(&l);
+    }
+}
+
+// R^T of the block into shared memory (all threads of the CTA): B[n][k], n = 2o + po output real,
+// k = 2i + pi input real, split hi / lo, K-major core matrices (KS slices of N x 16).  The matrix
+// arrives as it was composed (FP32) and every CTA splits it for itself: a thread takes four
+// neighbouring elements of a row o, which are one 16-byte chunk of each of the rows 2o, 2o + 1,
+// with consecutive threads on consecutive o (two-way bank conflicts on the stores).  1024 such
+// items at k = 6, two a thread, read from L2.  Built on the host instead (software FP16
+// conversions, 64 KiB uploaded a block) a 6-qubit block cost the calling thread 200 us, a 5-qubit
+// one 45 us, more than the pass itself below 2^25 amplitudes: a 20-qubit, 27-block plan took 1245
+// us instead of 251, one 5-qubit block on 22 qubits 56 instead of 18.
+template <int K, bool BF>
+__device__ __forceinline__ void build_b(const float2 *m, uint8_t *bHi, uint8_t *bLo, int tid, int nthreads)
+{
+    constexpr int D = 1 << K, B_SLICE = 2 * D * 32;
+    for (int it = tid; it < D * (D / 4); it += nthreads) {
+        const int o = it & (D - 1), i4 = it >> K;
+        const float4 *src = reinterpret_cast<const float4 *>(m + o * D + 4 * i4);
+        const float4 a = src[0], b = src[1];
+        const float re[4] = {a.x, a.z, b.x, b.z}, im[4] = {a.y, a.w, b.y, b.w};
+        uint32_t h0[4], l0[4], h1[4], l1[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            split_pair<BF>(re[j], -im[j], h0[j], l0[j]);  // row 2o: Re out
+            split_pair<BF>(im[j], re[j], h1[j], l1[j]);   // row 2o + 1: Im out
+        }
+        const int n = 2 * o;
+        const uint32_t off = (i4 >> 1) * B_SLICE + (n >> 3) * 256 + (i4 & 1) * 128 + (n & 7) * 16;
+        *reinterpret_cast<uint4 *>(bHi + off) = make_uint4(h0[0], h0[1], h0[2], h0[3]);
+        *reinterpret_cast<uint4 *>(bHi + off + 16) = make_uint4(h1[0], h1[1], h1[2], h1[3]);
+        *reinterpret_cast<uint4 *>(bLo + off) = make_uint4(l0[0], l0[1], l0[2], l0[3]);
+        *reinterpret_cast<uint4 *>(bLo + off + 16) = make_uint4(l1[0], l1[1], l1[2], l1[3]);
+    }
+    asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // B is read by the MMA unit
+}
+
 // Per tile i (local index; stage s = i % S, stage phase (i / S) & 1; TMEM set i % 2, set phase
 // (i / 2) & 1):
 //   loader: wait drained[s] of tile i - S, load the runs into stage s (loaded[s] counts bytes);
@@ -291,7 +344,8 @@ __device__ __forceinline__ uint32_t cm_off(int row, int k) { return (row >> 3) *
 // needs, and a TMEM set reused only after its read, so no barrier can run a phase ahead of a
 // waiter that still has to see the previous phase.
 template <int K, int R2, bool LOWT, bool BF>
-__global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tcgen05(Tc5Geom g)
+__global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tcgen05(const __grid_constant__ Tc5Geom g,
+                                                                  const __grid_constant__ BlockMat<K> M)
 {
     using L = Tc5Layout<K, R2>;
     constexpr bool BULK = L::BULK_STORE && !LOWT;  // results back through the stage
@@ -309,12 +363,7 @@ __global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tcgen05(Tc5Geom g)
     const int n_runs = (R2 << (K + 7)) >> g.run_log2;
     const uint32_t run_bytes = 8u << g.run_log2;
 
-    {
-        const uint32_t *src = g.bmat;
-        uint32_t *dst = reinterpret_cast<uint32_t *>(bHi);
-        for (int i = tid; i < (2 * L::B_BYTES) / 4; i += blockDim.x) dst[i] = src[i];
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // B is read by the MMA unit
-    }
+    build_b<K, BF>(block_mat_ptr(M), bHi, bLo, tid, kThreadsTc5);
     if (tid == 0) {
         for (int st = 0; st < S; ++st) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&loaded[st])) : "memory");
@@ -401,19 +450,7 @@ __global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tcgen05(Tc5Geom g)
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         const float re = x[u][4 * cc + j].x * sc, im = x[u][4 * cc + j].y * sc;
-                        if constexpr (BF) {
-                            const __nv_bfloat162 h = __floats2bfloat162_rn(re, im);
-                            const float2 hf = __bfloat1622float2(h);
-                            const __nv_bfloat162 l = __floats2bfloat162_rn(re - hf.x, im - hf.y);
-                            hi[j] = *reinterpret_cast<const uint32_t *>(&h);
-                            lo[j] = *reinterpret_cast<const uint32_t *>(&l);
-                        } else {
-                            const __half2 h = __floats2half2_rn(re, im);
-                            const float2 hf = __half22float2(h);
-                            const __half2 l = __floats2half2_rn(re - hf.x, im - hf.y);
-                            hi[j] = *reinterpret_cast<const uint32_t *>(&h);
-                            lo[j] = *reinterpret_cast<const uint32_t *>(&l);
-                        }
+                        split_pair<BF>(re, im, hi[j], lo[j]);
                     }
                     if constexpr (LOWT) {  // position p of the chunk takes register p ^ (mu & 3)
                         if (mu & 1) {
@@ -665,26 +702,9 @@ __device__ __forceinline__ void tmem_st16(uint32_t ta, const uint32_t *r)
         : "memory");
 }
 
-template <bool BF>
-__device__ __forceinline__ void split_pair(float re, float im, uint32_t &hi, uint32_t &lo)
-{
-    if constexpr (BF) {
-        const __nv_bfloat162 h = __floats2bfloat162_rn(re, im);
-        const float2 hf = __bfloat1622float2(h);
-        const __nv_bfloat162 l = __floats2bfloat162_rn(re - hf.x, im - hf.y);
-        hi = *reinterpret_cast<const uint32_t *>(&h);
-        lo = *reinterpret_cast<const uint32_t *>(&l);
-    } else {
-        const __half2 h = __floats2half2_rn(re, im);
-        const float2 hf = __half22float2(h);
-        const __half2 l = __floats2half2_rn(re - hf.x, im - hf.y);
-        hi = *reinterpret_cast<const uint32_t *>(&h);
-        lo = *reinterpret_cast<const uint32_t *>(&l);
-    }
-}
-
 template <bool LOWT, bool BF>
-__global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tc6a(Tc5Geom g)
+__global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tc6a(const __grid_constant__ Tc5Geom g,
+                                                               const __grid_constant__ BlockMat<6> M)
 {
     constexpr int D = 64, KS = 8, N = 128, S = kTc6Stages, H = D / 2;  // H members per thread
     constexpr int B_SLICE = N * 32;
@@ -700,12 +720,7 @@ __global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tc6a(Tc5Geom g)
     const int n_runs = (1 << (6 + 7)) >> g.run_log2;
     const uint32_t run_bytes = 8u << g.run_log2;
 
-    {
-        const uint32_t *src = g.bmat;
-        uint32_t *dst = reinterpret_cast<uint32_t *>(bHi);
-        for (int i = tid; i < (2 * kTc6BBytes) / 4; i += blockDim.x) dst[i] = src[i];
-        asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // B is read by the MMA unit
-    }
+    build_b<6, BF>(block_mat_ptr(M), bHi, bLo, tid, kThreadsTc5);
     if (tid == 0) {
         for (int st = 0; st < S; ++st) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&loaded[st])) : "memory");
@@ -910,58 +925,6 @@ __global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tc6a(Tc5Geom g)
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
 }
 
-uint16_t half_bits(float f)
-{
-    const __half h = __float2half_rn(f);
-    uint16_t u;
-    std::memcpy(&u, &h, 2);
-    return u;
-}
-
-float half_value(uint16_t u)
-{
-    __half h;
-    std::memcpy(&h, &u, 2);
-    return __half2float(h);
-}
-
-uint16_t bf16_bits(float f)
-{
-    const __nv_bfloat16 h = __float2bfloat16_rn(f);
-    uint16_t u;
-    std::memcpy(&u, &h, 2);
-    return u;
-}
-
-float bf16_value(uint16_t u)
-{
-    __nv_bfloat16 h;
-    std::memcpy(&h, &u, 2);
-    return __bfloat162float(h);
-}
-
-// Host: R^T = B[n][k] (n = 2o + po output real, k = 2i + pi input real), split hi/lo in FP16 (or
-// BF16), written in the K-major core-matrix layout, KS slices of N x 16.
-template <int K, bool BF>
-void build_b(const float2 *mat, uint16_t *out)
-{
-    using L = Tc5Layout<K, 1>;
-    constexpr int D = L::D, N = L::N;
-    uint16_t *hi = out, *lo = out + L::B_BYTES / 2;
-    for (int n = 0; n < N; n++)
-        for (int k = 0; k < 2 * D; k++) {
-            const int o = n >> 1, po = n & 1, i = k >> 1, pi = k & 1;
-            const float2 m = mat[o * D + i];
-            const float v = po == 0 ? (pi == 0 ? m.x : -m.y) : (pi == 0 ? m.y : m.x);
-            const uint16_t h = BF ? bf16_bits(v) : half_bits(v);
-            const uint16_t l = BF ? bf16_bits(v - bf16_value(h)) : half_bits(v - half_value(h));
-            const int s = k >> 4, kk = k & 15;
-            const size_t off = ((size_t)s * L::B_SLICE + (n >> 3) * 256 + (kk >> 3) * 128 + (n & 7) * 16 + (kk & 7) * 2) / 2;
-            hi[off] = h;
-            lo[off] = l;
-        }
-}
-
 // The tile's free address bits F (ascending): the targets and the `rows` lowest other bits.  The
 // staging index of an amplitude is its address bits on F, packed: bit i = address bit F[i].
 // Returns the length L of F's prefix 0, 1, .., L-1 (the contiguous run), or -1.
@@ -1008,7 +971,7 @@ int tile_geometry(int nbits, const int *tpos, int rows, Tc5Geom &g)
 }
 
 template <int K, int R2, bool LOWT, bool BF>
-int launch_tc5_kr(const Tc5Geom &g, int nbits, cudaStream_t st, int *grid_out)
+int launch_tc5_kr(const Tc5Geom &g, const BlockMat<K> &M, int nbits, cudaStream_t st, int *grid_out)
 {
     using L = Tc5Layout<K, R2>;
     auto kern = k_apply_tcgen05<K, R2, LOWT, BF>;
@@ -1029,12 +992,12 @@ int launch_tc5_kr(const Tc5Geom &g, int nbits, cudaStream_t st, int *grid_out)
     gg.n_tiles = 1ull << (nbits - K - 7 - (R2 == 2));
     const uint64_t grid = std::min<uint64_t>(gg.n_tiles, (uint64_t)cfg.sms);
     if (grid_out) *grid_out = (int)grid;
-    kern<<<(unsigned)grid, kThreadsTc5, L::SMEM, st>>>(gg);
+    kern<<<(unsigned)grid, kThreadsTc5, L::SMEM, st>>>(gg, M);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
 template <bool LOWT, bool BF>
-int launch_tc6a(const Tc5Geom &g, int nbits, cudaStream_t st, int *grid_out)
+int launch_tc6a(const Tc5Geom &g, const BlockMat<6> &M, int nbits, cudaStream_t st, int *grid_out)
 {
     auto kern = k_apply_tc6a<LOWT, BF>;
     static std::atomic<uint64_t> smem_done{0};
@@ -1052,20 +1015,19 @@ int launch_tc6a(const Tc5Geom &g, int nbits, cudaStream_t st, int *grid_out)
     gg.n_tiles = 1ull << (nbits - 6 - 7);
     const uint64_t grid = std::min<uint64_t>(gg.n_tiles, (uint64_t)cfg.sms);
     if (grid_out) *grid_out = (int)grid;
-    kern<<<(unsigned)grid, kThreadsTc5, kTc6Smem, st>>>(gg);
+    kern<<<(unsigned)grid, kThreadsTc5, kTc6Smem, st>>>(gg, M);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-// Geometry of the block and launch, B (hi, lo) already in device memory at d_b.
+// Geometry of the block and launch.
 template <int K, bool BF>
-int launch_tc5_staged(sim_t *h, float2 *psi, int nbits, const int *tpos, const uint32_t *d_b, cudaStream_t st,
-                      double *red = nullptr, int *grid_out = nullptr)
+int launch_tc5(sim_t *h, float2 *psi, int nbits, const int *tpos, const BlockMat<K> &M, cudaStream_t st, double *red,
+               int *grid_out)
 {
     Tc5Geom g{};
     g.psi = psi;
     g.red = red;
     for (int i = 0; i < K; i++) g.tpos[i] = tpos[i];  // ascending
-    g.bmat = d_b;
     g.err = h->d_errflag;
     g.nlow = 0;
     while (g.nlow < K && tpos[g.nlow] < 4) g.nlow++;
@@ -1073,11 +1035,11 @@ int launch_tc5_staged(sim_t *h, float2 *psi, int nbits, const int *tpos, const u
     if constexpr (K == 6) {  // 128-group tiles only: two 256-column accumulator sets fill the TMEM
         if (tile_geometry<K>(nbits, tpos, 7, g) < 0) return -1;
 #if SYCSIM_TC6_ATMEM
-        if (g.nlow > 0) return launch_tc6a<true, BF>(g, nbits, st, grid_out);
-        return launch_tc6a<false, BF>(g, nbits, st, grid_out);
+        if (g.nlow > 0) return launch_tc6a<true, BF>(g, M, nbits, st, grid_out);
+        return launch_tc6a<false, BF>(g, M, nbits, st, grid_out);
 #else
-        if (g.nlow > 0) return launch_tc5_kr<K, 1, true, BF>(g, nbits, st, grid_out);
-        return launch_tc5_kr<K, 1, false, BF>(g, nbits, st, grid_out);
+        if (g.nlow > 0) return launch_tc5_kr<K, 1, true, BF>(g, M, nbits, st, grid_out);
+        return launch_tc5_kr<K, 1, false, BF>(g, M, nbits, st, grid_out);
 #endif
     } else {
         // 128-group tiles when their runs reach 2 KiB (bit 7 is a target, or a target lies below
@@ -1087,26 +1049,13 @@ int launch_tc5_staged(sim_t *h, float2 *psi, int nbits, const int *tpos, const u
         const int run = tile_geometry<K>(nbits, tpos, 7, g);
         if (run < 0) return -1;
         if (g.nlow > 0) {
-            if constexpr (K == 5) return launch_tc5_kr<K, 1, true, BF>(g, nbits, st, grid_out);
+            if constexpr (K == 5) return launch_tc5_kr<K, 1, true, BF>(g, M, nbits, st, grid_out);
             return -2;
         }
-        if (run >= 8 || nbits < K + 8) return launch_tc5_kr<K, 1, false, BF>(g, nbits, st, grid_out);
+        if (run >= 8 || nbits < K + 8) return launch_tc5_kr<K, 1, false, BF>(g, M, nbits, st, grid_out);
         if (tile_geometry<K>(nbits, tpos, 8, g) < 8) return -1;
-        return launch_tc5_kr<K, 2, false, BF>(g, nbits, st, grid_out);
+        return launch_tc5_kr<K, 2, false, BF>(g, M, nbits, st, grid_out);
     }
-}
-
-template <int K, bool BF>
-int launch_tc5_k(sim_t *h, float2 *psi, int nbits, const int *tpos, const float2 *mat, cudaStream_t st,
-                 uint32_t *h_frag, uint32_t *d_frag, cudaEvent_t ev)
-{
-    using L = Tc5Layout<K, 1>;
-    build_b<K, BF>(mat, reinterpret_cast<uint16_t *>(h_frag));
-    if (cudaMemcpyAsync(d_frag, h_frag, 2 * L::B_BYTES, cudaMemcpyHostToDevice, st) != cudaSuccess) return -1;
-    const int rc = launch_tc5_staged<K, BF>(h, psi, nbits, tpos, d_frag, st);
-    // the staging slot is free again once this kernel, which reads it, has run (on any stream)
-    if (cudaEventRecord(ev, st) != cudaSuccess) return -1;
-    return rc;
 }
 
 }  // namespace
@@ -1127,55 +1076,19 @@ bool tcgen05_eligible(int nbits, int k, const int *tpos)
     return low <= (k >= 5 ? 1 : 0);
 }
 
-size_t tcgen05_staged_bytes(int k)
+int launch_apply_tcgen05(sim_t *h, float2 *psi, int nbits, int k, const int *tpos, const float2 *mat,
+                         const float2 *mat6_dev, bool bf16, cudaStream_t st, double *red, int *grid_out)
 {
+    auto go = [&](auto kc) {
+        constexpr int K = decltype(kc)::value;
+        const BlockMat<K> M = block_mat<K>(mat, mat6_dev);
+        return bf16 ? launch_tc5<K, true>(h, psi, nbits, tpos, M, st, red, grid_out)
+                    : launch_tc5<K, false>(h, psi, nbits, tpos, M, st, red, grid_out);
+    };
     switch (k) {
-    case 4: return 2 * Tc5Layout<4, 1>::B_BYTES;
-    case 5: return 2 * Tc5Layout<5, 1>::B_BYTES;
-    case 6: return 2 * Tc5Layout<6, 1>::B_BYTES;
-    default: return 0;
-    }
-}
-
-void tcgen05_build_staged(int k, const float2 *mat, bool bf16, void *h_out)
-{
-    uint16_t *o = static_cast<uint16_t *>(h_out);
-    if (k == 4) bf16 ? build_b<4, true>(mat, o) : build_b<4, false>(mat, o);
-    if (k == 5) bf16 ? build_b<5, true>(mat, o) : build_b<5, false>(mat, o);
-    if (k == 6) bf16 ? build_b<6, true>(mat, o) : build_b<6, false>(mat, o);
-}
-
-int tcgen05_launch_staged(sim_t *h, float2 *psi, int nbits, int k, const int *tpos, bool bf16,
-                          const void *d_staged, cudaStream_t st, double *red, int *grid_out)
-{
-    const uint32_t *d_b = static_cast<const uint32_t *>(d_staged);
-    switch (k) {
-    case 4: return bf16 ? launch_tc5_staged<4, true>(h, psi, nbits, tpos, d_b, st, red, grid_out)
-                        : launch_tc5_staged<4, false>(h, psi, nbits, tpos, d_b, st, red, grid_out);
-    case 5: return bf16 ? launch_tc5_staged<5, true>(h, psi, nbits, tpos, d_b, st, red, grid_out)
-                        : launch_tc5_staged<5, false>(h, psi, nbits, tpos, d_b, st, red, grid_out);
-    case 6: return bf16 ? launch_tc5_staged<6, true>(h, psi, nbits, tpos, d_b, st, red, grid_out)
-                        : launch_tc5_staged<6, false>(h, psi, nbits, tpos, d_b, st, red, grid_out);
-    default: return -1;
-    }
-}
-
-int launch_apply_tcgen05(sim_t *h, float2 *psi, int nbits, int k, const int *tpos, const float2 *mat, bool bf16,
-                         cudaStream_t st)
-{
-    const int slot = h->frag_next;
-    h->frag_next = (slot + 1) % sim_s::kFragSlots;
-    if (cudaEventSynchronize(h->frag_ev[slot]) != cudaSuccess) return -1;
-    uint32_t *hf = h->h_frag + sim_s::kFragWords * slot;
-    uint32_t *df = h->d_frag + sim_s::kFragWords * slot;
-    cudaEvent_t ev = h->frag_ev[slot];
-    switch (k) {
-    case 4: return bf16 ? launch_tc5_k<4, true>(h, psi, nbits, tpos, mat, st, hf, df, ev)
-                        : launch_tc5_k<4, false>(h, psi, nbits, tpos, mat, st, hf, df, ev);
-    case 5: return bf16 ? launch_tc5_k<5, true>(h, psi, nbits, tpos, mat, st, hf, df, ev)
-                        : launch_tc5_k<5, false>(h, psi, nbits, tpos, mat, st, hf, df, ev);
-    case 6: return bf16 ? launch_tc5_k<6, true>(h, psi, nbits, tpos, mat, st, hf, df, ev)
-                        : launch_tc5_k<6, false>(h, psi, nbits, tpos, mat, st, hf, df, ev);
+    case 4: return go(std::integral_constant<int, 4>{});
+    case 5: return go(std::integral_constant<int, 5>{});
+    case 6: return go(std::integral_constant<int, 6>{});
     default: return -1;
     }
 }

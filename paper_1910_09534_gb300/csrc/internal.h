@@ -63,14 +63,6 @@ struct sim_s {
     uint8_t *d_contract = nullptr;
     size_t contract_bytes = 0;
 
-    // tensor-core B fragments (fragment-major R^T, hi/lo) go through a device ring
-    static constexpr int kFragSlots = 8;
-    static constexpr int kFragWords = 2 * 16 * 16 * 64;  // k = 6, split: 128 KiB
-    uint32_t *d_frag = nullptr;
-    uint32_t *h_frag = nullptr;  // pinned staging
-    cudaEvent_t frag_ev[kFragSlots] = {};
-    int frag_next = 0;
-
     // fused reduction: sim_apply_plan's last block (tcgen05) leaves each CTA's (sum p, sum p^2) in
     // d_partials; sim_reduce then only combines them, while no call has written the state since
     // (write_epoch counts the calls that may write it) and the state's memory is the handle's own
@@ -79,7 +71,7 @@ struct sim_s {
     int red_blocks = 0;
     mutable bool state_exposed = false;
 
-    // a whole plan's staged block operands (sim_apply_plan), uploaded in one copy: two slots, each
+    // a whole plan's staged 6-qubit matrices (sim_apply_plan), uploaded in one copy: two slots, each
     // a pinned source and its device copy, reused once the plan that last used it has run
     char *h_plan[2] = {};
     char *d_plan[2] = {};
@@ -239,11 +231,12 @@ struct LaunchCfg {
 enum class BlockPath { CudaCore, MmaSync, Tcgen05 };
 BlockPath block_path(int nbits, int k, const int *tpos, int precision);
 // true if enqueue_block_on would not have to wait for a matrix-staging slot (non-blocking check)
-bool staging_slot_free(sim_t *h, int nbits, int k, const int *tpos, int precision);
-size_t block_staged_bytes(int nbits, int k, const int *tpos, int precision);
-void block_build_staged(int nbits, int k, const int *tpos, const float2 *mat, int precision, void *h_out);
-// red / red_grid: as for tcgen05_launch_staged, taken only by tcgen05 blocks (*red_grid stays 0
-// for the others)
+bool staging_slot_free(sim_t *h, int k);
+// bytes of a block's matrix that must be in device memory (d_staged) for launch_block_staged: its
+// FP32 matrix, float2 row-major in sorted-target order, for k = 6; 0 for narrower blocks
+size_t block_staged_bytes(int k);
+// red (may be NULL): a tcgen05 block also writes each CTA's (sum p, sum p^2) of its results at
+// red[2 cta]; *red_grid (may be NULL) receives the number of CTAs (0 for the other kernels)
 int launch_block_staged(sim_t *h, float2 *psi, int nbits, int k, const int *tpos, const float2 *mat,
                         int precision, const void *d_staged, cudaStream_t st, double *red = nullptr,
                         int *red_grid = nullptr);
@@ -274,24 +267,14 @@ inline bool f16x3_mode(int precision)
 
 // ---- apply_tcgen05.cu (5th-generation tensor cores, TMEM) ----
 bool tcgen05_eligible(int nbits, int k, const int *tpos);
-// operands staged once in device memory (CUDA graphs): B hi/lo of one block
-size_t tcgen05_staged_bytes(int k);
-void tcgen05_build_staged(int k, const float2 *mat, bool bf16, void *h_out);
-// red (may be NULL): the kernel also writes each CTA's (sum p, sum p^2) of its results at
-// red[2 cta]; *grid_out (may be NULL) receives the number of CTAs
-int tcgen05_launch_staged(sim_t *h, float2 *psi, int nbits, int k, const int *tpos, bool bf16,
-                          const void *d_staged, cudaStream_t st, double *red = nullptr, int *grid_out = nullptr);
-int launch_apply_tcgen05(sim_t *h, float2 *psi, int nbits, int k, const int *tpos, const float2 *mat, bool bf16,
-                         cudaStream_t st);
+int launch_apply_tcgen05(sim_t *h, float2 *psi, int nbits, int k, const int *tpos, const float2 *mat,
+                         const float2 *mat6_dev, bool bf16, cudaStream_t st, double *red = nullptr,
+                         int *grid_out = nullptr);
 
 // ---- apply_tc.cu (tensor cores) ----
 bool tc_eligible(int nbits, int k, const int *tpos);
 bool tc_eligible_low4(int nbits, int k);
-size_t tc_staged_bytes(int k, int precision);
-void tc_build_staged(int k, const float2 *mat, int precision, void *h_out);
-int tc_launch_staged(float2 *psi, int nbits, int k, const int *tpos, int precision, const void *d_staged,
-                     cudaStream_t st);
-int launch_apply_tc(sim_t *h, float2 *psi, int nbits, int k, const int *tpos, const float2 *mat,
+int launch_apply_tc(float2 *psi, int nbits, int k, const int *tpos, const float2 *mat, const float2 *mat6_dev,
                     int precision, cudaStream_t st);
 
 // ---- kernel launchers (apply.cu) ----

@@ -899,10 +899,10 @@ int sim_apply_plan(sim_t *h, const sim_plan_t *p)
     if (h->store != SIM_STORE_DEVICE)
         return fail(h, SIM_E_UNSUPPORTED, "sim_apply_plan: host-store state: use sim_run_phase");
     SIM_DEVICE_SCOPE(h, h->device);
-    // Every block's operands (tensor-core R^T fragments, 6-qubit matrices) are built on the host and
-    // uploaded in one copy before the first launch, then every block is launched from them: the
-    // calling thread never waits for the device inside the plan (a per-block staging ring would make
-    // it wait for the block launched a ring's length earlier), and a plan costs one small copy.
+    // The 6-qubit blocks' matrices are uploaded in one copy before the first launch (narrower blocks
+    // carry theirs in the launch), then every block is launched: the calling thread never waits for
+    // the device inside the plan (a per-block staging ring would make it wait for the block launched
+    // a ring's length earlier), and a plan costs at most one small copy.
     struct Prep {
         int k;
         int tpos[kMaxK];
@@ -924,7 +924,7 @@ int sim_apply_plan(sim_t *h, const sim_plan_t *p)
         const int rc = prepare_block(h, pb.k, b.qubits.data(), b.mat.data(), pb.tpos, mats.data() + mtot);
         if (rc != SIM_OK) return rc;
         mtot += (size_t)1 << (2 * pb.k);
-        pb.bytes = block_staged_bytes(h->n, pb.k, pb.tpos, p->precision);
+        pb.bytes = block_staged_bytes(pb.k);
         pb.off = total;
         total += (pb.bytes + 255) & ~size_t(255);
     }
@@ -954,9 +954,7 @@ int sim_apply_plan(sim_t *h, const sim_plan_t *p)
             h->plan_bytes[slot] = want;
         }
         for (size_t i = 0; i < nb; i++)
-            if (prep[i].bytes)
-                block_build_staged(h->n, prep[i].k, prep[i].tpos, mats.data() + prep[i].moff, p->precision,
-                                   h->h_plan[slot] + prep[i].off);
+            if (prep[i].bytes) std::memcpy(h->h_plan[slot] + prep[i].off, mats.data() + prep[i].moff, prep[i].bytes);
         SIM_CUDA_TRY(h, cudaMemcpyAsync(h->d_plan[slot], h->h_plan[slot], total, cudaMemcpyHostToDevice, h->stream));
         d_ops = h->d_plan[slot];
     }
@@ -1013,7 +1011,7 @@ int sim_graph_create(sim_t *h, const sim_plan_t *p, sim_graph_t **out)
         const int rc = prepare_block(h, sb.k, b.qubits.data(), b.mat.data(), sb.tpos, mat);
         if (rc != SIM_OK) return rc;
         sb.mat.assign(mat, mat + (1 << (2 * sb.k)));
-        sb.bytes = block_staged_bytes(h->n, sb.k, sb.tpos, p->precision);
+        sb.bytes = block_staged_bytes(sb.k);
         sb.off = total;
         total += (sb.bytes + 255) & ~size_t(255);
     }
@@ -1031,7 +1029,7 @@ int sim_graph_create(sim_t *h, const sim_plan_t *p, sim_graph_t **out)
     if (total) {
         std::vector<char> host(total);
         for (auto &sb : blocks)
-            if (sb.bytes) block_build_staged(h->n, sb.k, sb.tpos, sb.mat.data(), p->precision, host.data() + sb.off);
+            if (sb.bytes) std::memcpy(host.data() + sb.off, sb.mat.data(), sb.bytes);
         if (cudaMalloc(&g->d_staged, total) != cudaSuccess) return cleanup(SIM_E_NOMEM_DEV, "staging buffer");
         if (cudaMemcpy(g->d_staged, host.data(), total, cudaMemcpyHostToDevice) != cudaSuccess)
             return cleanup(SIM_E_CUDA, "staging upload");

@@ -492,7 +492,7 @@ int advance_unpacked(srv_t *s, const std::shared_ptr<Req> &r, bool *progressed)
         const int t = r->next_block < (size_t)r->nt[0] ? 0 : (r->next_block < tensor_blocks ? 1 : -1);
         float2 *buf = t < 0 || !r->split ? r->d_state : r->d_t[t];
         const int nbits = t < 0 || !r->split ? r->n : r->nw[t];
-        if (!staging_slot_free(h, nbits, b.k, b.tpos, r->precision)) return SIM_OK;
+        if (!staging_slot_free(h, b.k)) return SIM_OK;
         const int rc = enqueue_block_on(h, buf, nbits, b.k, b.tpos, b.mat.data(), r->precision, st);
         if (rc != SIM_OK) return rc;
         r->next_block++;

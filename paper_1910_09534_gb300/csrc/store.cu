@@ -638,12 +638,12 @@ int run_phase(sim_t *h, int set, const sim_plan_t *p, const std::function<int(fl
         int rc = prepare_block_map(h, pb.k, b.qubits.data(), b.mat.data(), h->slice_phys[set], nl,
                                    pb.tpos, pb.mat.data());
         if (rc != SIM_OK) return rc;
-        pb.bytes = block_staged_bytes(nl, pb.k, pb.tpos, p->precision);
+        pb.bytes = block_staged_bytes(pb.k);
         pb.off = staged_total;
         staged_total += (pb.bytes + 255) & ~size_t(255);
     }
-    // Every slice gets the same blocks: their tensor-core operands (and 6-qubit matrices) are
-    // uploaded once for the phase, not once per block and slice -- such small copies would queue
+    // Every slice gets the same blocks: their 6-qubit matrices (narrower ones travel with the launch)
+    // are uploaded once for the phase, not once per block and slice -- such small copies would queue
     // behind the slice transfers on the copy engines and hold back every kernel.
     char *d_staged = nullptr;
     auto release = [&](int rc) {  // the staged operands go once the phase's last kernel is queued
@@ -664,7 +664,7 @@ int run_phase(sim_t *h, int set, const sim_plan_t *p, const std::function<int(fl
             h->h_ops_bytes = 2 * staged_total;
         }
         for (const Prepared &pb : blocks)
-            if (pb.bytes) block_build_staged(nl, pb.k, pb.tpos, pb.mat.data(), p->precision, h->h_ops + pb.off);
+            if (pb.bytes) std::memcpy(h->h_ops + pb.off, pb.mat.data(), pb.bytes);
         if (cudaMallocAsync(reinterpret_cast<void **>(&d_staged), staged_total, h->stream) != cudaSuccess) {
             d_staged = nullptr;
             return fail(h, SIM_E_NOMEM_DEV, "sim_run_phase: staged operands");
