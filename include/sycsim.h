@@ -308,9 +308,9 @@ int sim_apply_plan(sim_t *h, const sim_plan_t *p);
 /* ---- CUDA graphs (not in the paper) ----------------------------------------
  * Capture the block launches of a plan on h once and replay them.  For a plan run many times
  * (the same circuit from several initial states, repeated runs) a replay skips the per-block host
- * work -- matrix rounding, operand staging, the launch itself -- which dominates below ~2^24
- * amplitudes.  Every block's staged operands (tensor-core B fragments, 6-qubit matrices) are
- * uploaded once into device memory that the graph owns.  A graph is bound to h (its state
+ * work -- matrix rounding, operand staging, the launch itself -- which dominates below ~2^20
+ * amplitudes.  The 6-qubit blocks' matrices are uploaded once into device memory that the graph
+ * owns (narrower blocks carry theirs in the captured launches).  A graph is bound to h (its state
  * buffer, stream and layout): sim_graph_launch refuses with SIM_E_INVAL on another handle or
  * once h's layout has changed (sim_permute), and a graph must be destroyed before its handle.
  * SIM_E_UNSUPPORTED for host-store handles or a handle on the legacy default stream.

@@ -28,15 +28,22 @@
 #include <cstring>
 #include <type_traits>
 
-#include "block_mat.cuh"
 #include "internal.h"
+#include "pdl.cuh"
 
 namespace sycsim {
 namespace {
 
+// The CUDA-core kernels' matrix: a parameter that the FMAs read as constants (BlockMat's 16-byte
+// alignment, for wide loads, moved it in the constant bank and cost k = 4, 5 passes 1-1.5 %).
 template <int K>
-using MatP = BlockMat<K>;
-using MatPtr = BlockMat<6>;
+struct MatP {
+    float2 m[(1 << K) * (1 << K)];
+};
+
+struct MatPtr {
+    const float2 *p;
+};
 
 struct DirectGeom {
     float2 *psi;
@@ -152,9 +159,11 @@ __global__ void __launch_bounds__(256, direct_min_blocks(K)) k_apply_direct(Dire
     constexpr int D = 1 << K;
     constexpr bool kSmemMat = std::is_same<MatSrc, MatPtr>::value;
     extern __shared__ float2 smem[];
+    pdl_launch_next();
     if constexpr (kSmemMat) stage_matrix<K>(smem, M.p);
     const uint64_t gi = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (gi >= g.n_groups) return;
+    pdl_wait();
     float2 *p = g.psi + insert_zero_bits(gi, g.tpos, K);
     float2 x[D];
 #pragma unroll
@@ -175,6 +184,7 @@ __global__ void __launch_bounds__(tiled_threads(K), tiled_min_blocks(K)) k_apply
     extern __shared__ float2 smem[];
     float2 *tile = smem;
     float2 *msm = smem + ((size_t)D << g.F);
+    pdl_launch_next();
     if constexpr (kSmemMat) stage_matrix<K>(msm, M.p);
 
     const uint32_t tid = threadIdx.x;
@@ -182,6 +192,7 @@ __global__ void __launch_bounds__(tiled_threads(K), tiled_min_blocks(K)) k_apply
     const uint32_t lowmask = (1u << g.nlow) - 1;
     const uint64_t base = insert_zero_bits((uint64_t)blockIdx.x << g.m, g.hpos, g.nhigh);
     float2 *gp = g.psi + base;
+    pdl_wait();
 
     // load: linear tile position p = tid + c 2^F; row r = c >> nlow, column ((c & lowmask) << F) | tid
 #pragma unroll
@@ -249,8 +260,7 @@ int launch_k(float2 *psi, int nbits, const int *tpos, const MatSrc &M, cudaStrea
         const uint64_t blocks = (g.n_groups + 255) / 256;
         auto kern = k_apply_direct<K, MatSrc>;
         if (ensure_smem(kern, mat_bytes) != cudaSuccess) return -1;
-        kern<<<(unsigned)blocks, 256, mat_bytes, st>>>(g, M);
-        return cudaGetLastError() == cudaSuccess ? 0 : -1;
+        return launch_pdl(kern, (unsigned)blocks, 256, mat_bytes, st, g, M) == cudaSuccess ? 0 : -1;
     }
 
     TiledGeom g{};
@@ -308,8 +318,7 @@ int launch_k(float2 *psi, int nbits, const int *tpos, const MatSrc &M, cudaStrea
     const size_t smem = (sizeof(float2) << (g.F + K)) + mat_bytes;
     auto kern = k_apply_tiled<K, MatSrc>;
     if (ensure_smem(kern, smem) != cudaSuccess) return -1;
-    kern<<<(unsigned)tiles, 1u << g.F, smem, st>>>(g, M);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    return launch_pdl(kern, (unsigned)tiles, 1u << g.F, smem, st, g, M) == cudaSuccess ? 0 : -1;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -384,6 +393,8 @@ __global__ void __launch_bounds__(256, reg_min_blocks(K, kLow)) k_apply_reg(RegG
 {
     constexpr int D = 1 << K;
     constexpr bool kPrefetch = reg_prefetch(K);
+    pdl_launch_next();
+    pdl_wait();
     const int lane = threadIdx.x & 31;
     const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     uint64_t w = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -449,8 +460,7 @@ int launch_reg_kernel(const RegGeom &g, const MatP<K> &M, cudaStream_t st)
     if (!cfg.ok) return -1;
     const uint64_t need = (g.n_wtiles + 7) / 8;  // 8 warps per CTA
     const uint64_t grid = std::min<uint64_t>(need, (uint64_t)cfg.sms * cfg.occ);
-    kern<<<(unsigned)grid, 256, 0, st>>>(g, M);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    return launch_pdl(kern, (unsigned)grid, 256, 0, st, g, M) == cudaSuccess ? 0 : -1;
 }
 
 template <int K>

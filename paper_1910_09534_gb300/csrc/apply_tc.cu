@@ -36,6 +36,7 @@
 
 #include "block_mat.cuh"
 #include "internal.h"
+#include "pdl.cuh"
 
 namespace sycsim {
 namespace {
@@ -129,11 +130,13 @@ __global__ void __launch_bounds__(256, mma_min_blocks(K)) k_apply_mma(const __gr
     constexpr int FRAG_WORDS = KS * NT * 64;
     extern __shared__ uint32_t sb[];
     build_frag_tf32<K, kSplit>(block_mat_ptr(M), sb);
+    pdl_wait();
 
     const int lane = threadIdx.x & 31, gid = lane >> 2, t = lane & 3;
     const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     for (uint64_t mt = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; mt < g.n_mtiles;
          mt += nw) {
+        if (mt + nw >= g.n_mtiles) pdl_launch_next();  // this warp's last tile
         const uint64_t grp = mt * 16 + gid;
         float2 *p0 = g.psi + insert_zero_bits_t(grp, g.tpos, K);
         float2 *p1 = g.psi + insert_zero_bits_t(grp + 8, g.tpos, K);
@@ -244,11 +247,13 @@ __global__ void __launch_bounds__(256, mma_min_blocks(K)) k_apply_mma_f16x3(cons
     constexpr int FRAG_WORDS = KS * NT * 64;
     extern __shared__ uint32_t sb[];
     build_frag_f16<K>(block_mat_ptr(M), sb);
+    pdl_wait();
 
     const int lane = threadIdx.x & 31, gid = lane >> 2, t = lane & 3;
     const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     for (uint64_t mt = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; mt < g.n_mtiles;
          mt += nw) {
+        if (mt + nw >= g.n_mtiles) pdl_launch_next();  // this warp's last tile
         const uint64_t grp = mt * 16 + gid;
         float2 *p0 = g.psi + insert_zero_bits_t(grp, g.tpos, K);
         float2 *p1 = g.psi + insert_zero_bits_t(grp + 8, g.tpos, K);
@@ -345,8 +350,7 @@ int launch_mma(float2 *psi, int nbits, const int *tpos, const BlockMat<K> &M, cu
     if (!cfg.ok) return -1;
     const uint64_t need = (g.n_mtiles + 7) / 8;
     const uint64_t grid = std::min<uint64_t>(need, (uint64_t)cfg.sms * cfg.occ);
-    kern<<<(unsigned)grid, 256, kBytes, st>>>(g, M);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    return launch_pdl(kern, (unsigned)grid, 256, kBytes, st, g, M) == cudaSuccess ? 0 : -1;
 }
 
 }  // namespace

@@ -55,6 +55,7 @@
 
 #include "block_mat.cuh"
 #include "internal.h"
+#include "pdl.cuh"
 
 namespace sycsim {
 namespace {
@@ -388,6 +389,7 @@ __global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tcgen05(const __grid_c
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem = tmem_base;
+    pdl_wait();  // all above is this CTA's own; the state from here on
     volatile int *ab = &abort_flag;
     auto give_up = [&]() {
         *ab = 1;
@@ -481,6 +483,7 @@ __global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tcgen05(const __grid_c
                 if (lane == 0) give_up();
                 break;
             }
+            if (tile + gridDim.x >= g.n_tiles) pdl_launch_next();  // this CTA's last tile
             const uint64_t base = insert_zero_bits_g(tile * (kRows * R2), g.tpos, K);
             const uint32_t bar = smem_u32(&loaded[st]);
             if (lane == 0) {
@@ -745,6 +748,7 @@ __global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tc6a(const __grid_cons
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem = tmem_base;
+    pdl_wait();  // all above is this CTA's own; the state from here on
     volatile int *ab = &abort_flag;
     auto give_up = [&]() {
         *ab = 1;
@@ -832,6 +836,7 @@ __global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tc6a(const __grid_cons
                 if (lane == 0) give_up();
                 break;
             }
+            if (tile + gridDim.x >= g.n_tiles) pdl_launch_next();  // this CTA's last tile
             const uint64_t base = insert_zero_bits_g(tile * kRows, g.tpos, 6);
             const uint32_t bar = smem_u32(&loaded[st]);
             if (lane == 0) mbar_expect_tx(bar, kTc6Stage);  // before any of the copies can complete
@@ -992,8 +997,7 @@ int launch_tc5_kr(const Tc5Geom &g, const BlockMat<K> &M, int nbits, cudaStream_
     gg.n_tiles = 1ull << (nbits - K - 7 - (R2 == 2));
     const uint64_t grid = std::min<uint64_t>(gg.n_tiles, (uint64_t)cfg.sms);
     if (grid_out) *grid_out = (int)grid;
-    kern<<<(unsigned)grid, kThreadsTc5, L::SMEM, st>>>(gg, M);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    return launch_pdl(kern, (unsigned)grid, kThreadsTc5, L::SMEM, st, gg, M) == cudaSuccess ? 0 : -1;
 }
 
 template <bool LOWT, bool BF>
@@ -1015,8 +1019,7 @@ int launch_tc6a(const Tc5Geom &g, const BlockMat<6> &M, int nbits, cudaStream_t 
     gg.n_tiles = 1ull << (nbits - 6 - 7);
     const uint64_t grid = std::min<uint64_t>(gg.n_tiles, (uint64_t)cfg.sms);
     if (grid_out) *grid_out = (int)grid;
-    kern<<<(unsigned)grid, kThreadsTc5, kTc6Smem, st>>>(gg, M);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    return launch_pdl(kern, (unsigned)grid, kThreadsTc5, kTc6Smem, st, gg, M) == cudaSuccess ? 0 : -1;
 }
 
 // Geometry of the block and launch.

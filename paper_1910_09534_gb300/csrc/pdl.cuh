@@ -1,0 +1,42 @@
+// pdl.cuh -- programmatic dependent launch between the kernels of a handle's stream.
+//
+// A plan is a chain of passes over the same buffer.  Launched the ordinary way, a pass starts once
+// the one before has drained and the launch has reached the SMs: 2-3 us a pass on GB300, as long as
+// the pass itself below 2^20 amplitudes.  Kernels launched through launch_pdl may become resident
+// while the one before still runs; they do what does not depend on it (the block's matrix into
+// shared memory, barriers, tensor memory) and call pdl_wait before their first access to anything
+// that earlier work of the stream writes or reads.  pdl_wait returns when every earlier kernel has
+// completed and its writes are visible, so an early start changes no result.  A copy, a memset or
+// an event between two kernels orders them fully, as ever.
+#pragma once
+
+#include <cuda_runtime.h>
+
+#include <utility>
+
+namespace sycsim {
+
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
+// The next kernel of the stream may start, once every CTA of this one has got here or left.  The
+// persistent tensor-core kernels call it at a CTA's last tile (2 % faster on a 20-qubit plan than
+// at the start, where the next kernel's CTAs crowd the SMs that are still idle).
+__device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
+template <typename... P, typename... A>
+cudaError_t launch_pdl(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A &&...args)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+}
+
+}  // namespace sycsim

@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "pdl.cuh"
 
 // Measured on 2^30 amplitudes: 16-byte accesses 13-17 % faster than 8-byte on every pattern;
 // minimum tiles of 2^11-2^12 amplitudes help tiles that permute in place a little and tile pairs
@@ -68,6 +69,8 @@ __device__ __forceinline__ uint64_t insert_zero_bits_p(uint64_t x, const int *po
 __global__ void __launch_bounds__(256) k_permute_pass(PermGeom g)
 {
     extern __shared__ float2 sm[];
+    pdl_launch_next();
+    pdl_wait();
     const uint64_t baseA = insert_zero_bits_p((uint64_t)blockIdx.x << g.LB, g.rowpos, g.q);
     uint64_t baseB = baseA;
     for (int i = 0; i < g.nhh; ++i) {
@@ -155,6 +158,7 @@ __global__ void __launch_bounds__(256) k_permute_tile_bulk(PermGeom g, int *err)
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t p_it[64], sig_it[64];  // the iteration part of p, and its image under sig
     __shared__ int ok;
+    pdl_launch_next();
     const int nloc = g.LB + g.q, T = 1 << nloc;
     const uint32_t row_bytes = 8u << g.LB;
     const uint64_t base = insert_zero_bits_p((uint64_t)blockIdx.x << g.LB, g.rowpos, g.q);
@@ -178,6 +182,7 @@ __global__ void __launch_bounds__(256) k_permute_tile_bulk(PermGeom g, int *err)
     if (threadIdx.x == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(sbar) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        pdl_wait();  // this thread issues every access to the state
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(sbar),
                      "r"((uint32_t)(ntile * T) * 8u)
                      : "memory");
@@ -390,8 +395,7 @@ int launch_involution(float2 *psi, int nbits, const int *inv, cudaStream_t st, i
                 cudaSuccess)
             return -1;
         choose_lane_bits(g);
-        k_permute_tile_bulk<<<(unsigned)tiles, 256, tsm, st>>>(g, err);
-        return cudaGetLastError() == cudaSuccess ? 0 : -1;
+        return launch_pdl(k_permute_tile_bulk, (unsigned)tiles, 256, tsm, st, g, err) == cudaSuccess ? 0 : -1;
     }
     const size_t smem = (g.nhh ? 2 : 1) * sizeof(float2) << (LB + q);  // a tile pair, or one tile
     if (smem > 48 * 1024 &&
@@ -399,8 +403,7 @@ int launch_involution(float2 *psi, int nbits, const int *inv, cudaStream_t st, i
                              (int)smem) != cudaSuccess)
         return -1;
     const int threads = std::min(256, 1 << (LB + q));
-    k_permute_pass<<<(unsigned)tiles, threads, smem, st>>>(g);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    return launch_pdl(k_permute_pass, (unsigned)tiles, threads, smem, st, g) == cudaSuccess ? 0 : -1;
 }
 
 }  // namespace
