@@ -249,14 +249,12 @@ bool precision_ok(int precision);
 // reduction no longer describe it
 inline void state_written(sim_t *h) { h->write_epoch++; }
 // the final combine of the reduction over nblocks (sum p, sum p^2) pairs (reduce.cu)
-int launch_reduce_final(const double *partials, int nblocks, double *d_result, cudaStream_t st);
+int launch_reduce_final(const double *partials, int nblocks, uint64_t amps, double *d_result, cudaStream_t st);
 // Entries first .. first + count - 1 (logical indices through bit_of, or physical ones when bit_of
 // is NULL) whose physical index p lies in [lo, hi): buf[j] = base[p - lo] (scatter: the reverse);
 // the others untouched.  The device part of a hybrid host store's readout and load.
 int launch_gather_region(float2 *base, uint64_t lo, uint64_t hi, float2 *buf, uint64_t first, uint64_t count, int n,
                          const int *bit_of, int scatter, cudaStream_t st);
-// d_result[4..6] = {d_result[0], scale * d_result[1], scale * d_result[1] - 1} (one thread)
-int launch_result3(double *d_result, double scale, cudaStream_t st);
 // the modes whose 4- to 6-qubit blocks take the tcgen05 kernel where it is eligible
 inline bool tmem_mode(int precision) { return precision == SIM_FP16X3_TMEM || precision == SIM_BF16X3; }
 // the modes whose mma.sync blocks use the 3xFP16 kernel (BF16X3 hands it what tcgen05 leaves)
@@ -290,11 +288,12 @@ int launch_apply_fp32(sim_t *h, float2 *psi, int nbits, int k, const int *tpos,
 int launch_permute(sim_t *h, float2 *psi, int nbits, const int *perm, cudaStream_t st);
 
 // ---- reduce.cu ----
-int launch_reduce(sim_t *h, const float2 *psi, uint64_t amps, double *d_partials,
-                  double *d_result, cudaStream_t st);
+// d_result[0..1] = (sum p, sum p^2), d_result[4..6] = {sum p, amps sum p^2, that minus 1}
+int launch_reduce(const float2 *psi, uint64_t amps, double *d_partials, double *d_result, cudaStream_t st);
 int launch_gather_logical(const float2 *psi, float2 *dst, uint64_t first, uint64_t count,
                           int n, const int *bit_of, int scatter, cudaStream_t st);
-int launch_set_basis(float2 *psi, uint64_t amps, uint64_t phys, cudaStream_t st);
+// the basis state |phys>, every amplitude written
+int launch_reset(float2 *psi, uint64_t amps, uint64_t phys, cudaStream_t st);
 
 // ---- store.cu (host store) ----
 int host_store_create(sim_t *h, const sim_opts &o);

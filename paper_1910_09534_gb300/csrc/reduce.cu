@@ -10,6 +10,7 @@
 #include <mutex>
 
 #include "internal.h"
+#include "pdl.cuh"
 
 namespace sycsim {
 namespace {
@@ -27,6 +28,8 @@ __device__ __forceinline__ double warp_sum(double v)
 __global__ void __launch_bounds__(kReduceThreads) k_reduce_partials(const float4 *psi4, uint64_t n4,
                                                                     double *partials)
 {
+    pdl_launch_next();
+    pdl_wait();
     double s1 = 0.0, s2 = 0.0;
     const uint64_t stride = (uint64_t)gridDim.x * kReduceThreads * kReduceUnroll;
     for (uint64_t b = (uint64_t)blockIdx.x * kReduceThreads * kReduceUnroll + threadIdx.x; b < n4;
@@ -67,8 +70,13 @@ __global__ void __launch_bounds__(kReduceThreads) k_reduce_partials(const float4
     }
 }
 
-__global__ void k_reduce_final(const double *partials, int nblocks, double *out)
+// The CTAs' pairs, combined by one warp in a fixed order.  sums (may be NULL): (sum p, sum p^2);
+// three (may be NULL): sum p, scale * sum p^2, and that minus 1 -- the values a caller reads, written
+// here rather than by a launch of their own.
+__global__ void k_reduce_final(const double *partials, int nblocks, double *sums, double *three, double scale)
 {
+    pdl_launch_next();
+    pdl_wait();
     double s1 = 0.0, s2 = 0.0;
     for (int i = threadIdx.x; i < nblocks; i += 32) {
         s1 += partials[2 * i];
@@ -77,18 +85,24 @@ __global__ void k_reduce_final(const double *partials, int nblocks, double *out)
     s1 = warp_sum(s1);
     s2 = warp_sum(s2);
     if (threadIdx.x == 0) {
-        out[0] = s1;
-        out[1] = s2;
+        if (sums) {
+            sums[0] = s1;
+            sums[1] = s2;
+        }
+        if (three) {
+            three[0] = s1;
+            three[1] = s2 * scale;
+            three[2] = s2 * scale - 1.0;
+        }
     }
 }
 
-// r[4..6] = {sum p, scale * sum p^2, scale * sum p^2 - 1} from r[0..1] = (sum p, sum p^2)
-__global__ void k_result3(double *r, double scale)
+// CTAs of a reduction over n4 pairs of amplitudes: as many as have work, at most kReduceBlocks (a CTA
+// without work would add zeros).
+unsigned reduce_grid(uint64_t n4)
 {
-    const double s2 = r[1] * scale;
-    r[4] = r[0];
-    r[5] = s2;
-    r[6] = s2 - 1.0;
+    const uint64_t need = (n4 + kReduceThreads * kReduceUnroll - 1) / (kReduceThreads * kReduceUnroll);
+    return (unsigned)(need < (uint64_t)kReduceBlocks ? need : (uint64_t)kReduceBlocks);
 }
 
 struct BitMap {
@@ -129,22 +143,16 @@ __global__ void k_gather_region(float2 *base, uint64_t lo, uint64_t hi, float2 *
     }
 }
 
-__global__ void k_set_basis(float2 *psi, uint64_t phys) { psi[phys] = make_float2(1.f, 0.f); }
-
-// Final step of the allocation-free reduction: sum p, scale * sum p^2, and that minus 1.
-__global__ void k_reduce_final3(const double *partials, int nblocks, double scale, double *out)
+// |phys> into a state of 2 n4 amplitudes: zeros and the one, in one launch and one write of the state.
+__global__ void __launch_bounds__(256) k_reset(float4 *psi4, uint64_t n4, uint64_t phys)
 {
-    double s1 = 0.0, s2 = 0.0;
-    for (int i = threadIdx.x; i < nblocks; i += 32) {
-        s1 += partials[2 * i];
-        s2 += partials[2 * i + 1];
-    }
-    s1 = warp_sum(s1);
-    s2 = warp_sum(s2);
-    if (threadIdx.x == 0) {
-        out[0] = s1;
-        out[1] = s2 * scale;
-        out[2] = s2 * scale - 1.0;
+    pdl_launch_next();
+    pdl_wait();
+    const uint64_t one = phys >> 1;
+    for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (uint64_t)gridDim.x * blockDim.x) {
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (i == one) (phys & 1 ? v.z : v.x) = 1.f;
+        psi4[i] = v;
     }
 }
 
@@ -165,25 +173,30 @@ static __device__ __align__(256) double g_noalloc_partials[sycsim::kNoAllocParti
 
 namespace sycsim {
 
-int launch_reduce(sim_t *, const float2 *psi, uint64_t amps, double *d_partials, double *d_result,
-                  cudaStream_t st)
+static int enqueue_reduction(const float2 *psi, uint64_t amps, double *partials, double *sums, double *three,
+                             cudaStream_t st)
 {
-    const uint64_t n4 = amps / 2;  // amps >= 2 (n >= 1)
-    k_reduce_partials<<<kReduceBlocks, kReduceThreads, 0, st>>>((const float4 *)psi, n4, d_partials);
-    k_reduce_final<<<1, 32, 0, st>>>(d_partials, kReduceBlocks, d_result);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    const uint64_t n4 = amps / 2;  // amps >= 2
+    const unsigned grid = reduce_grid(n4);
+    if (launch_pdl(k_reduce_partials, grid, kReduceThreads, 0, st, (const float4 *)psi, n4, partials) != cudaSuccess)
+        return -1;
+    return launch_pdl(k_reduce_final, 1, 32, 0, st, (const double *)partials, (int)grid, sums, three, (double)amps) ==
+                   cudaSuccess
+               ? 0
+               : -1;
 }
 
-int launch_reduce_final(const double *partials, int nblocks, double *d_result, cudaStream_t st)
+int launch_reduce(const float2 *psi, uint64_t amps, double *d_partials, double *d_result, cudaStream_t st)
 {
-    k_reduce_final<<<1, 32, 0, st>>>(partials, nblocks, d_result);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    return enqueue_reduction(psi, amps, d_partials, d_result, d_result + 4, st);
 }
 
-int launch_result3(double *d_result, double scale, cudaStream_t st)
+int launch_reduce_final(const double *partials, int nblocks, uint64_t amps, double *d_result, cudaStream_t st)
 {
-    k_result3<<<1, 1, 0, st>>>(d_result, scale);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    return launch_pdl(k_reduce_final, 1, 32, 0, st, partials, nblocks, d_result, d_result + 4, (double)amps) ==
+                   cudaSuccess
+               ? 0
+               : -1;
 }
 
 int launch_gather_region(float2 *base, uint64_t lo, uint64_t hi, float2 *buf, uint64_t first, uint64_t count, int n,
@@ -252,22 +265,20 @@ extern "C" int sim_reduce_noalloc(const void *d_state, uint64_t n_amps, double *
         partials = g_noalloc_addr[dev];
     }
     cudaStream_t st = (cudaStream_t)stream;
-    k_reduce_partials<<<kReduceBlocks, kReduceThreads, 0, st>>>((const float4 *)d_state, n_amps / 2,
-                                                                partials);
-    k_reduce_final3<<<1, 32, 0, st>>>(partials, kReduceBlocks, (double)n_amps, d_out);
-    e = cudaGetLastError();
-    if (e != cudaSuccess)
-        return fail(nullptr, SIM_E_CUDA, "sim_reduce_noalloc: launch: %s", cudaGetErrorString(e));
+    if (enqueue_reduction((const float2 *)d_state, n_amps, partials, nullptr, d_out, st) != 0)
+        return fail(nullptr, SIM_E_CUDA, "sim_reduce_noalloc: launch: %s", cudaGetErrorString(cudaGetLastError()));
     return SIM_OK;
 }
 
 namespace sycsim {
 
-int launch_set_basis(float2 *psi, uint64_t amps, uint64_t phys, cudaStream_t st)
+int launch_reset(float2 *psi, uint64_t amps, uint64_t phys, cudaStream_t st)
 {
     if (phys >= amps) return -1;
-    k_set_basis<<<1, 1, 0, st>>>(psi, phys);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    const uint64_t n4 = amps / 2;
+    const uint64_t need = (n4 + 1023) / 1024;  // four 16-byte stores a thread, up to 8 CTAs an SM
+    const unsigned grid = (unsigned)(need < 152 * 8 ? need : 152 * 8);
+    return launch_pdl(k_reset, grid, 256, 0, st, reinterpret_cast<float4 *>(psi), n4, phys) == cudaSuccess ? 0 : -1;
 }
 
 }  // namespace sycsim

@@ -439,8 +439,7 @@ int start_unpacked(srv_t *s, int i, const std::shared_ptr<Req> &r)
                 r->d_t[t] = nullptr;
                 return SIM_E_NOMEM_DEV;
             }
-            if (cudaMemsetAsync(r->d_t[t], 0, sizeof(float2) * ta, st) != cudaSuccess) return SIM_E_CUDA;
-            if (launch_set_basis(r->d_t[t], ta, 0, st) != 0) return SIM_E_CUDA;
+            if (launch_reset(r->d_t[t], ta, 0, st) != 0) return SIM_E_CUDA;
         }
         if (cudaMallocAsync(reinterpret_cast<void **>(&r->d_scratch), contraction_scratch_bytes(r->split.get()), st) !=
             cudaSuccess) {
@@ -449,8 +448,7 @@ int start_unpacked(srv_t *s, int i, const std::shared_ptr<Req> &r)
         }
         return SIM_OK;
     }
-    if (cudaMemsetAsync(r->d_state, 0, sizeof(float2) * amps, st) != cudaSuccess) return SIM_E_CUDA;
-    if (launch_set_basis(r->d_state, amps, 0, st) != 0) return SIM_E_CUDA;
+    if (launch_reset(r->d_state, amps, 0, st) != 0) return SIM_E_CUDA;
     return SIM_OK;
 }
 
@@ -502,7 +500,7 @@ int advance_unpacked(srv_t *s, const std::shared_ptr<Req> &r, bool *progressed)
         const int rc = contract();
         if (rc != SIM_OK) return rc;
     }
-    if (launch_reduce(h, r->d_state, amps, h->d_partials, h->d_result, st) != 0) return SIM_E_CUDA;
+    if (launch_reduce(r->d_state, amps, h->d_partials, h->d_result, st) != 0) return SIM_E_CUDA;
     if (cudaMemcpyAsync(r->h_res, h->d_result, 2 * sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return SIM_E_CUDA;
     if (r->out_amps && !r->back.empty() && launch_permute(h, r->d_state, r->n, r->back.data(), st) != 0)
@@ -667,7 +665,7 @@ int start_graph(srv_t *s, const std::shared_ptr<Req> &r)
     sim_t *h = E.h;
     cudaStream_t st = h->stream;
     if (sim_reset(h, 0) != SIM_OK || sim_graph_launch(h, E.g) != SIM_OK) return SIM_E_CUDA;
-    if (launch_reduce(h, h->d_state, h->amps, h->d_partials, h->d_result, st) != 0) return SIM_E_CUDA;
+    if (launch_reduce(h->d_state, h->amps, h->d_partials, h->d_result, st) != 0) return SIM_E_CUDA;
     if (cudaMemcpyAsync(r->h_res, h->d_result, 2 * sizeof(double), cudaMemcpyDeviceToHost, st) != cudaSuccess)
         return SIM_E_CUDA;
     if (r->out_amps && !E.back.empty() && launch_permute(h, h->d_state, r->n, E.back.data(), st) != 0)

@@ -245,9 +245,8 @@ int sim_reset(sim_t *h, uint64_t basis)
         return fail(h, SIM_E_INVAL, "sim_reset: basis index has bits above n=%d", h->n);
     SIM_DEVICE_SCOPE(h, h->device);
     if (h->store == SIM_STORE_HOST) return host_reset(h, basis);
-    SIM_CUDA_TRY(h, cudaMemsetAsync(h->d_state, 0, h->amps * sizeof(float2), h->stream));
     const int ps = prof_begin(h, SIM_PROF_OTHER, 0.0, h->stream);
-    const int rc = launch_set_basis(h->d_state, h->amps, logical_to_physical(h, basis), h->stream);
+    const int rc = launch_reset(h->d_state, h->amps, logical_to_physical(h, basis), h->stream);
     prof_end(h, ps, h->stream);
     return rc == 0 ? SIM_OK
                    : fail(h, SIM_E_CUDA, "sim_reset: launch failed: %s",
@@ -407,11 +406,11 @@ int enqueue_reduce(sim_t *h)
 {
     if (h->red_epoch == h->write_epoch && h->red_blocks > 0) {
         h->launches++;
-        return launch_reduce_final(h->d_partials, h->red_blocks, h->d_result, h->stream);
+        return launch_reduce_final(h->d_partials, h->red_blocks, h->amps, h->d_result, h->stream);
     }
     const int ps = prof_begin(h, SIM_PROF_REDUCE, 8.0 * (double)h->amps, h->stream);
     h->launches++;  // the reduction is two kernels (partials + final)
-    const int rc = launch_reduce(h, h->d_state, h->amps, h->d_partials, h->d_result, h->stream);
+    const int rc = launch_reduce(h->d_state, h->amps, h->d_partials, h->d_result, h->stream);
     prof_end(h, ps, h->stream);
     return rc;
 }
@@ -427,9 +426,8 @@ int sim_reduce_async(sim_t *h, double *out)
     if (h->store != SIM_STORE_DEVICE)
         return fail(h, SIM_E_UNSUPPORTED, "sim_reduce_async: host-store state: use sim_reduce");
     SIM_DEVICE_SCOPE(h, h->device);
-    if (enqueue_reduce(h) != 0 || launch_result3(h->d_result, std::ldexp(1.0, h->n), h->stream) != 0)
+    if (enqueue_reduce(h) != 0)
         return fail(h, SIM_E_CUDA, "sim_reduce_async: launch failed: %s", cudaGetErrorString(cudaGetLastError()));
-    h->launches++;
     SIM_CUDA_TRY(h, cudaMemcpyAsync(out, h->d_result + 4, sizeof(double) * 3, cudaMemcpyDeviceToHost, h->stream));
     return SIM_OK;
 }

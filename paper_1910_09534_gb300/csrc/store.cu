@@ -359,7 +359,7 @@ int host_reduce(sim_t *h, double *s1, double *s2)
         if (rc != SIM_OK) return rc;
         const int ps = prof_begin(h, SIM_PROF_REDUCE, 8.0 * (double)slice, h->stream);
         h->launches++;
-        rc = launch_reduce(h, h->d_slot[slot], slice, h->d_partials, h->d_result, h->stream);
+        rc = launch_reduce(h->d_slot[slot], slice, h->d_partials, h->d_result, h->stream);
         prof_end(h, ps, h->stream);
         if (rc != 0) return fail(h, SIM_E_CUDA, "sim_reduce: launch failed");
         SIM_CUDA_TRY(h, cudaMemcpyAsync(h->h_partials + 2 * v, h->d_result, sizeof(double) * 2,
