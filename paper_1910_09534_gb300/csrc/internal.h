@@ -282,6 +282,12 @@ int launch_apply_tc(float2 *psi, int nbits, int k, const int *tpos, const float2
 int launch_apply_fp32(sim_t *h, float2 *psi, int nbits, int k, const int *tpos,
                       const float2 *mat, const float2 *mat6_dev, cudaStream_t st);
 
+// ---- plan_cluster.cu: a whole plan on a small state in a few launches (FP32) ----
+bool plan_cluster_eligible(int n, int nblocks, int max_k);
+// block i: k[i] targets tpos[i] (ascending physical bits), matrix mats[i]; *launches: kernels launched
+int launch_plan_cluster(float2 *psi, int n, int nblocks, const int *k, const int *const *tpos,
+                        const float2 *const *mats, cudaStream_t st, int *launches);
+
 // ---- permute.cu ----
 // In-place bit permutation of 2^nbits amplitudes: element i moves to pi(i) where pi
 // moves bit b to bit perm[b].

@@ -39,4 +39,25 @@ cudaError_t launch_pdl(void (*kern)(P...), unsigned grid, unsigned block, size_t
     return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
 }
 
+// The same with the grid in clusters of `cluster` CTAs.
+template <typename... P, typename... A>
+cudaError_t launch_cluster(void (*kern)(P...), unsigned grid, unsigned cluster, unsigned block, size_t smem,
+                           cudaStream_t st, A &&...args)
+{
+    cudaLaunchAttribute attr[2] = {};
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+}
+
 }  // namespace sycsim

@@ -913,6 +913,7 @@ int sim_apply_plan(sim_t *h, const sim_plan_t *p)
     const size_t nb = p->blocks.size();
     prep.resize(nb);
     size_t mtot = 0, total = 0;
+    int max_k = 0;
     for (size_t i = 0; i < nb; i++) mtot += (size_t)1 << (2 * p->blocks[i].qubits.size());
     mats.resize(mtot);
     mtot = 0;
@@ -927,6 +928,27 @@ int sim_apply_plan(sim_t *h, const sim_plan_t *p)
         pb.bytes = block_staged_bytes(pb.k);
         pb.off = total;
         total += (pb.bytes + 255) & ~size_t(255);
+        max_k = std::max(max_k, pb.k);
+    }
+    if (p->precision == SIM_FP32 && plan_cluster_eligible(h->n, (int)nb, max_k)) {
+        // a small state: its blocks are applied by one cluster, many a launch
+        std::vector<int> ks(nb);
+        std::vector<const int *> tp(nb);
+        std::vector<const float2 *> ms(nb);
+        for (size_t i = 0; i < nb; i++) {
+            ks[i] = prep[i].k;
+            tp[i] = prep[i].tpos;
+            ms[i] = mats.data() + prep[i].moff;
+        }
+        const int ps = prof_begin(h, SIM_PROF_APPLY, 16.0 * std::ldexp((double)nb, h->n), h->stream);
+        int launches = 0;
+        const int rc = launch_plan_cluster(h->d_state, h->n, (int)nb, ks.data(), tp.data(), ms.data(), h->stream,
+                                           &launches);
+        prof_end(h, ps, h->stream);
+        h->launches += launches > 1 ? launches - 1 : 0;  // prof_begin counted one
+        h->red_blocks = 0;
+        return rc == 0 ? SIM_OK
+                       : fail(h, SIM_E_CUDA, "sim_apply_plan: launch failed: %s", cudaGetErrorString(cudaGetLastError()));
     }
     char *d_ops = nullptr;
     int slot = -1;

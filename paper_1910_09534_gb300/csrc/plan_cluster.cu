@@ -1,0 +1,101 @@
+// plan_cluster.cu -- a plan's blocks on a small state, many a launch (cluster_run.cuh).
+#include <cuda_runtime.h>
+
+#include <atomic>
+#include <cstring>
+
+#include "cluster_run.cuh"
+#include "internal.h"
+#include "pdl.cuh"
+
+namespace sycsim {
+namespace {
+
+// A launch's blocks: as many as fit the parameter space (14 of 4 qubits, 3 of 5), so that nothing is
+// uploaded and the launch can be captured; a longer plan takes several launches.
+constexpr int kTableBlocks = 14;
+constexpr int kTableElems = kTableBlocks * 256;
+struct PlanTable {
+    ClBlock blocks[kTableBlocks];
+    alignas(16) float2 mats[kTableElems];
+};
+
+__global__ void __launch_bounds__(kClThreads, 1) k_plan_cluster(float2 *psi, int n, int nblocks,
+                                                                const __grid_constant__ PlanTable t)
+{
+    __shared__ ClShared sh;
+    pdl_launch_next();
+    const float2 *mats = t.mats;
+    asm volatile("" : "+l"(mats));  // read with ordinary loads, not as constants (block_mat.cuh)
+    pdl_wait();
+    cl_run_blocks(psi, n, t.blocks, mats, nblocks, sh);
+}
+
+}  // namespace
+
+// CTAs of the cluster on the current device: 16 (beyond the portable 8) where the device can place
+// such a cluster, else 8.
+static int plan_ctas()
+{
+    static std::atomic<uint64_t> wide{0}, known{0};  // bit d: device d < 64
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 8;
+    const uint64_t bit = 1ull << dev;
+    if (!(known.load(std::memory_order_acquire) & bit)) {
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = 16;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(16);
+        cfg.blockDim = dim3(kClThreads);
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaFuncSetAttribute(k_plan_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&n, k_plan_cluster, &cfg) == cudaSuccess && n > 0)
+            wide.fetch_or(bit, std::memory_order_acq_rel);
+        else
+            cudaGetLastError();  // not an error of this call: the narrower cluster is used
+        known.fetch_or(bit, std::memory_order_acq_rel);
+    }
+    return wide.load(std::memory_order_acquire) & bit ? 16 : 8;
+}
+
+// Where one cluster is faster than a launch per block on all SMs.  Measured (12 cycles, us a plan,
+// cluster of 16 / of 8 / separate launches from a CUDA graph): k_max 4: 12 qubits 23 / 25 / 45, 14
+// qubits 39 / 41 / 63, 15 qubits 48 / 67 / 76, 16 qubits 60 / 101 / 74, 17 qubits 121 / 215 / 89; k_max
+// 5, whose separate kernel is slow to start: 14 qubits 50 / 68 / 158, 16 qubits 87 / 131 / 230, 17 qubits
+// 138 / 246 / 230, 18 qubits 280 / 524 / 259.
+bool plan_cluster_eligible(int n, int nblocks, int max_k)
+{
+    if (nblocks < 2 || max_k > kClMaxK) return false;
+    const int top = max_k == 5 ? 17 : 16;
+    return n <= top - 1 || (n <= top && plan_ctas() == 16);
+}
+
+int launch_plan_cluster(float2 *psi, int n, int nblocks, const int *k, const int *const *tpos,
+                        const float2 *const *mats, cudaStream_t st, int *launches)
+{
+    static thread_local PlanTable t;
+    *launches = 0;
+    const int ctas = plan_ctas();
+    for (int i = 0; i < nblocks;) {
+        int c = 0;
+        uint32_t off = 0;
+        for (; i < nblocks && c < kTableBlocks && off + (1u << (2 * k[i])) <= (uint32_t)kTableElems; i++, c++) {
+            ClBlock &b = t.blocks[c];
+            b.k = k[i];
+            for (int q = 0; q < kMaxK; q++) b.tpos[q] = q < k[i] ? tpos[i][q] : 0;
+            b.mat_off = off;
+            std::memcpy(t.mats + off, mats[i], sizeof(float2) << (2 * k[i]));
+            off += 1u << (2 * k[i]);
+        }
+        if (launch_cluster(k_plan_cluster, ctas, ctas, kClThreads, 0, st, psi, n, c, t) != cudaSuccess)
+            return -1;
+        ++*launches;
+    }
+    return 0;
+}
+
+}  // namespace sycsim
