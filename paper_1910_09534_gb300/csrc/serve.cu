@@ -9,10 +9,10 @@
 //    scratch) fits the HBM budget; a request that does not fit may be overtaken by smaller
 //    ones at most kMaxBypass times, after which admission waits for it (no starvation);
 //  * runs small circuits (n <= small_n) through a device-side queue served by a persistent
-//    worker kernel (k_packed_worker): one CTA runs one whole circuit -- reset, every block, the
+//    worker kernel (k_packed_worker): one cluster of CTAs runs one whole circuit -- reset, every block, the
 //    reduction -- with the block matrix in shared memory; circuits are uploaded in units, published
-//    to the queue, claimed by idle CTAs of a worker already running (or of a new one when the
-//    running workers have fewer CTAs than jobs waiting), and a worker leaves after 200 us without
+//    to the queue, claimed by idle clusters of a worker already running (or of a new one when the
+//    running workers have fewer clusters than jobs waiting), and a worker leaves after 200 us without
 //    new work, so small circuits that arrive while others run start without a new launch;
 //  * runs larger circuits on one of several slot streams with stream-ordered allocation, so
 //    circuits of different sizes overlap on the device; their blocks are enqueued a few at a
@@ -38,6 +38,7 @@
 #include <unordered_map>
 #include <vector>
 
+#include "cluster_run.cuh"
 #include "internal.h"
 
 namespace sycsim {
@@ -45,11 +46,7 @@ namespace {
 
 using Clock = std::chrono::steady_clock;
 
-struct PackedBlock {
-    int k;
-    int tpos[kMaxK];
-    uint32_t mat_off;  // float2 offset of the block's matrix in the batch's matrix table
-};
+using PackedBlock = ClBlock;
 
 struct PackedJob {
     float2 *psi;
@@ -59,89 +56,31 @@ struct PackedJob {
     int n, nblocks;
 };
 
-constexpr int kPackThreads = 256;
-constexpr int kPackMaxK = 5;
-
-__device__ __forceinline__ uint64_t insert_zero_bits_s(uint64_t x, const int *pos, int cnt)
-{
-    for (int i = 0; i < cnt; ++i) {
-        const int p = pos[i];
-        const uint64_t lo = x & ((1ull << p) - 1);
-        x = ((x >> p) << (p + 1)) | lo;
-    }
-    return x;
-}
-
-template <int K>
-__device__ __forceinline__ void cta_block(float2 *psi, int n, const int *tpos, const float2 *M,
-                                          const uint32_t *moff)
-{
-    constexpr int D = 1 << K;
-    const uint64_t ngroups = 1ull << (n - K);
-    for (uint64_t gi = threadIdx.x; gi < ngroups; gi += blockDim.x) {
-        float2 *p = psi + insert_zero_bits_s(gi, tpos, K);
-        float2 x[D];
-#pragma unroll
-        for (int j = 0; j < D; ++j) x[j] = p[moff[j]];
-#pragma unroll
-        for (int r = 0; r < D; ++r) {
-            float yr = 0.f, yi = 0.f;
-#pragma unroll
-            for (int c = 0; c < D; ++c) {
-                const float2 m = M[r * D + c];
-                yr = fmaf(m.x, x[c].x, yr);
-                yr = fmaf(m.y, -x[c].y, yr);
-                yi = fmaf(m.x, x[c].y, yi);
-                yi = fmaf(m.y, x[c].x, yi);
-            }
-            p[moff[r]] = make_float2(yr, yi);
-        }
-    }
-}
+constexpr int kPackMaxK = kClMaxK;
+constexpr int kPackCtas = 8;  // CTAs of the cluster that runs one packed circuit
 
 struct PackShared {
-    float2 M[32 * 32];
-    uint32_t moff[32];
-    int tpos[kMaxK];
-    double red[2][kPackThreads / 32];
+    ClShared run;
+    double red[2][kClThreads / 32];
+    double part[2][kPackCtas];  // the leader's: each CTA's sums
 };
 
-// One whole small circuit on one CTA: reset to |0...0>, every block with its matrix in shared
-// memory, then (sum p, sum p^2) into out[0..1].
-__device__ void run_circuit_cta(const PackedJob &J, PackShared &sh, double *out)
+// One whole small circuit on one cluster: reset to |0...0>, every block (cluster_run.cuh), then
+// (sum p, sum p^2) into out[0..1].  Measured one CTA to a circuit before: 18 qubits, 12 cycles 5.4
+// ms, with the other SMs idle unless many circuits were waiting.
+__device__ __forceinline__ void run_circuit_cluster(const PackedJob &J, PackShared &sh, double *out)
 {
-    float2 *M = sh.M;
-    uint32_t *moff = sh.moff;
-    int *tpos = sh.tpos;
-    const uint64_t amps = 1ull << J.n;
-    for (uint64_t i = threadIdx.x; i < amps; i += blockDim.x) J.psi[i] = make_float2(0.f, 0.f);
-    __syncthreads();
-    if (threadIdx.x == 0) J.psi[0] = make_float2(1.f, 0.f);
-    for (int b = 0; b < J.nblocks; ++b) {
-        const PackedBlock B = J.blocks[b];
-        const int D = 1 << B.k;
-        __syncthreads();  // previous block done with M, psi and tpos
-        for (int i = threadIdx.x; i < D * D; i += blockDim.x) M[i] = J.mats[B.mat_off + i];
-        if (threadIdx.x < D) {
-            uint32_t o = 0;
-            for (int q = 0; q < B.k; ++q)
-                if ((threadIdx.x >> q) & 1) o += 1u << B.tpos[q];
-            moff[threadIdx.x] = o;
-        }
-        if (threadIdx.x < kMaxK) tpos[threadIdx.x] = B.tpos[threadIdx.x];
-        __syncthreads();
-        switch (B.k) {
-        case 1: cta_block<1>(J.psi, J.n, tpos, M, moff); break;
-        case 2: cta_block<2>(J.psi, J.n, tpos, M, moff); break;
-        case 3: cta_block<3>(J.psi, J.n, tpos, M, moff); break;
-        case 4: cta_block<4>(J.psi, J.n, tpos, M, moff); break;
-        default: cta_block<5>(J.psi, J.n, tpos, M, moff); break;
-        }
-    }
-    __syncthreads();
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const uint32_t rank = cl.block_rank();
+    const uint64_t amps = 1ull << J.n, step = (uint64_t)kPackCtas * kClThreads;
+    const uint64_t first = (uint64_t)rank * kClThreads + threadIdx.x;
+    for (uint64_t i = first; i < amps; i += step) J.psi[i] = make_float2(i == 0 ? 1.f : 0.f, 0.f);
+    if (J.nblocks == 0) cl.sync();
+    cl_run_blocks(J.psi, J.n, J.blocks, J.mats, J.nblocks, sh.run);
     double s1 = 0.0, s2 = 0.0;
-    for (uint64_t i = threadIdx.x; i < amps; i += blockDim.x) {
-        const float2 v = J.psi[i];
+    for (uint64_t i = first; i < amps; i += step) {
+        const float2 v = __ldcg(J.psi + i);
         const double p = (double)v.x * v.x + (double)v.y * v.y;
         s1 += p;
         s2 += p * p;
@@ -158,9 +97,20 @@ __device__ void run_circuit_cta(const PackedJob &J, PackShared &sh, double *out)
     __syncthreads();
     if (threadIdx.x == 0) {
         double a = 0.0, c = 0.0;
-        for (int w = 0; w < kPackThreads / 32; ++w) {
+        for (int w = 0; w < kClThreads / 32; ++w) {
             a += sh.red[0][w];
             c += sh.red[1][w];
+        }
+        PackShared *lead = cl.map_shared_rank(&sh, 0);
+        lead->part[0][rank] = a;
+        lead->part[1][rank] = c;
+    }
+    cl.sync();
+    if (rank == 0 && threadIdx.x == 0) {  // in the order of the CTAs
+        double a = 0.0, c = 0.0;
+        for (int r = 0; r < kPackCtas; ++r) {
+            a += sh.part[0][r];
+            c += sh.part[1][r];
         }
         out[0] = a;
         out[1] = c;
@@ -193,18 +143,24 @@ __device__ __forceinline__ uint32_t ld_acquire_sys(const uint32_t *p)
     return v;
 }
 
-// Persistent worker: each CTA claims the next published job (compare-and-swap on the claim
-// counter, so no claimed index is ever abandoned), runs it, publishes its results and done flag,
-// and looks for the next one; it leaves once no job has been published for kWorkerIdleNs.  Jobs
-// published while the kernel runs are picked up without a new launch.  The only wait is on the
-// host's published count, bounded by the idle time.
-__global__ void __launch_bounds__(kPackThreads) k_packed_worker(const uint32_t *published, QSlot *ring, uint32_t *head)
+// Persistent worker: the leading CTA of each cluster claims the next published job
+// (compare-and-swap on the claim counter, so no claimed index is ever abandoned) and hands it to the
+// others; together they run it, the leader publishes its results and done flag and looks for the
+// next one; the cluster leaves once no job has been published for kWorkerIdleNs.  Jobs published while
+// the kernel runs are picked up without a new launch.  The only wait for the host is on its published
+// count, bounded by the idle time; the cluster's barriers wait for CTAs that are resident together.
+__global__ void __cluster_dims__(kPackCtas, 1, 1) __launch_bounds__(kClThreads, 2)
+    k_packed_worker(const uint32_t *published, QSlot *ring, uint32_t *head)
 {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
     __shared__ PackShared sh;
     __shared__ PackedJob J;
     __shared__ uint32_t job;
+    const bool lead = cl.block_rank() == 0 && threadIdx.x == 0;
+    cl.sync();  // every CTA has started before any writes another's shared memory
     for (;;) {
-        if (threadIdx.x == 0) {
+        if (lead) {
             uint32_t got = 0xffffffffu;
             const uint64_t t0 = pack_now_ns();
             for (;;) {
@@ -220,19 +176,22 @@ __global__ void __launch_bounds__(kPackThreads) k_packed_worker(const uint32_t *
                 if (pack_now_ns() - t0 > kWorkerIdleNs) break;
                 __nanosleep(1000);
             }
-            job = got;
-            if (got != 0xffffffffu) J = ring[got % kQueueCap].job;
+            PackedJob mine{};
+            if (got != 0xffffffffu) mine = ring[got % kQueueCap].job;
+            for (int r = 0; r < kPackCtas; ++r) {
+                *cl.map_shared_rank(&job, r) = got;
+                *cl.map_shared_rank(&J, r) = mine;
+            }
         }
-        __syncthreads();
+        cl.sync();
         if (job == 0xffffffffu) break;
         QSlot *slot = ring + job % kQueueCap;
-        run_circuit_cta(J, sh, slot->res);
-        __syncthreads();
-        if (threadIdx.x == 0) {
+        run_circuit_cluster(J, sh, slot->res);
+        if (lead) {
             __threadfence_system();  // results visible to the host before the flag
             asm volatile("st.release.sys.global.u32 [%0], %1;" ::"l"(&slot->done), "r"(1u) : "memory");
         }
-        __syncthreads();  // job and J are rewritten by the next claim
+        cl.sync();  // job and J are rewritten by the next claim
     }
 }
 
@@ -298,6 +257,7 @@ struct Batch {
     cudaEvent_t ev = nullptr;       // upload done, then copy-out done
     void *d_mem = nullptr;          // states + tables, one stream-ordered allocation
     char *h_stage = nullptr;        // pinned copy source of the tables
+    std::vector<char *> outgrown;   // its smaller predecessors
     size_t stage_bytes = 0;
     uint64_t first = 0;             // queue index of the first job
     State state = Free;
@@ -345,7 +305,7 @@ struct srv_s {
     uint64_t next_index = 0, published = 0, retired = 0;
     cudaStream_t wst[2] = {nullptr, nullptr};
     cudaEvent_t wev[2] = {nullptr, nullptr};
-    int wctas[2] = {0, 0};  // CTAs of a worker still running (0: none)
+    int wclusters[2] = {0, 0};  // clusters of a worker still running (0: none)
     int sms = 0;
     double *h_results = nullptr;  // pinned ring of result pairs for unpacked requests
     std::thread worker;
@@ -551,7 +511,10 @@ int upload_packed(srv_t *s, Batch &B)
     const size_t table_bytes = off_state;
     const size_t total = off_state + state_amps * sizeof(float2);
     if (B.stage_bytes < table_bytes) {
-        if (B.h_stage) cudaFreeHost(B.h_stage);
+        // the outgrown buffer is given back with the server: cudaFreeHost waits for the kernels that
+        // run, here with the lock held (9 ms stalls of srv_submit); sizes at least double, so the
+        // kept ones add up to less than the last
+        if (B.h_stage) B.outgrown.push_back(B.h_stage);
         B.h_stage = nullptr;
         B.stage_bytes = 0;  // a failed allocation leaves no buffer behind
         if (cudaHostAlloc(&B.h_stage, table_bytes * 2, cudaHostAllocDefault) != cudaSuccess) {
@@ -636,22 +599,22 @@ int copy_out_packed(Batch &B)
     return rc;
 }
 
-// Jobs published and not yet seen done; launch a worker when they outnumber the CTAs of the
+// Jobs published and not yet seen done; launch a worker when they outnumber the clusters of the
 // workers still running (scheduler thread, lock held).
 void manage_workers(srv_t *s, uint64_t not_done, bool *progressed)
 {
     int running = 0;
     for (int w = 0; w < 2; w++) {
-        if (s->wctas[w] && cudaEventQuery(s->wev[w]) != cudaErrorNotReady) s->wctas[w] = 0;
-        running += s->wctas[w];
+        if (s->wclusters[w] && cudaEventQuery(s->wev[w]) != cudaErrorNotReady) s->wclusters[w] = 0;
+        running += s->wclusters[w];
     }
     if (not_done <= (uint64_t)running) return;
     for (int w = 0; w < 2; w++)
-        if (!s->wctas[w]) {
-            const int ctas = (int)std::min<uint64_t>(not_done - running, (uint64_t)(2 * s->sms));
-            k_packed_worker<<<ctas, kPackThreads, 0, s->wst[w]>>>(s->d_ctl, s->d_ring, s->d_head);
+        if (!s->wclusters[w]) {
+            const int clusters = (int)std::min<uint64_t>(not_done - running, (uint64_t)(2 * s->sms / kPackCtas));
+            k_packed_worker<<<clusters * kPackCtas, kClThreads, 0, s->wst[w]>>>(s->d_ctl, s->d_ring, s->d_head);
             if (cudaGetLastError() != cudaSuccess || cudaEventRecord(s->wev[w], s->wst[w]) != cudaSuccess) return;
-            s->wctas[w] = ctas;
+            s->wclusters[w] = clusters;
             *progressed = true;
             return;
         }
@@ -901,6 +864,7 @@ void srv_release(srv_t *s)
         if (B.ev) cudaEventDestroy(B.ev);
         if (B.st) cudaStreamDestroy(B.st);
         if (B.h_stage) cudaFreeHost(B.h_stage);
+        for (char *p : B.outgrown) cudaFreeHost(p);
     }
     if (s->ring) cudaFreeHost(s->ring);
     if (s->ctl) cudaFreeHost(s->ctl);
@@ -1130,7 +1094,7 @@ int srv_submit(srv_t *s, int n_qubits, int n_gates, const sim_gate *gates, void 
         s->rejected++;
         return srv_fail(s, rc, "srv_submit: %s", sim_last_error(nullptr));
     }
-    // where the qubits sit: the identity for packed circuits (one CTA each, no HBM passes); for
+    // where the qubits sit: the identity for packed circuits (one cluster each, in the L2); for
     // the others the layout sim_plan_layout picks, the state permuted back before a readout
     int phys[kMaxQubits];
     for (int q = 0; q < kMaxQubits; q++) phys[q] = q;
@@ -1327,7 +1291,7 @@ int srv_autotune(srv_t *s, int n_samples, const int *n_qubits, const int *n_gate
         if (kmax_out) kmax_out[i] = 0;
         if (front_out) front_out[i] = 0;
         if (ms_out) ms_out[i] = 0.0;
-        if (n <= s->o.small_n) continue;  // packed: one CTA per circuit, blocks of <= 5 qubits
+        if (n <= s->o.small_n) continue;  // packed: one cluster per circuit, blocks of <= 5 qubits
         sim_opts so{};
         so.device = s->o.device;
         sim_t *h = nullptr;
