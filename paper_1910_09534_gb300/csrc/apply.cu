@@ -6,21 +6,24 @@
 // Each group is replaced by M times itself.  One pass reads and writes every amplitude
 // once: 16 bytes per amplitude of HBM traffic, 8 * 2^k - 2 real flops per amplitude.
 //
-// Three kernels:
-//  * reg (default for k <= 5, n >= k + 5) -- see the comment above k_apply_reg: persistent
-//    warps, register-resident groups, warp-shuffle exchange for targets below bit 5.
+// Four kernels:
+//  * reg (default for k <= 4, n >= k + 5) -- see the comment above k_apply_reg: persistent warps,
+//    register-resident groups, an exchange through the warp's own shared memory for targets
+//    below bit 5.
+//  * rtile (k = 5, 6, n >= k + 6) -- see above k_apply_rtile: tiles in shared memory, each thread a
+//    register tile of rows x groups, the matrix in shared memory.
 //  * direct -- every target >= 5: thread = group; the 32 threads of a warp take 32
 //    consecutive groups, so each member load/store is one contiguous 256-byte run.
 //    Amplitudes go straight to registers; no shared memory.  Used for k <= 3.
-//  * tiled -- small states and k = 6: a CTA stages a tile of 2^(F+k) amplitudes (2^h rows of
+//  * tiled -- the smallest states: a CTA stages a tile of 2^(F+k) amplitudes (2^h rows of
 //    2^m contiguous amplitudes, the rows indexed by the h targets >= m) through shared
 //    memory with coalesced loads, each of its 2^F threads applies M to one group, and
 //    the tile is written back.  An XOR swizzle maps the low target bits onto free bits
 //    so that shared-memory accesses stay conflict-free for any target set.
 //
-// The matrix (FP32, complex64) is a kernel parameter for k <= 5: the FMAs read it
-// straight from the constant bank.  k = 6 (32 KiB) exceeds the parameter space and is
-// read from device memory into shared memory once per CTA.
+// The matrix (FP32, complex64) is a kernel parameter for k <= 5: up to k = 4 (2 KiB) the FMAs read it
+// straight from the constant bank; k = 5, 6 (8, 32 KiB, more than the constant cache keeps) are
+// copied to shared memory once per CTA, k = 6 from device memory.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -49,7 +52,7 @@ struct DirectGeom {
     float2 *psi;
     uint64_t n_groups;
     int tpos[kMaxK];     // ascending physical target bits
-    uint64_t moff[64];   // offset of member j
+    uint64_t moff[8];    // offset of member j (k <= 3)
 };
 
 struct TiledGeom {
@@ -149,18 +152,14 @@ __device__ __forceinline__ void stage_matrix(float2 *sm, const float2 *gm)
 }
 
 // Occupancy targets (CTAs per SM) that bound the register count of each width.
-constexpr int direct_min_blocks(int k) { return k <= 3 ? 4 : (k <= 5 ? 2 : 1); }
 constexpr int tiled_threads(int k) { return k <= 4 ? 256 : (k == 5 ? 128 : 64); }
 constexpr int tiled_min_blocks(int k) { return k <= 3 ? 4 : (k <= 5 ? 2 : 4); }
 
-template <int K, typename MatSrc>
-__global__ void __launch_bounds__(256, direct_min_blocks(K)) k_apply_direct(DirectGeom g, MatSrc M)
+template <int K>
+__global__ void __launch_bounds__(256, 4) k_apply_direct(DirectGeom g, MatP<K> M)
 {
     constexpr int D = 1 << K;
-    constexpr bool kSmemMat = std::is_same<MatSrc, MatPtr>::value;
-    extern __shared__ float2 smem[];
     pdl_launch_next();
-    if constexpr (kSmemMat) stage_matrix<K>(smem, M.p);
     const uint64_t gi = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (gi >= g.n_groups) return;
     pdl_wait();
@@ -169,11 +168,8 @@ __global__ void __launch_bounds__(256, direct_min_blocks(K)) k_apply_direct(Dire
 #pragma unroll
     for (int j = 0; j < D; ++j) x[j] = __ldcs(p + g.moff[j]);
     float2 *const q = opaque(p);
-    auto st = [&](int r, float2 y) { __stcs(q + g.moff[r], y); };
-    if constexpr (kSmemMat)
-        apply_group<K, false>(x, [&](int r, int c) { return smem[r * D + c]; }, st);
-    else
-        apply_group<K, true>(x, [&](int r, int c) { return M.m[r * D + c]; }, st);
+    apply_group<K, true>(x, [&](int r, int c) { return M.m[r * D + c]; },
+                         [&](int r, float2 y) { __stcs(q + g.moff[r], y); });
 }
 
 template <int K, typename MatSrc>
@@ -239,30 +235,30 @@ cudaError_t ensure_smem(Kern kern, size_t bytes)
     return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
+template <int K>
+int launch_direct(float2 *psi, int nbits, const int *tpos, const MatP<K> &M, cudaStream_t st)
+{
+    constexpr int D = 1 << K;
+    DirectGeom g{};
+    g.psi = psi;
+    g.n_groups = 1ull << (nbits - K);
+    for (int i = 0; i < K; i++) g.tpos[i] = tpos[i];
+    for (int j = 0; j < D; j++) {
+        uint64_t o = 0;
+        for (int b = 0; b < K; b++)
+            if ((j >> b) & 1) o += 1ull << tpos[b];
+        g.moff[j] = o;
+    }
+    const uint64_t blocks = (g.n_groups + 255) / 256;
+    return launch_pdl(k_apply_direct<K>, (unsigned)blocks, 256, 0, st, g, M) == cudaSuccess ? 0 : -1;
+}
+
 template <int K, typename MatSrc>
-int launch_k(float2 *psi, int nbits, const int *tpos, const MatSrc &M, cudaStream_t st)
+int launch_tiled(float2 *psi, int nbits, const int *tpos, const MatSrc &M, cudaStream_t st)
 {
     constexpr int D = 1 << K;
     constexpr bool kSmemMat = std::is_same<MatSrc, MatPtr>::value;
     const size_t mat_bytes = kSmemMat ? sizeof(float2) * D * D : 0;
-    const bool direct = tpos[0] >= 5 && nbits - K >= 8;
-    if (direct) {
-        DirectGeom g{};
-        g.psi = psi;
-        g.n_groups = 1ull << (nbits - K);
-        for (int i = 0; i < K; i++) g.tpos[i] = tpos[i];
-        for (int j = 0; j < D; j++) {
-            uint64_t o = 0;
-            for (int b = 0; b < K; b++)
-                if ((j >> b) & 1) o += 1ull << tpos[b];
-            g.moff[j] = o;
-        }
-        const uint64_t blocks = (g.n_groups + 255) / 256;
-        auto kern = k_apply_direct<K, MatSrc>;
-        if (ensure_smem(kern, mat_bytes) != cudaSuccess) return -1;
-        return launch_pdl(kern, (unsigned)blocks, 256, mat_bytes, st, g, M) == cudaSuccess ? 0 : -1;
-    }
-
     TiledGeom g{};
     g.psi = psi;
     g.F = std::min(tiled_F(K), nbits - K);
@@ -322,16 +318,29 @@ int launch_k(float2 *psi, int nbits, const int *tpos, const MatSrc &M, cudaStrea
 }
 
 // ---------------------------------------------------------------------------------------
-// Register-resident apply for k <= 5 (the default path when n >= k + 5).
+// Register-resident apply for k <= 4 (the default path when n >= k + 5).
 //
 // A warp owns a "warp tile": 32 lanes (index bits 0..4) x 2^k registers.  Register bit
 // j < J (J = number of targets below bit 5) first stands for a free index bit E_j >= 5,
 // register bits j >= J for the high targets.  Loads and stores are therefore 256-byte runs
-// per register.  Each low target t_j (a lane bit) is then exchanged with register bit j by
-// warp shuffles, after which every lane holds one complete group in registers and applies M
-// with the matrix read from the constant bank; the same exchanges undo the transpose before
-// the stores.  Warps are persistent.  (Double-buffering the next tile in registers was
-// measured slower than simply running more CTAs per SM, so it is off by default.)
+// per register.  Each low target t_j (a lane bit) is then exchanged with register bit j, after
+// which every lane holds one complete group in registers and applies M with the matrix read from
+// the constant bank; the same exchange undoes the transpose before the stores.  Warps are
+// persistent.  (Double-buffering the next tile in registers was measured slower than simply
+// running more CTAs per SM.)
+//
+// The exchange goes through 2^(k+5) amplitudes of shared memory that only this warp uses.  Register x
+// of lane l is written at x 32 + (l ^ s(x)), s(x) = sum of bit j of x << t_j, and lane l's register r
+// of the transpose is found at ((r without its J low bits) + (the J target bits of l)) 32 + (l ^ s(r)):
+// for one register the 16 lanes of an access phase cover 16 distinct bank pairs either way, and each
+// lane's results go back where it read its members, so two __syncwarp a tile are all the ordering.
+// 2^(k+2) 8-byte accesses a tile whatever J is; exchanging by warp shuffles took 4 J 2^k instructions
+// (two shuffles and four selects a pair, both ways), which made k = 4 issue-bound (79 % issue active).
+// Measured on 2^28 amplitudes, J = 1 .. k targets below bit 5, us a pass (the traffic alone: 641):
+// k = 4 831, 904, 988, 1074 by shuffles -> 818, 804, 803, 799 (708 with J = 0: the accesses and their
+// addresses are still issued beside 1024 FMAs a tile); k = 3 673, 695, 777 -> 675, 688, 681; k = 1, 2
+// with J = k 755, 681 -> 696, 652.  Staging whole tiles with cp.async instead, group a thread: k = 4
+// 820-1030, k = 3 654-674.
 // ---------------------------------------------------------------------------------------
 struct RegGeom {
     float2 *psi;
@@ -340,59 +349,18 @@ struct RegGeom {
     int lt[5];          // their bit positions (lane bits), ascending
     int nfix;           // index bits >= 5 owned by registers (high targets + E), ascending
     int fix[kMaxK];
-    uint64_t xoff[32];  // offset of register x (pre-exchange meaning)
+    uint64_t xoff[16];  // offset of register x (pre-exchange meaning)
+    uint32_t cw[16];    // byte address in the warp's exchange tile: (8 lane) ^ cw[x] before the
+    uint32_t cr[16];    // exchange, (8 lane | 256 (its target bits)) ^ cr[r] after it
 };
 
-template <int K>
-__device__ __forceinline__ void lane_reg_exchange(float2 (&v)[1 << K], const RegGeom &g, int lane)
-{
-#pragma unroll
-    for (int b = 0; b < (K < 5 ? K : 5); ++b) {
-        if (b < g.J) {
-            const int t = g.lt[b];
-            const bool s = (lane >> t) & 1;
-#pragma unroll
-            for (int x = 0; x < (1 << K); ++x) {
-                if (x & (1 << b)) continue;
-                const int x1 = x | (1 << b);
-                const float2 send = s ? v[x] : v[x1];
-                float2 r;
-                r.x = __shfl_xor_sync(0xffffffffu, send.x, 1 << t);
-                r.y = __shfl_xor_sync(0xffffffffu, send.y, 1 << t);
-                v[x] = s ? r : v[x];
-                v[x1] = s ? v[x1] : r;
-            }
-        }
-    }
-}
-
-// Tuning constants (overridable at build time): widest k that double-buffers the next tile
-// in registers, and the CTAs per SM each width is compiled for.
-#ifndef SYCSIM_REG_PREFETCH_KMAX
-#define SYCSIM_REG_PREFETCH_KMAX 0
-#endif
-#ifndef SYCSIM_REG_MINB_K3
-#define SYCSIM_REG_MINB_K3 4
-#endif
-#ifndef SYCSIM_REG_MINB_K4
-#define SYCSIM_REG_MINB_K4 3
-#endif
-#ifndef SYCSIM_REG_MINB_K5
-#define SYCSIM_REG_MINB_K5 1
-#endif
-constexpr bool reg_prefetch(int k) { return k <= SYCSIM_REG_PREFETCH_KMAX; }
-constexpr int reg_min_blocks(int k, bool low)
-{
-    return k <= 2 ? 4
-                  : (k == 3 ? SYCSIM_REG_MINB_K3
-                            : (k == 4 ? SYCSIM_REG_MINB_K4 : (low ? SYCSIM_REG_MINB_K5 : 2)));
-}
+constexpr int reg_min_blocks(int k) { return k <= 3 ? 4 : 3; }
 
 template <int K, bool kLow>
-__global__ void __launch_bounds__(256, reg_min_blocks(K, kLow)) k_apply_reg(RegGeom g, MatP<K> M)
+__global__ void __launch_bounds__(256, reg_min_blocks(K)) k_apply_reg(RegGeom g, MatP<K> M)
 {
     constexpr int D = 1 << K;
-    constexpr bool kPrefetch = reg_prefetch(K);
+    __shared__ float2 xch[kLow ? 8 * 32 * D : 1];
     pdl_launch_next();
     pdl_wait();
     const int lane = threadIdx.x & 31;
@@ -403,6 +371,14 @@ __global__ void __launch_bounds__(256, reg_min_blocks(K, kLow)) k_apply_reg(RegG
         return g.psi + insert_zero_bits(wt << 5, g.fix, g.nfix) + lane;
     };
     auto MatAt = [&](int r, int c) { return M.m[r * D + c]; };
+    uint8_t *const my = reinterpret_cast<uint8_t *>(xch + (kLow ? (threadIdx.x >> 5) * 32 * D : 0));
+    const uint32_t bw = 8 * lane;
+    uint32_t br = bw;
+    if constexpr (kLow) {
+#pragma unroll
+        for (int b = 0; b < 5; ++b)
+            if (b < g.J) br |= (uint32_t)((lane >> g.lt[b]) & 1) << (8 + b);
+    }
     float2 x[D];
     {
         const float2 *p = tile_ptr(w);
@@ -411,29 +387,23 @@ __global__ void __launch_bounds__(256, reg_min_blocks(K, kLow)) k_apply_reg(RegG
     }
     for (; w < g.n_wtiles; w += nw) {
         const uint64_t wn = w + nw;
-        float2 xn[D];
-        if constexpr (kPrefetch) {
-            if (wn < g.n_wtiles) {
-                const float2 *pn = tile_ptr(wn);
-#pragma unroll
-                for (int j = 0; j < D; ++j) xn[j] = __ldcs(pn + g.xoff[j]);
-            }
-        }
         float2 *const q = opaque(tile_ptr(w));
         if constexpr (kLow) {
-            lane_reg_exchange<K>(x, g, lane);
-            float2 y[D];
-            apply_group<K, true>(x, MatAt, [&](int r, float2 v) { y[r] = v; });
-            lane_reg_exchange<K>(y, g, lane);
 #pragma unroll
-            for (int j = 0; j < D; ++j) __stcs(q + g.xoff[j], y[j]);
+            for (int j = 0; j < D; ++j) *reinterpret_cast<float2 *>(my + (bw ^ g.cw[j])) = x[j];
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < D; ++j) x[j] = *reinterpret_cast<const float2 *>(my + (br ^ g.cr[j]));
+            apply_group<K, true>(x, MatAt,
+                                 [&](int r, float2 v) { *reinterpret_cast<float2 *>(my + (br ^ g.cr[r])) = v; });
+            __syncwarp();
+#pragma unroll
+            for (int j = 0; j < D; ++j)
+                __stcs(q + g.xoff[j], *reinterpret_cast<const float2 *>(my + (bw ^ g.cw[j])));
         } else {
             apply_group<K, true>(x, MatAt, [&](int r, float2 v) { __stcs(q + g.xoff[r], v); });
         }
-        if constexpr (kPrefetch) {
-#pragma unroll
-            for (int j = 0; j < D; ++j) x[j] = xn[j];
-        } else if (wn < g.n_wtiles) {
+        if (wn < g.n_wtiles) {
             const float2 *pn = tile_ptr(wn);
 #pragma unroll
             for (int j = 0; j < D; ++j) x[j] = __ldcs(pn + g.xoff[j]);
@@ -490,13 +460,258 @@ int launch_reg(float2 *psi, int nbits, const int *tpos, const MatP<K> &M, cudaSt
     std::sort(g.fix, g.fix + g.nfix);
     for (int x = 0; x < (1 << K); x++) {
         uint64_t o = 0;
+        uint32_t sx = 0;
         for (int b = 0; b < g.J; b++)
-            if ((x >> b) & 1) o += 1ull << extra[b];
+            if ((x >> b) & 1) o += 1ull << extra[b], sx |= 1u << g.lt[b];
         for (int i = 0; i < nh; i++)
             if ((x >> (g.J + i)) & 1) o += 1ull << high[i];
         g.xoff[x] = o;
+        g.cw[x] = 8 * sx | 256 * (uint32_t)x;
+        g.cr[x] = 8 * sx | 256 * (uint32_t)(x >> g.J << g.J);
     }
     return g.J ? launch_reg_kernel<K, true>(g, M, st) : launch_reg_kernel<K, false>(g, M, st);
+}
+
+// ---------------------------------------------------------------------------------------
+// Register-tiled apply for k = 5 and 6 (n >= k + 6), on CUDA cores.
+//
+// At these widths the FMAs bind (4 2^k an amplitude: k = 5 takes 0.93 ms per 2^28 amplitudes at 128
+// FMAs a clock and SM, against 0.64 ms of HBM traffic), so what matters is what else is issued
+// beside them.  One group a thread needs the whole matrix per group: as constants 8 KiB miss the
+// constant cache (63 FMAs a clock and SM), and 2^k members plus results leave 8 warps an SM.  Here a
+// CTA keeps a tile of 64 groups in shared memory and thread (row group, group pair) sums a register
+// tile of RT rows x 2 groups: per column one 16-byte load of its groups' members and RT/2 broadcast
+// loads of the matrix feed 8 RT FMAs.  The tile lies in address order, 16-byte units XOR-swizzled
+// (address bits 1-3 taken by targets are fed from the group bits of the lanes), so every target set
+// is loaded and stored without bank conflicts; with bit 0 a target, a unit is two members of a
+// group instead of one member of two groups (LOW0).  The next tile is fetched with cp.async during
+// the sums (two buffers), and 2-5 CTAs an SM cover the exchange of the results through the tile.
+// Sums run over the columns in ascending order, as everywhere here: bit-identical results.
+// Measured on 2^28 amplitudes: k = 5 1.88-2.54 ms (register kernel, by targets) -> 1.43 ms for all
+// (48 TFLOP/s), k = 6 2.78-7.63 ms (2.78 only with every target above bit 5) -> 2.65 ms.  Tried:
+// 4 x 8 and 8 x 4 tiles on 128 or 256 groups 1.45-1.75 ms; one buffer 1.77; packed FMAs
+// (fma.rn.f32x2), which do not raise the FMA rate but need operand pairs, 1.73.
+// ---------------------------------------------------------------------------------------
+constexpr int kRtF = 6;  // log2 groups a tile
+
+struct RtGeom {
+    float2 *psi;
+    uint64_t n_tiles;
+    int tpos[kMaxK];
+    uint64_t off[16];   // global offset of local bit b (b < kRtF + k)
+    uint32_t sw[16];    // staging byte address (swizzled) of local bit b
+    uint32_t mem[64];   // staging byte address of member c
+    uint32_t grp[kRtF]; // staging byte address of group bit i
+};
+
+constexpr int rtile_rows(int k) { return k == 5 ? 8 : 16; }
+constexpr int rtile_threads(int k) { return 32 * ((1 << k) / rtile_rows(k)); }
+constexpr int rtile_min_blocks(int k) { return k == 5 ? 4 : 2; }
+constexpr size_t rtile_smem(int k) { return ((size_t)16 << (kRtF + k)) + ((size_t)8 << (2 * k)); }
+
+template <int K, bool LOW0, typename MatSrc>
+__global__ void __launch_bounds__(rtile_threads(K), rtile_min_blocks(K))
+    k_apply_rtile(const __grid_constant__ RtGeom g, const __grid_constant__ MatSrc mat)
+{
+    constexpr int D = 1 << K, RT = rtile_rows(K), NT = rtile_threads(K), T = D << kRtF;
+    constexpr int NI = T / 2 / NT;  // 16-byte units a thread moves
+    constexpr int LT = __builtin_ctz(NT);
+    extern __shared__ __align__(128) uint8_t sm[];
+    float2 *M = reinterpret_cast<float2 *>(sm + 2 * T * 8);  // [row group][column][row]
+    __shared__ uint64_t ioff[NI];
+    __shared__ uint32_t isw[NI];
+    const int tid = threadIdx.x, lane = tid & 31, rg = tid >> 5;
+    pdl_launch_next();
+    {
+        const float2 *src;
+        if constexpr (K == 6) {
+            src = mat.p;
+        } else {
+            src = mat.m;
+            asm volatile("" : "+l"(src));  // ordinary loads, not constants (32 addresses a warp)
+        }
+        for (int i = tid; i < D * D; i += NT) {
+            const int r = i / D, c = i % D;
+            M[((r / RT) * D + c) * RT + r % RT] = src[i];
+        }
+    }
+    // unit tid + i NT of a tile: local bits 1 .. LT from tid, the others from i
+    if (tid < NI) {
+        uint64_t o = 0;
+        uint32_t s = 0;
+        for (int b = 0; 1 + LT + b < kRtF + K; ++b)
+            if ((tid >> b) & 1) {
+                o += g.off[1 + LT + b];
+                s ^= g.sw[1 + LT + b];
+            }
+        ioff[tid] = o;
+        isw[tid] = s;
+    }
+    uint64_t toff = 0;
+    uint32_t tsw = 0;
+#pragma unroll
+    for (int b = 0; b < LT; ++b)
+        if ((tid >> b) & 1) {
+            toff += g.off[1 + b];
+            tsw ^= g.sw[1 + b];
+        }
+    // this thread's two groups: LOW0: group bits 0-4 = lane, bit 5 = which of the two; else bit 0 =
+    // which (one unit holds both), bits 1-5 = lane
+    uint32_t base[2] = {0, 0};
+#pragma unroll
+    for (int b = 0; b < 5; ++b)
+        if ((lane >> b) & 1) base[0] ^= g.grp[(LOW0 ? 0 : 1) + b];
+    if constexpr (LOW0) base[1] = base[0] ^ g.grp[5];
+    const uint32_t s0 = (uint32_t)__cvta_generic_to_shared(sm);
+    auto fetch = [&](uint64_t t, int buf) {
+        const float2 *tp = g.psi + insert_zero_bits(t << kRtF, g.tpos, K) + toff;
+#pragma unroll
+        for (int i = 0; i < NI; ++i)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(s0 + buf * T * 8 + (tsw ^ isw[i])),
+                         "l"(tp + ioff[i])
+                         : "memory");
+    };
+    __syncthreads();
+    pdl_wait();
+    if (blockIdx.x < g.n_tiles) fetch(blockIdx.x, 0);
+    int buf = 0;
+    for (uint64_t t = blockIdx.x; t < g.n_tiles; t += gridDim.x, buf ^= 1) {
+        cp_async_wait_all();
+        __syncthreads();  // the tile is here; the other buffer's results have been read out
+        if (t + gridDim.x < g.n_tiles) fetch(t + gridDim.x, buf ^ 1);
+        uint8_t *sb = sm + buf * T * 8;
+        float2 y[RT][2];
+#pragma unroll
+        for (int r = 0; r < RT; ++r) y[r][0] = y[r][1] = make_float2(0.f, 0.f);
+        const float4 *mr = reinterpret_cast<const float4 *>(M + rg * RT * D);
+#pragma unroll 2
+        for (int c = 0; c < D; c += 2) {
+            const uint32_t m0 = g.mem[c], m1 = g.mem[c + 1];
+            const float4 u = *reinterpret_cast<const float4 *>(sb + (base[0] ^ m0));
+            const float4 v = *reinterpret_cast<const float4 *>(sb + (LOW0 ? base[1] ^ m0 : base[0] ^ m1));
+            // x[column][group]
+            const float2 x[2][2] = {{make_float2(u.x, u.y), LOW0 ? make_float2(v.x, v.y) : make_float2(u.z, u.w)},
+                                    {LOW0 ? make_float2(u.z, u.w) : make_float2(v.x, v.y), make_float2(v.z, v.w)}};
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                float2 m[RT];
+#pragma unroll
+                for (int r = 0; r < RT; r += 2) {
+                    const float4 w = mr[((c + e) * RT + r) / 2];
+                    m[r] = make_float2(w.x, w.y);
+                    m[r + 1] = make_float2(w.z, w.w);
+                }
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+#pragma unroll
+                    for (int r = 0; r < RT; ++r) {
+                        y[r][j].x = fmaf(m[r].x, x[e][j].x, y[r][j].x);
+                        y[r][j].y = fmaf(m[r].x, x[e][j].y, y[r][j].y);
+                    }
+#pragma unroll
+                    for (int r = 0; r < RT; ++r) {
+                        y[r][j].x = fmaf(m[r].y, -x[e][j].y, y[r][j].x);
+                        y[r][j].y = fmaf(m[r].y, x[e][j].x, y[r][j].y);
+                    }
+                }
+            }
+        }
+        __syncthreads();  // every member has been read
+#pragma unroll
+        for (int r = 0; r < RT; r += 2) {
+            const uint32_t m0 = g.mem[rg * RT + r], m1 = g.mem[rg * RT + r + 1];
+            if constexpr (LOW0) {
+#pragma unroll
+                for (int j = 0; j < 2; ++j)
+                    *reinterpret_cast<float4 *>(sb + (base[j] ^ m0)) =
+                        make_float4(y[r][j].x, y[r][j].y, y[r + 1][j].x, y[r + 1][j].y);
+            } else {
+                *reinterpret_cast<float4 *>(sb + (base[0] ^ m0)) =
+                    make_float4(y[r][0].x, y[r][0].y, y[r][1].x, y[r][1].y);
+                *reinterpret_cast<float4 *>(sb + (base[0] ^ m1)) =
+                    make_float4(y[r + 1][0].x, y[r + 1][0].y, y[r + 1][1].x, y[r + 1][1].y);
+            }
+        }
+        __syncthreads();
+        float2 *tp = g.psi + insert_zero_bits(t << kRtF, g.tpos, K) + toff;
+#pragma unroll
+        for (int i = 0; i < NI; ++i)
+            __stcs(reinterpret_cast<float4 *>(tp + ioff[i]), *reinterpret_cast<const float4 *>(sb + (tsw ^ isw[i])));
+    }
+}
+
+template <int K, bool LOW0, typename MatSrc>
+int launch_rtile_kernel(const RtGeom &g, const MatSrc &M, cudaStream_t st)
+{
+    auto kern = k_apply_rtile<K, LOW0, MatSrc>;
+    constexpr size_t smem = rtile_smem(K);
+    static std::atomic<uint64_t> smem_done{0};
+    if (smem > 48 * 1024 && !smem_opt_in(kern, (int)smem, smem_done)) return -1;
+    static const LaunchCfg cfg = [&] {
+        LaunchCfg c;
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return c;
+        if (cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return c;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&c.occ, kern, rtile_threads(K), smem) != cudaSuccess ||
+            c.occ < 1)
+            c.occ = 1;
+        c.ok = true;
+        return c;
+    }();
+    if (!cfg.ok) return -1;
+    const uint64_t grid = std::min<uint64_t>(g.n_tiles, (uint64_t)cfg.sms * cfg.occ);
+    return launch_pdl(kern, (unsigned)grid, rtile_threads(K), smem, st, g, M) == cudaSuccess ? 0 : -1;
+}
+
+template <int K, typename MatSrc>
+int launch_rtile(float2 *psi, int nbits, const int *tpos, const MatSrc &M, cudaStream_t st)
+{
+    RtGeom g{};
+    g.psi = psi;
+    g.n_tiles = 1ull << (nbits - K - kRtF);
+    bool is_target[64] = {};
+    for (int q = 0; q < K; q++) {
+        g.tpos[q] = tpos[q];
+        is_target[tpos[q]] = true;
+    }
+    // local bits: the targets and the kRtF lowest other bits, ascending
+    int addr[16], mpos[kMaxK], gpos[kRtF], nl = 0, nm = 0, ng = 0;
+    for (int b = 0; b < nbits && nl < K + kRtF; b++) {
+        if (is_target[b])
+            mpos[nm++] = nl;
+        else if (ng < kRtF)
+            gpos[ng++] = nl;
+        else
+            continue;
+        addr[nl++] = b;
+    }
+    if (nl != K + kRtF) return -1;
+    // the lanes' three lowest group bits must reach address bits 1-3 (the 16-byte units of a 128-byte
+    // line): those that lie higher are XORed into the bits that targets occupy, in order
+    const int l0 = is_target[0] ? 0 : 1;
+    int src[3], ns = 0, dst[3], nd = 0;
+    for (int b = 1; b <= 3; b++)
+        if (is_target[b]) dst[nd++] = b;
+    for (int i = 0; i < 3; i++)
+        if (gpos[l0 + i] > 3) src[ns++] = gpos[l0 + i];
+    if (ns != nd) return -1;
+    auto swz = [&](uint32_t p) {
+        uint32_t x = p;
+        for (int i = 0; i < nd; i++) x ^= ((p >> src[i]) & 1u) << dst[i];
+        return 8 * x;
+    };
+    for (int x = 0; x < nl; x++) {
+        g.off[x] = 1ull << addr[x];
+        g.sw[x] = swz(1u << x);
+    }
+    for (int c = 0; c < (1 << K); c++) {
+        uint32_t p = 0;
+        for (int q = 0; q < K; q++)
+            if ((c >> q) & 1) p |= 1u << mpos[q];
+        g.mem[c] = swz(p);
+    }
+    for (int i = 0; i < kRtF; i++) g.grp[i] = swz(1u << gpos[i]);
+    return is_target[0] ? launch_rtile_kernel<K, true>(g, M, st) : launch_rtile_kernel<K, false>(g, M, st);
 }
 
 template <int K>
@@ -507,10 +722,15 @@ int launch_param(float2 *psi, int nbits, const int *tpos, const float2 *mat, cud
     // Measured on GB300 at n = 30: for k <= 3 with every target >= 5 the one-group-per-thread
     // kernel streams at ~7.0 TB/s, ~10% above the persistent register kernel; everywhere
     // else (k = 4, or any target below bit 5) the register kernel is faster.
-    const bool all_high = tpos[0] >= 5;
-    if (K <= 3 && all_high && nbits - K >= 8) return launch_k<K, MatP<K>>(psi, nbits, tpos, M, st);
-    if (nbits >= K + 5) return launch_reg<K>(psi, nbits, tpos, M, st);
-    return launch_k<K, MatP<K>>(psi, nbits, tpos, M, st);
+    if constexpr (K <= 3) {
+        if (tpos[0] >= 5 && nbits - K >= 8) return launch_direct<K>(psi, nbits, tpos, M, st);
+    }
+    if constexpr (K <= 4) {
+        if (nbits >= K + 5) return launch_reg<K>(psi, nbits, tpos, M, st);
+    } else {
+        if (nbits >= K + kRtF) return launch_rtile<K>(psi, nbits, tpos, M, st);
+    }
+    return launch_tiled<K, MatP<K>>(psi, nbits, tpos, M, st);
 }
 
 }  // namespace
@@ -524,7 +744,9 @@ int launch_apply_fp32(sim_t *, float2 *psi, int nbits, int k, const int *tpos, c
     case 3: return launch_param<3>(psi, nbits, tpos, mat, st);
     case 4: return launch_param<4>(psi, nbits, tpos, mat, st);
     case 5: return launch_param<5>(psi, nbits, tpos, mat, st);
-    case 6: return launch_k<6, MatPtr>(psi, nbits, tpos, MatPtr{mat6_dev}, st);
+    case 6:
+        if (nbits >= 6 + kRtF) return launch_rtile<6>(psi, nbits, tpos, MatPtr{mat6_dev}, st);
+        return launch_tiled<6, MatPtr>(psi, nbits, tpos, MatPtr{mat6_dev}, st);
     default: return -1;
     }
 }
