@@ -11,6 +11,7 @@
 // A CTA loads a tile pair (2^(LB+q) amplitudes each, rows of 2^LB contiguous amplitudes) with
 // 16-byte loads, permutes it in shared memory and writes it back with coalesced 16-byte stores.  Tiles that
 // nothing moves are skipped, so a single high-bit swap touches half of the state.
+#include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -25,9 +26,6 @@
 // much less (persistent CTAs looping over tile pairs were slower still).
 #ifndef SYCSIM_PERM_TILE
 #define SYCSIM_PERM_TILE 10  // minimum tile: 2^SYCSIM_PERM_TILE amplitudes
-#endif
-#ifndef SYCSIM_PERM_BULK
-#define SYCSIM_PERM_BULK 1  // in-place tiles through bulk copies (k_permute_tile_bulk)
 #endif
 #ifndef SYCSIM_PERM_TILE_SAME
 #define SYCSIM_PERM_TILE_SAME 12  // the same when no tile pairs swap (measured best of 10..13)
@@ -137,14 +135,6 @@ __global__ void __launch_bounds__(256) k_permute_pass(PermGeom g)
     }
 }
 
-// The global side done by the bulk-copy engine: one copy per row of 2^LB contiguous amplitudes
-// into shared memory (completion counted in bytes on an mbarrier) -- the tile, and for a tile
-// pair (high-high transpositions) its partner's rows too --, the threads swap the pairs
-// (p, sig(p)) the in-tile involution exchanges in each tile, and one bulk store per row writes
-// the tile back, or, for a pair, each tile to its partner's rows.  sig is XOR-linear in
-// the local index p: sig(p) = sig(p_thread) ^ sig(p_iter), the second from a per-CTA table.
-// The only wait (the copies' mbarrier) is bounded by %globaltimer: on a timeout the CTA records
-// the failure, writes nothing back and waits (again bounded) for its copies before leaving.
 __device__ __forceinline__ uint64_t perm_now_ns()
 {
     uint64_t t;
@@ -152,6 +142,13 @@ __device__ __forceinline__ uint64_t perm_now_ns()
     return t;
 }
 
+// Tiles that only permute in place, with at most 3 row bits (rows of 2 KiB and more): one CTA a tile, one
+// bulk copy a row into shared memory (completion counted in bytes on an mbarrier), the threads swap
+// the pairs (p, sig(p)), one bulk store a row back.  sig is XOR-linear in the local index p: sig(p) =
+// sig(p_thread) ^ sig(p_iter), the second from a per-CTA table.  Measured on 2^28 amplitudes: 606-615 us a
+// pass, against 660-685 on the pipeline of k_permute_tma; with 4 and 5 row bits 727 and 737 against
+// 670-690.  The only wait (the copies' mbarrier) is bounded by %globaltimer: on a timeout the CTA
+// records the failure, writes nothing back and waits (again bounded) for its copies before leaving.
 __global__ void __launch_bounds__(256) k_permute_tile_bulk(PermGeom g, int *err)
 {
     extern __shared__ __align__(128) float2 tile[];
@@ -162,15 +159,6 @@ __global__ void __launch_bounds__(256) k_permute_tile_bulk(PermGeom g, int *err)
     const int nloc = g.LB + g.q, T = 1 << nloc;
     const uint32_t row_bytes = 8u << g.LB;
     const uint64_t base = insert_zero_bits_p((uint64_t)blockIdx.x << g.LB, g.rowpos, g.q);
-    uint64_t baseB = base;
-    for (int i = 0; i < g.nhh; ++i) {
-        const uint64_t ba = (base >> g.hh_a[i]) & 1, bb = (base >> g.hh_b[i]) & 1;
-        if (ba != bb) baseB ^= (1ull << g.hh_a[i]) | (1ull << g.hh_b[i]);
-    }
-    if (baseB < base) return;  // the partner CTA moves this pair
-    const bool same = baseB == base;
-    if (same && g.trivial_in) return;  // nothing in this tile moves
-    const int ntile = same ? 1 : 2;
     const uint32_t sbar = (uint32_t)__cvta_generic_to_shared(&bar);
     const uint32_t stile = (uint32_t)__cvta_generic_to_shared(tile);
     auto sig_of = [&](uint32_t p) {
@@ -184,15 +172,14 @@ __global__ void __launch_bounds__(256) k_permute_tile_bulk(PermGeom g, int *err)
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         pdl_wait();  // this thread issues every access to the state
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(sbar),
-                     "r"((uint32_t)(ntile * T) * 8u)
+                     "r"((uint32_t)T * 8u)
                      : "memory");
-        for (int t = 0; t < ntile; ++t)
-            for (int r = 0; r < (1 << g.q); ++r)
-                asm volatile(
-                    "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-                        stile + (uint32_t)t * T * 8u + r * row_bytes),
-                    "l"(g.psi + (t ? baseB : base) + g.rowoff[r]), "r"(row_bytes), "r"(sbar)
-                    : "memory");
+        for (int r = 0; r < (1 << g.q); ++r)
+            asm volatile(
+                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
+                    stile + r * row_bytes),
+                "l"(g.psi + base + g.rowoff[r]), "r"(row_bytes), "r"(sbar)
+                : "memory");
     }
     for (int it = threadIdx.x; it < (T >> 8); it += blockDim.x) {
         uint32_t p = 0;
@@ -222,26 +209,22 @@ __global__ void __launch_bounds__(256) k_permute_tile_bulk(PermGeom g, int *err)
         for (int j = 0; j < 8; ++j)
             if ((threadIdx.x >> j) & 1) p_t |= 1u << g.tbit[j];
         const uint32_t s_t = sig_of(p_t);
-        for (int t = 0; t < ntile && !g.trivial_in; ++t) {
-            float2 *tt = tile + t * T;
-            for (int it = 0; it < (T >> 8); ++it) {
-                const uint32_t p = p_t | p_it[it], q = s_t ^ sig_it[it];
-                if (p < q) {
-                    const float2 a = tt[p], c = tt[q];
-                    tt[p] = c;
-                    tt[q] = a;
-                }
+        for (int it = 0; it < (T >> 8); ++it) {
+            const uint32_t p = p_t | p_it[it], q = s_t ^ sig_it[it];
+            if (p < q) {
+                const float2 a = tile[p], c = tile[q];
+                tile[p] = c;
+                tile[q] = a;
             }
         }
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // the bulk stores read the tile
         __syncthreads();
-        if (threadIdx.x == 0) {  // a pair's tiles go to each other's rows
-            for (int t = 0; t < ntile; ++t)
-                for (int r = 0; r < (1 << g.q); ++r)
-                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(
-                                     g.psi + ((t == 0) == same ? base : baseB) + g.rowoff[r]),
-                                 "r"(stile + (uint32_t)t * T * 8u + r * row_bytes), "r"(row_bytes)
-                                 : "memory");
+        if (threadIdx.x == 0) {
+            for (int r = 0; r < (1 << g.q); ++r)
+                asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(g.psi + base +
+                                                                                                  g.rowoff[r]),
+                             "r"(stile + r * row_bytes), "r"(row_bytes)
+                             : "memory");
             asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
             asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");  // the tile is read out
         }
@@ -255,6 +238,270 @@ __global__ void __launch_bounds__(256) k_permute_tile_bulk(PermGeom g, int *err)
                 : "=r"(done)
                 : "r"(sbar)
                 : "memory");
+    }
+}
+
+// The same pass as a pipeline fed by tensor-map (TMA) copies.  A tile's local bits lie apart in the
+// address (the low block and up to 5 row bits); a 5-dimensional tensor map whose dimensions begin at
+// those bits moves a tile in at most four copies of 2 KiB and more, where one bulk copy a row of 256
+// bytes ran into the copy engine's operation rate.  A stage is 2^11 amplitudes: a tile pair (high-high
+// transpositions) or, without any, one tile of twice the size.
+//  * warp 0, producer: its lanes look at up to 32 tiles at a time (the partner's base, whether anything
+//    moves); lane 0 loads the tiles that do into the stage ring (bytes counted on an mbarrier);
+//  * warps 2-17, swappers, four groups of 128 threads, a stage to each in turn: 16 amplitudes a
+//    thread, read where the in-tile involution sig puts them from, a barrier among the group, written
+//    to their places.  The maps are XOR-linear: a thread part computed once, an iteration part from
+//    the parameters;
+//  * warp 1, storer: lane 0 stores the stage (a pair's tiles crosswise) and releases it once read.
+// The copies lay a tile out with the 128-byte swizzle (16-byte unit bits ^= local bits 4-6), so lanes
+// on two of bits 0-3 and two of the row bits find 16 bank pairs on both sides (choose_lane_bits).
+// What bounds it: HBM, 16 bytes an amplitude that moves.  Measured on 2^28 amplitudes, us a pass
+// (641 for a whole pass): every low bit with a high one and 9 high pairs 1286 -> 694, 5 low-high pairs
+// 737 -> 673, 3 high pairs 587 -> 584; random permutations (two passes) of 2^29 3.2-4.5 -> 2.75-3.03 ms,
+// of 2^24 127-136 -> 93-110 us.  The kernel before, one CTA a tile pair and 4 amplitudes a thread, was
+// issue-bound (76 %) on setting up its maps.
+// Every wait is bounded by %globaltimer: on a timeout the kernel records the failure, every role
+// leaves, and the CTA waits (again bounded) for its own copies.
+constexpr int kPtRing = 98304;                    // bytes of stages (64 KiB: 10-20 % slower); a stage is one tile or a tile pair
+constexpr int kPtMaxStages = 16;
+constexpr int kPtGroups = 2;                      // swapper groups, a stage to each in turn
+constexpr int kPtSwap = 128;                      // threads a group
+constexpr int kPtThreads = 64 + kPtGroups * kPtSwap;
+constexpr unsigned long long kPtWaitNs = 4000000000ull;
+
+struct PermTma {
+    CUtensorMap map;
+    int LB, q;
+    int rowpos[kMaxRow];
+    int nhh, hh_a[20], hh_b[20];
+    int trivial_in;
+    uint64_t n_tiles;             // candidates: every value of the non-tile bits
+    int per;                      // candidates the producer looks at together (<= 32)
+    int nloc;                     // local bits of a tile (a pair has one more: which tile)
+    int stages;                   // a multiple of kPtGroups: a stage belongs to one group, which sees every
+                                  // phase of its barriers in turn (a wait for a parity would otherwise be
+                                  // satisfied by the phase before the one before)
+    uint32_t stage_bytes;
+    int start[5];                 // first address bit of each tensor-map dimension
+    uint32_t size_mask[5];
+    int nops;                     // copies a tile
+    uint32_t op_bytes;
+    uint64_t op_off[4];           // address offset of copy i of a tile
+    uint32_t tp[7], tq[7];        // stage byte of thread-index bit j, and of its image under sig
+    uint32_t ip[16], iq[16];      // the same of iteration i
+};
+
+__device__ __forceinline__ bool perm_try(uint32_t bar, uint32_t parity, uint32_t hint_ns)
+{
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(done)
+        : "r"(bar), "r"(parity), "r"(hint_ns)
+        : "memory");
+    return done != 0;
+}
+
+__device__ __forceinline__ bool perm_wait(uint32_t bar, uint32_t parity, volatile int *abort_flag)
+{
+    if (perm_try(bar, parity, 0)) return true;
+    const uint64_t t0 = perm_now_ns();
+    for (;;) {
+        if (perm_try(bar, parity, 20000)) return true;
+        if (*abort_flag || perm_now_ns() - t0 > kPtWaitNs) return false;
+    }
+}
+
+__device__ __forceinline__ bool perm_bar_and(int id, int n, bool p)
+{
+    uint32_t r;
+    asm volatile(
+        "{\n\t.reg .pred pi, po;\n\tsetp.ne.u32 pi, %1, 0;\n\tbar.red.and.pred po, %2, %3, pi;\n\t"
+        "selp.u32 %0, 1, 0, po;\n\t}\n"
+        : "=r"(r)
+        : "r"((uint32_t)p), "r"(id), "r"(n)
+        : "memory");
+    return r != 0;
+}
+
+__device__ __forceinline__ uint32_t perm_smem(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__global__ void __launch_bounds__(kPtThreads, 2) k_permute_tma(const __grid_constant__ PermTma g, int *err)
+{
+    extern __shared__ uint8_t sm_raw[];
+    uint8_t *const sm = sm_raw + ((1024 - (perm_smem(sm_raw) & 1023)) & 1023);  // the swizzle's period
+    __shared__ __align__(8) uint64_t full[kPtMaxStages], swapped[kPtMaxStages], empty[kPtMaxStages];
+    __shared__ uint64_t dst_a[kPtMaxStages], dst_b[kPtMaxStages];  // where a stage's first and second tile go
+    __shared__ int abort_flag, ntile_of[kPtMaxStages];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const uint32_t S = (uint32_t)g.stages;
+    pdl_launch_next();
+    if (tid == 0) {
+        for (uint32_t i = 0; i < S; ++i) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(perm_smem(&full[i])) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(perm_smem(&swapped[i])), "r"(kPtSwap / 32) : "memory");
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(perm_smem(&empty[i])) : "memory");
+        }
+        abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    }
+    __syncthreads();
+    volatile int *ab = &abort_flag;
+    auto give_up = [&]() {
+        *ab = 1;
+        if (err) atomicExch(err, 1);
+    };
+    const uint32_t stage0 = perm_smem(sm);
+    // one tile between the stage (at byte `at`) and the state (from address offset `base`)
+    auto copy_tile = [&](bool load, uint32_t at, uint64_t base, uint32_t bar) {
+        for (int i = 0; i < g.nops; ++i) {
+            const uint64_t a = base + g.op_off[i];
+            const int c0 = (int)(a & g.size_mask[0]), c1 = (int)((a >> g.start[1]) & g.size_mask[1]),
+                      c2 = (int)((a >> g.start[2]) & g.size_mask[2]), c3 = (int)((a >> g.start[3]) & g.size_mask[3]),
+                      c4 = (int)((a >> g.start[4]) & g.size_mask[4]);
+            const uint32_t s = at + i * g.op_bytes;
+            if (load)
+                asm volatile(
+                    "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+                    "%5, %6}], [%7];\n" ::"r"(s),
+                    "l"(&g.map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(bar)
+                    : "memory");
+            else
+                asm volatile("cp.async.bulk.tensor.5d.global.shared::cta.bulk_group [%0, {%1, %2, %3, %4, %5}], [%6];\n" ::"l"(
+                                 &g.map),
+                             "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(s)
+                             : "memory");
+        }
+    };
+    const uint32_t tile_bytes = 8u << g.nloc;
+
+    if (warp == 0) {
+        // ---------------- producer ----------------
+        pdl_wait();
+        uint32_t it = 0;
+        bool stop = false;
+        for (uint64_t c0 = (uint64_t)blockIdx.x * g.per; c0 < g.n_tiles && !stop; c0 += (uint64_t)gridDim.x * g.per) {
+            const uint64_t t = c0 + lane;
+            uint64_t a = 0, b = 0;
+            bool moves = false;
+            if (lane < g.per && t < g.n_tiles) {
+                a = insert_zero_bits_p(t << g.LB, g.rowpos, g.q);
+                b = a;
+                for (int i = 0; i < g.nhh; ++i) {
+                    const uint64_t x = ((a >> g.hh_a[i]) ^ (a >> g.hh_b[i])) & 1;
+                    b ^= (x << g.hh_a[i]) | (x << g.hh_b[i]);
+                }
+                moves = b > a || (b == a && !g.trivial_in);  // b < a: the partner's turn moves the pair
+            }
+            for (uint32_t m = __ballot_sync(0xffffffffu, moves); m; m &= m - 1) {
+                const int src = __ffs(m) - 1;
+                const uint64_t ta = __shfl_sync(0xffffffffu, a, src), tb = __shfl_sync(0xffffffffu, b, src);
+                const uint32_t st = it % S;
+                bool ok = true;
+                if (lane == 0 && it >= S) ok = perm_wait(perm_smem(&empty[st]), (it / S - 1) & 1, ab);
+                if (!__shfl_sync(0xffffffffu, ok, 0)) {
+                    if (lane == 0) give_up();
+                    stop = true;
+                    break;
+                }
+                if (lane == 0) {
+                    const int nt = ta == tb ? 1 : 2;
+                    dst_a[st] = tb;  // a pair's tiles go to each other's places
+                    dst_b[st] = ta;
+                    ntile_of[st] = nt;
+                    const uint32_t bar = perm_smem(&full[st]);
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(nt * tile_bytes)
+                                 : "memory");
+                    copy_tile(true, stage0 + st * g.stage_bytes, ta, bar);
+                    if (nt == 2) copy_tile(true, stage0 + st * g.stage_bytes + tile_bytes, tb, bar);
+                }
+                ++it;
+            }
+        }
+        if (lane == 0) {
+            // the end: items of no tiles, one for each swapper group, in order behind the loaded ones
+            uint32_t marks = 0;
+            for (; !stop && marks < (uint32_t)kPtGroups; ++marks) {
+                const uint32_t e = it + marks;
+                if (e >= S && !perm_wait(perm_smem(&empty[e % S]), (e / S - 1) & 1, ab)) break;
+                ntile_of[e % S] = 0;
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(perm_smem(&full[e % S])) : "memory");
+            }
+            if (marks < (uint32_t)kPtGroups) {
+                // given up: no copy may still be writing a stage when the CTA leaves.  (Otherwise the
+                // storer has waited for every one of them, and the end marks have moved barriers on.)
+                give_up();
+                for (uint32_t j = it + marks > S ? it + marks - S : 0; j < it; ++j) {
+                    const uint64_t t0 = perm_now_ns();
+                    while (!perm_try(perm_smem(&full[j % S]), (j / S) & 1, 20000) &&
+                           perm_now_ns() - t0 <= kPtWaitNs) {
+                    }
+                }
+            }
+        }
+    } else if (warp == 1) {
+        // ---------------- storer ----------------
+        if (lane == 0) {
+            uint32_t it = 0;
+            for (;; ++it) {
+                const uint32_t st = it % S;
+                if (!perm_wait(perm_smem(&full[st]), (it / S) & 1, ab)) {
+                    give_up();
+                    break;
+                }
+                const int nt = ntile_of[st];
+                if (nt == 0) break;
+                if (!g.trivial_in && !perm_wait(perm_smem(&swapped[st]), (it / S) & 1, ab)) {
+                    give_up();
+                    break;
+                }
+                copy_tile(false, stage0 + st * g.stage_bytes, dst_a[st], 0);
+                if (nt == 2) copy_tile(false, stage0 + st * g.stage_bytes + tile_bytes, dst_b[st], 0);
+                asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+                if (it > 0) {  // the stage before this one has been read out
+                    asm volatile("cp.async.bulk.wait_group.read 1;\n" ::: "memory");
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(perm_smem(&empty[(it - 1) % S]))
+                                 : "memory");
+                }
+            }
+            asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
+            if (it > 0)  // the producer's end mark may wait for this stage
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(perm_smem(&empty[(it - 1) % S])) : "memory");
+        }
+    } else if (!g.trivial_in) {
+        // ---------------- swappers ----------------
+        const int w = (tid - 64) & (kPtSwap - 1), grp = (tid - 64) / kPtSwap;
+        uint32_t pt = 0, qt = 0;
+#pragma unroll
+        for (int j = 0; j < 7; ++j)
+            if ((w >> j) & 1) {
+                pt ^= g.tp[j];
+                qt ^= g.tq[j];
+            }
+        // a group takes the items congruent to its number, the last of them an end mark
+        for (uint32_t it = grp;; it += kPtGroups) {
+            const uint32_t st = it % S;
+            const bool ok = perm_wait(perm_smem(&full[st]), (it / S) & 1, ab);
+            if (!perm_bar_and(1 + grp, kPtSwap, ok)) {  // all leave together: the barrier below counts them
+                give_up();
+                break;
+            }
+            const int nt = ntile_of[st];
+            if (nt == 0) break;
+            uint8_t *sb = sm + st * g.stage_bytes;
+            const int n = (nt << g.nloc) / kPtSwap;
+            float2 v[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                if (i < n) v[i] = *reinterpret_cast<const float2 *>(sb + (qt ^ g.iq[i]));
+            asm volatile("bar.sync %0, 128;\n" ::"r"(1 + grp) : "memory");
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                if (i < n) *reinterpret_cast<float2 *>(sb + (pt ^ g.ip[i])) = v[i];
+            asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // the store reads the stage
+            __syncwarp();
+            if ((tid & 31) == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(perm_smem(&swapped[st])) : "memory");
+        }
     }
 }
 
@@ -332,6 +579,214 @@ int build_geom(float2 *psi, int nbits, const int *inv, int min_tile, PermGeom &g
     return 0;
 }
 
+// ---- the tensor-map pass: geometry, tensor map, launch ----
+
+using EncodeTiled = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
+                                 const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
+                                 CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+
+EncodeTiled encode_tiled()
+{
+    static const EncodeTiled fn = [] {  // the driver's entry: the library itself links only the runtime
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult st;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &st) != cudaSuccess ||
+            st != cudaDriverEntryPointSuccess)
+            p = nullptr;
+        return reinterpret_cast<EncodeTiled>(p);
+    }();
+    return fn;
+}
+
+// Bank pair (0-15, a vector of 4 bits) of local bit x in the swizzled stage: bit 0 as it is, bits 1-3
+// the 16-byte unit, which local bits 4-6 are XORed into.
+uint32_t bank_of(int x) { return x < 4 ? 1u << x : (x < 7 ? 1u << (x - 3) : 0u); }
+uint32_t stage_byte(uint32_t p) { return 8 * p ^ (((p >> 4) & 7u) << 4); }
+
+// Thread-index and iteration bits of the swappers over nl local bits with in-tile involution sig: the
+// four bits of a half-warp's lanes are taken so that the ranks of their bank pairs, at p and at
+// sig(p), are as large as can be (4 and 4: no conflicts), then the remaining bits ascending.
+void swap_bits(PermTma &g, const int *sig, int nl)
+{
+    // the span of a set of bank vectors as a mask of 16 bits (bit v: v is in it)
+    auto grown = [](uint32_t span, uint32_t v) {
+        uint32_t x = span;
+        if (v & 1) x = ((x & 0x5555u) << 1) | ((x >> 1) & 0x5555u);
+        if (v & 2) x = ((x & 0x3333u) << 2) | ((x >> 2) & 0x3333u);
+        if (v & 4) x = ((x & 0x0f0fu) << 4) | ((x >> 4) & 0x0f0fu);
+        if (v & 8) x = ((x & 0x00ffu) << 8) | ((x >> 8) & 0x00ffu);
+        return span | x;
+    };
+    const int nsel = std::min(nl, 11);
+    int order[16], no = 4, pick[4], best = -1;
+    // depth first, both ranks growing at every step; the best partial choice is completed greedily
+    auto search = [&](auto &&self, int depth, uint32_t sp, uint32_t sq, int from) -> bool {
+        if (depth > best) {
+            best = depth;
+            uint32_t p = sp, q = sq;
+            std::copy(pick, pick + depth, order);
+            for (int d = depth; d < 4; d++) {
+                int bx = -1, bg = -1;
+                for (int x = 0; x < nsel; x++) {
+                    if (std::find(order, order + d, x) != order + d) continue;
+                    const int gn = !((p >> bank_of(x)) & 1) + !((q >> bank_of(sig[x])) & 1);
+                    if (gn > bg) bg = gn, bx = x;
+                }
+                order[d] = bx;
+                p = grown(p, bank_of(bx));
+                q = grown(q, bank_of(sig[bx]));
+            }
+        }
+        if (depth == 4) return true;
+        for (int x = from; x < nsel; x++) {
+            const uint32_t vp = bank_of(x), vq = bank_of(sig[x]);
+            if (((sp >> vp) & 1) || ((sq >> vq) & 1)) continue;
+            pick[depth] = x;
+            if (self(self, depth + 1, grown(sp, vp), grown(sq, vq), x + 1)) return true;
+        }
+        return false;
+    };
+    search(search, 0, 1u, 1u, 0);
+    bool used[16] = {};
+    for (int j = 0; j < 4; j++) used[order[j]] = true;
+    for (int x = 0; x < nl; x++)
+        if (!used[x]) order[no++] = x;  // a pair's tile bit, the highest, comes last
+    for (int j = 0; j < 7; j++) {
+        g.tp[j] = stage_byte(1u << order[j]);
+        g.tq[j] = stage_byte(1u << sig[order[j]]);
+    }
+    for (int i = 0; i < 16; i++) {
+        g.ip[i] = g.iq[i] = 0;
+        for (int b = 0; 7 + b < nl; b++)
+            if ((i >> b) & 1) {
+                g.ip[i] ^= stage_byte(1u << order[7 + b]);
+                g.iq[i] ^= stage_byte(1u << sig[order[7 + b]]);
+            }
+    }
+}
+
+// Everything but the encoded map; false if the involution has no such geometry.
+bool permute_tma_geom(int nbits, const int *inv, PermTma &g, cuuint32_t *box, cuuint64_t *dim, cuuint64_t *stride)
+{
+    if (nbits < 11 || nbits > 35) return false;
+    // the widest low block whose tile (2^11 amplitudes; 2^10 where tiles swap in pairs) fits a stage
+    for (int LB = 5; LB <= 11; LB++) {
+        int row[kMaxRow], q = 0, pairs = 0;
+        for (int b = 0; b < LB && q <= 5; b++)
+            if (inv[b] >= LB) row[q < kMaxRow ? q : 0] = inv[b], q++;
+        if (q > 5) continue;
+        std::sort(row, row + q);
+        int hh_a[20], hh_b[20];
+        for (int b = LB; b < nbits; b++)
+            if (inv[b] > b) {
+                bool is_row = false;
+                for (int i = 0; i < q; i++) is_row |= row[i] == b || row[i] == inv[b];
+                if (is_row) continue;
+                if (pairs == 20) return false;
+                hh_a[pairs] = b;
+                hh_b[pairs++] = inv[b];
+            }
+        if (LB + q > (pairs ? 10 : 11)) continue;
+        g.LB = LB;
+        g.q = q;
+        g.nhh = pairs;
+        std::copy(row, row + q, g.rowpos);
+        std::copy(hh_a, hh_a + pairs, g.hh_a);
+        std::copy(hh_b, hh_b + pairs, g.hh_b);
+    }
+    if (g.LB == 0) return false;
+    const int LB = g.LB, q = g.q;
+    g.nloc = LB + q;
+    if (g.nloc < 9) return false;
+    g.stage_bytes = 8u << (g.nloc + (g.nhh ? 1 : 0));
+    g.stages = std::min<int>(kPtMaxStages, kPtRing / g.stage_bytes) / kPtGroups * kPtGroups;
+    g.n_tiles = 1ull << (nbits - g.nloc);
+    // the involution on local bits: low bits, row bits, and (a pair) which tile
+    int sig[16];
+    g.trivial_in = 1;
+    for (int x = 0; x < 16; x++) sig[x] = x;
+    for (int b = 0; b < LB; b++) {
+        if (inv[b] == b) continue;
+        g.trivial_in = 0;
+        if (inv[b] < LB) {
+            sig[b] = inv[b];
+        } else {
+            int i = 0;
+            while (g.rowpos[i] != inv[b]) i++;
+            sig[b] = LB + i;
+            sig[LB + i] = b;
+        }
+    }
+    swap_bits(g, sig, g.nloc + (g.nhh ? 1 : 0));
+    // tensor-map dimensions: bits 0-3 (128 bytes, the swizzle's rows), then one from each tile bit that
+    // does not continue the dimension before it; tile bits beyond the fifth dimension are looped over
+    int tile_bit[16], nt = 0;
+    for (int b = 4; b < LB; b++) tile_bit[nt++] = b;
+    for (int i = 0; i < q; i++) tile_bit[nt++] = g.rowpos[i];
+    for (int d = 0; d < 5; d++) box[d] = d ? 1 : 16;
+    int nd = 1, i = 0;
+    for (; i < nt; i++) {
+        if (nd > 1 && tile_bit[i] == tile_bit[i - 1] + 1) {
+            box[nd - 1] *= 2;
+            continue;
+        }
+        if (nd == 5) break;
+        g.start[nd] = tile_bit[i];
+        box[nd++] = 2;
+    }
+    const int looped = nt - i;
+    if (looped > 2) return false;
+    g.nops = 1 << looped;
+    g.op_bytes = (8u << g.nloc) >> looped;
+    for (int o = 0; o < g.nops; o++)
+        for (int b = 0; b < looped; b++)
+            if ((o >> b) & 1) g.op_off[o] += 1ull << tile_bit[i + b];
+    for (int d = 0; d < 5; d++) {
+        const int lo = d < nd ? g.start[d] : nbits, hi = d + 1 < nd ? g.start[d + 1] : nbits;
+        if (hi - lo > 31) return false;
+        dim[d] = 1ull << (hi - lo);
+        g.start[d] = d < nd ? lo : 0;
+        g.size_mask[d] = d < nd ? (uint32_t)(dim[d] - 1) : 0;
+        if (d > 0) stride[d - 1] = 8ull << lo;
+    }
+    return true;
+}
+
+// The pass as tensor-map copies: 0 launched, 1 not a geometry for it, < 0 an error.
+int launch_permute_tma(float2 *psi, int nbits, const int *inv, cudaStream_t st, int *err)
+{
+    PermTma g{};
+    cuuint32_t box[5];
+    const cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+    cuuint64_t dim[5], stride[4];
+    if (((uintptr_t)psi & 15) != 0 || !encode_tiled() || !permute_tma_geom(nbits, inv, g, box, dim, stride)) return 1;
+    if (encode_tiled()(&g.map, CU_TENSOR_MAP_DATA_TYPE_INT64, 5, psi, dim, stride, box, estr,
+                       CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return 1;
+    constexpr int smem = kPtRing + 1024;
+    static std::atomic<uint64_t> smem_done{0};
+    if (!smem_opt_in(k_permute_tma, smem, smem_done)) return -1;
+    static const LaunchCfg cfg = [] {
+        LaunchCfg c;
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return c;
+        if (cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return c;
+        c.ok = true;
+        return c;
+    }();
+    if (!cfg.ok) return -1;
+    const uint64_t ctas = 2 * (uint64_t)cfg.sms;
+    // candidates a producer takes at a time: many, since evaluating them costs its warp the same for 1
+    // and for 32, but at least 16 turns a CTA, so that the last one is not half empty (2^24 amplitudes:
+    // 127-141 us two random passes with 32 at a time, 94-110 with 4)
+    g.per = 32;
+    while (g.per > 1 && g.n_tiles / g.per < 16 * ctas) g.per >>= 1;
+    if (g.nhh == 0) g.per = std::min(g.per, 4);  // no pairs: little to evaluate, neighbours together
+    const uint64_t grid = std::min<uint64_t>(ctas, (g.n_tiles + g.per - 1) / g.per);
+    return launch_pdl(k_permute_tma, (unsigned)grid, kPtThreads, smem, st, g, err) == cudaSuccess ? 0 : -1;
+}
+
 // Bits of the local index the 32 lanes of a warp run over in k_permute_tile_bulk: a warp reads
 // and writes both p and sig(p); with 8-byte elements the bank pair is bits 0-3 of the index, so a
 // set of lane bits costs max(2, 32 >> |bits in 0-3|) wavefronts for p, the same for sig(p).  The
@@ -377,26 +832,23 @@ int launch_involution(float2 *psi, int nbits, const int *inv, cudaStream_t st, i
     bool any = false;
     for (int b = 0; b < nbits; b++) any |= inv[b] != b;
     if (!any) return 0;
+    // in-place tiles (no tile pairs) of at most 3 row bits, rows of >= 2^5 amplitudes: bulk copies
     PermGeom g;
-    const int rc = build_geom(psi, nbits, inv, SYCSIM_PERM_TILE, g);
-    if (rc != 0) return rc;
-    // tiles that only permute in place (no tile pairs) gain from more work per CTA
-    if (g.nhh == 0 && SYCSIM_PERM_TILE_SAME > SYCSIM_PERM_TILE) {
-        PermGeom big;
-        if (build_geom(psi, nbits, inv, SYCSIM_PERM_TILE_SAME, big) == 0) g = big;
+    int rc = build_geom(psi, nbits, inv, SYCSIM_PERM_TILE_SAME, g);
+    if (rc == 0 && g.nhh == 0 && g.q <= 3 && g.LB >= 5 && g.LB + g.q >= 8 && g.LB + g.q <= 12 && ((uintptr_t)psi & 15) == 0) {
+        const uint64_t tiles = 1ull << (nbits - g.LB - g.q);
+        choose_lane_bits(g);
+        return launch_pdl(k_permute_tile_bulk, (unsigned)tiles, 256, sizeof(float2) << (g.LB + g.q), st, g, err) ==
+                       cudaSuccess
+                   ? 0
+                   : -1;
     }
+    const int tma = launch_permute_tma(psi, nbits, inv, st, err);
+    if (tma <= 0) return tma;
+    rc = build_geom(psi, nbits, inv, SYCSIM_PERM_TILE, g);
+    if (rc != 0) return rc;
     const int LB = g.LB, q = g.q;
     const uint64_t tiles = 1ull << (nbits - LB - q);
-    if (SYCSIM_PERM_BULK && LB >= 5 && LB + q >= 8 && LB + q <= 14 && ((uintptr_t)psi & 15) == 0 &&
-        (g.nhh == 0 ? 1 : 2) * (sizeof(float2) << (LB + q)) <= 128 * 1024) {
-        const size_t tsm = (g.nhh == 0 ? 1 : 2) * (sizeof(float2) << (LB + q));
-        if (tsm > 48 * 1024 &&
-            cudaFuncSetAttribute(k_permute_tile_bulk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm) !=
-                cudaSuccess)
-            return -1;
-        choose_lane_bits(g);
-        return launch_pdl(k_permute_tile_bulk, (unsigned)tiles, 256, tsm, st, g, err) == cudaSuccess ? 0 : -1;
-    }
     const size_t smem = (g.nhh ? 2 : 1) * sizeof(float2) << (LB + q);  // a tile pair, or one tile
     if (smem > 48 * 1024 &&
         cudaFuncSetAttribute(k_permute_pass, cudaFuncAttributeMaxDynamicSharedMemorySize,
