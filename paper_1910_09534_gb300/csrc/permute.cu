@@ -142,13 +142,16 @@ __device__ __forceinline__ uint64_t perm_now_ns()
     return t;
 }
 
-// Tiles that only permute in place, with at most 3 row bits (rows of 2 KiB and more): one CTA a tile, one
-// bulk copy a row into shared memory (completion counted in bytes on an mbarrier), the threads swap
-// the pairs (p, sig(p)), one bulk store a row back.  sig is XOR-linear in the local index p: sig(p) =
-// sig(p_thread) ^ sig(p_iter), the second from a per-CTA table.  Measured on 2^28 amplitudes: 606-615 us a
-// pass, against 660-685 on the pipeline of k_permute_tma; with 4 and 5 row bits 727 and 737 against
-// 670-690.  The only wait (the copies' mbarrier) is bounded by %globaltimer: on a timeout the CTA
-// records the failure, writes nothing back and waits (again bounded) for its copies before leaving.
+// Long rows: one CTA a tile (or tile pair), one bulk copy a row of 1 KiB and more into shared memory
+// (completion counted in bytes on an mbarrier), the threads swap the pairs (p, sig(p)) the in-tile
+// involution exchanges, one bulk store a row back, a pair's tiles to each other's rows.  sig is
+// XOR-linear in the local index p: sig(p) = sig(p_thread) ^ sig(p_iter), the second from a per-CTA table.
+// launch_involution takes it where it is the faster one; us a pass, this / k_permute_tma: 2^28
+// amplitudes in place with 0-3 row bits 606-630 / 660-685, with 4, 5 (rows of 256-512 bytes) 727, 737 /
+// 670-690; tile pairs with no row bits, 2^30 1225 / 1322, 2^28 575 / 590; pairs of 2^11 with rows of 1 KiB 687
+// / 740, of 2^10 809 / 690, with shorter rows 973-1286 / 690-711.
+// The only wait (the copies' mbarrier) is bounded by %globaltimer: on a timeout the CTA records the
+// failure, writes nothing back and waits (again bounded) for its copies before leaving.
 __global__ void __launch_bounds__(256) k_permute_tile_bulk(PermGeom g, int *err)
 {
     extern __shared__ __align__(128) float2 tile[];
@@ -159,6 +162,15 @@ __global__ void __launch_bounds__(256) k_permute_tile_bulk(PermGeom g, int *err)
     const int nloc = g.LB + g.q, T = 1 << nloc;
     const uint32_t row_bytes = 8u << g.LB;
     const uint64_t base = insert_zero_bits_p((uint64_t)blockIdx.x << g.LB, g.rowpos, g.q);
+    uint64_t baseB = base;
+    for (int i = 0; i < g.nhh; ++i) {
+        const uint64_t ba = (base >> g.hh_a[i]) & 1, bb = (base >> g.hh_b[i]) & 1;
+        if (ba != bb) baseB ^= (1ull << g.hh_a[i]) | (1ull << g.hh_b[i]);
+    }
+    if (baseB < base) return;  // the partner CTA moves this pair
+    const bool same = baseB == base;
+    if (same && g.trivial_in) return;  // nothing in this tile moves
+    const int ntile = same ? 1 : 2;
     const uint32_t sbar = (uint32_t)__cvta_generic_to_shared(&bar);
     const uint32_t stile = (uint32_t)__cvta_generic_to_shared(tile);
     auto sig_of = [&](uint32_t p) {
@@ -172,14 +184,15 @@ __global__ void __launch_bounds__(256) k_permute_tile_bulk(PermGeom g, int *err)
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         pdl_wait();  // this thread issues every access to the state
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(sbar),
-                     "r"((uint32_t)T * 8u)
+                     "r"((uint32_t)(ntile * T) * 8u)
                      : "memory");
-        for (int r = 0; r < (1 << g.q); ++r)
-            asm volatile(
-                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
-                    stile + r * row_bytes),
-                "l"(g.psi + base + g.rowoff[r]), "r"(row_bytes), "r"(sbar)
-                : "memory");
+        for (int t = 0; t < ntile; ++t)
+            for (int r = 0; r < (1 << g.q); ++r)
+                asm volatile(
+                    "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(
+                        stile + (uint32_t)t * T * 8u + r * row_bytes),
+                    "l"(g.psi + (t ? baseB : base) + g.rowoff[r]), "r"(row_bytes), "r"(sbar)
+                    : "memory");
     }
     for (int it = threadIdx.x; it < (T >> 8); it += blockDim.x) {
         uint32_t p = 0;
@@ -209,22 +222,26 @@ __global__ void __launch_bounds__(256) k_permute_tile_bulk(PermGeom g, int *err)
         for (int j = 0; j < 8; ++j)
             if ((threadIdx.x >> j) & 1) p_t |= 1u << g.tbit[j];
         const uint32_t s_t = sig_of(p_t);
-        for (int it = 0; it < (T >> 8); ++it) {
-            const uint32_t p = p_t | p_it[it], q = s_t ^ sig_it[it];
-            if (p < q) {
-                const float2 a = tile[p], c = tile[q];
-                tile[p] = c;
-                tile[q] = a;
+        for (int t = 0; t < ntile && !g.trivial_in; ++t) {
+            float2 *tt = tile + t * T;
+            for (int it = 0; it < (T >> 8); ++it) {
+                const uint32_t p = p_t | p_it[it], q = s_t ^ sig_it[it];
+                if (p < q) {
+                    const float2 a = tt[p], c = tt[q];
+                    tt[p] = c;
+                    tt[q] = a;
+                }
             }
         }
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // the bulk stores read the tile
         __syncthreads();
-        if (threadIdx.x == 0) {
-            for (int r = 0; r < (1 << g.q); ++r)
-                asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(g.psi + base +
-                                                                                                  g.rowoff[r]),
-                             "r"(stile + r * row_bytes), "r"(row_bytes)
-                             : "memory");
+        if (threadIdx.x == 0) {  // a pair's tiles go to each other's rows
+            for (int t = 0; t < ntile; ++t)
+                for (int r = 0; r < (1 << g.q); ++r)
+                    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(
+                                     g.psi + ((t == 0) == same ? base : baseB) + g.rowoff[r]),
+                                 "r"(stile + (uint32_t)t * T * 8u + r * row_bytes), "r"(row_bytes)
+                                 : "memory");
             asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
             asm volatile("cp.async.bulk.wait_group.read 0;\n" ::: "memory");  // the tile is read out
         }
@@ -247,18 +264,18 @@ __global__ void __launch_bounds__(256) k_permute_tile_bulk(PermGeom g, int *err)
 // bytes ran into the copy engine's operation rate.  A stage is 2^11 amplitudes: a tile pair (high-high
 // transpositions) or, without any, one tile of twice the size.
 //  * warp 0, producer: its lanes look at up to 32 tiles at a time (the partner's base, whether anything
-//    moves); lane 0 loads the tiles that do into the stage ring (bytes counted on an mbarrier);
+//    moves); the tiles that do are loaded into the stage ring, a copy a lane (bytes counted on an mbarrier);
 //  * warps 2-17, swappers, four groups of 128 threads, a stage to each in turn: 16 amplitudes a
 //    thread, read where the in-tile involution sig puts them from, a barrier among the group, written
 //    to their places.  The maps are XOR-linear: a thread part computed once, an iteration part from
 //    the parameters;
-//  * warp 1, storer: lane 0 stores the stage (a pair's tiles crosswise) and releases it once read.
+//  * warp 1, storer: stores the stage (a pair's tiles crosswise) and releases it once read.
 // The copies lay a tile out with the 128-byte swizzle (16-byte unit bits ^= local bits 4-6), so lanes
 // on two of bits 0-3 and two of the row bits find 16 bank pairs on both sides (choose_lane_bits).
 // What bounds it: HBM, 16 bytes an amplitude that moves.  Measured on 2^28 amplitudes, us a pass
 // (641 for a whole pass): every low bit with a high one and 9 high pairs 1286 -> 694, 5 low-high pairs
-// 737 -> 673, 3 high pairs 587 -> 584; random permutations (two passes) of 2^29 3.2-4.5 -> 2.75-3.03 ms,
-// of 2^24 127-136 -> 93-110 us.  The kernel before, one CTA a tile pair and 4 amplitudes a thread, was
+// 737 -> 673, 3 high pairs 587 -> 584; random permutations (two passes) of 2^29 3.2-4.5 -> 2.70-2.93 ms,
+// of 2^24 127-141 -> 85-94 us.  The kernel before, one CTA a tile pair and 4 amplitudes a thread, was
 // issue-bound (76 %) on setting up its maps.
 // Every wait is bounded by %globaltimer: on a timeout the kernel records the failure, every role
 // leaves, and the CTA waits (again bounded) for its own copies.
@@ -352,28 +369,30 @@ __global__ void __launch_bounds__(kPtThreads, 2) k_permute_tma(const __grid_cons
         if (err) atomicExch(err, 1);
     };
     const uint32_t stage0 = perm_smem(sm);
-    // one tile between the stage (at byte `at`) and the state (from address offset `base`)
-    auto copy_tile = [&](bool load, uint32_t at, uint64_t base, uint32_t bar) {
-        for (int i = 0; i < g.nops; ++i) {
-            const uint64_t a = base + g.op_off[i];
-            const int c0 = (int)(a & g.size_mask[0]), c1 = (int)((a >> g.start[1]) & g.size_mask[1]),
-                      c2 = (int)((a >> g.start[2]) & g.size_mask[2]), c3 = (int)((a >> g.start[3]) & g.size_mask[3]),
-                      c4 = (int)((a >> g.start[4]) & g.size_mask[4]);
-            const uint32_t s = at + i * g.op_bytes;
-            if (load)
-                asm volatile(
-                    "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
-                    "%5, %6}], [%7];\n" ::"r"(s),
-                    "l"(&g.map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(bar)
-                    : "memory");
-            else
-                asm volatile("cp.async.bulk.tensor.5d.global.shared::cta.bulk_group [%0, {%1, %2, %3, %4, %5}], [%6];\n" ::"l"(
-                                 &g.map),
-                             "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(s)
-                             : "memory");
-        }
-    };
+    // one copy between a stage and the state, to each lane its own: copy `lane % nops` of tile `lane / nops`
+    // (at address offset ta or tb).  Issued by one thread one after the other, the address arithmetic of up
+    // to 8 copies took longer than the stage's share of HBM time.
+    const int op = lane & (g.nops - 1), op_tile = lane / g.nops;
     const uint32_t tile_bytes = 8u << g.nloc;
+    const uint32_t op_at = op_tile * tile_bytes + op * g.op_bytes;
+    const uint64_t op_off = g.op_off[op];
+    auto copy = [&](bool load, uint32_t at, uint64_t ta, uint64_t tb, uint32_t bar) {
+        const uint64_t a = (op_tile ? tb : ta) + op_off;
+        const int c0 = (int)(a & g.size_mask[0]), c1 = (int)((a >> g.start[1]) & g.size_mask[1]),
+                  c2 = (int)((a >> g.start[2]) & g.size_mask[2]), c3 = (int)((a >> g.start[3]) & g.size_mask[3]),
+                  c4 = (int)((a >> g.start[4]) & g.size_mask[4]);
+        if (load)
+            asm volatile(
+                "cp.async.bulk.tensor.5d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, "
+                "%5, %6}], [%7];\n" ::"r"(at + op_at),
+                "l"(&g.map), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(bar)
+                : "memory");
+        else
+            asm volatile("cp.async.bulk.tensor.5d.global.shared::cta.bulk_group [%0, {%1, %2, %3, %4, %5}], [%6];\n" ::"l"(
+                             &g.map),
+                         "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(c4), "r"(at + op_at)
+                         : "memory");
+    };
 
     if (warp == 0) {
         // ---------------- producer ----------------
@@ -404,17 +423,17 @@ __global__ void __launch_bounds__(kPtThreads, 2) k_permute_tma(const __grid_cons
                     stop = true;
                     break;
                 }
+                const int nt = ta == tb ? 1 : 2;
+                const uint32_t bar = perm_smem(&full[st]);
                 if (lane == 0) {
-                    const int nt = ta == tb ? 1 : 2;
                     dst_a[st] = tb;  // a pair's tiles go to each other's places
                     dst_b[st] = ta;
                     ntile_of[st] = nt;
-                    const uint32_t bar = perm_smem(&full[st]);
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(nt * tile_bytes)
-                                 : "memory");
-                    copy_tile(true, stage0 + st * g.stage_bytes, ta, bar);
-                    if (nt == 2) copy_tile(true, stage0 + st * g.stage_bytes + tile_bytes, tb, bar);
+                                 : "memory");  // before any of the copies can complete
                 }
+                __syncwarp();
+                if (op_tile < nt) copy(true, stage0 + st * g.stage_bytes, ta, tb, bar);
                 ++it;
             }
         }
@@ -441,33 +460,31 @@ __global__ void __launch_bounds__(kPtThreads, 2) k_permute_tma(const __grid_cons
         }
     } else if (warp == 1) {
         // ---------------- storer ----------------
-        if (lane == 0) {
-            uint32_t it = 0;
-            for (;; ++it) {
-                const uint32_t st = it % S;
-                if (!perm_wait(perm_smem(&full[st]), (it / S) & 1, ab)) {
-                    give_up();
-                    break;
-                }
-                const int nt = ntile_of[st];
-                if (nt == 0) break;
-                if (!g.trivial_in && !perm_wait(perm_smem(&swapped[st]), (it / S) & 1, ab)) {
-                    give_up();
-                    break;
-                }
-                copy_tile(false, stage0 + st * g.stage_bytes, dst_a[st], 0);
-                if (nt == 2) copy_tile(false, stage0 + st * g.stage_bytes + tile_bytes, dst_b[st], 0);
-                asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
-                if (it > 0) {  // the stage before this one has been read out
-                    asm volatile("cp.async.bulk.wait_group.read 1;\n" ::: "memory");
+        uint32_t it = 0;
+        for (;; ++it) {
+            const uint32_t st = it % S;
+            bool ok = perm_wait(perm_smem(&full[st]), (it / S) & 1, ab);
+            const int nt = ok ? ntile_of[st] : 0;
+            if (ok && nt && !g.trivial_in) ok = perm_wait(perm_smem(&swapped[st]), (it / S) & 1, ab);
+            if (!__all_sync(0xffffffffu, ok)) {
+                if (lane == 0) give_up();
+                break;
+            }
+            if (nt == 0) break;
+            if (op_tile < nt) copy(false, stage0 + st * g.stage_bytes, dst_a[st], dst_b[st], 0);
+            asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
+            if (it > 0) {  // every lane's copies of the stage before this one have been read out
+                asm volatile("cp.async.bulk.wait_group.read 1;\n" ::: "memory");
+                __syncwarp();
+                if (lane == 0)
                     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(perm_smem(&empty[(it - 1) % S]))
                                  : "memory");
-                }
             }
-            asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
-            if (it > 0)  // the producer's end mark may wait for this stage
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(perm_smem(&empty[(it - 1) % S])) : "memory");
         }
+        asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
+        __syncwarp();
+        if (lane == 0 && it > 0)  // the producer's end mark may wait for this stage
+            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(perm_smem(&empty[(it - 1) % S])) : "memory");
     } else if (!g.trivial_in) {
         // ---------------- swappers ----------------
         const int w = (tid - 64) & (kPtSwap - 1), grp = (tid - 64) / kPtSwap;
@@ -776,7 +793,9 @@ int launch_permute_tma(float2 *psi, int nbits, const int *inv, cudaStream_t st, 
         return c;
     }();
     if (!cfg.ok) return -1;
-    const uint64_t ctas = 2 * (uint64_t)cfg.sms;
+    // odd: which tiles lead a pair follows their address bits, and with 304 CTAs, a multiple of 16, the
+    // low 4 bits of a CTA's turns would never change (a swap of bits 12 and 18 left half the CTAs idle)
+    const uint64_t ctas = 2 * (uint64_t)cfg.sms - 1;
     // candidates a producer takes at a time: many, since evaluating them costs its warp the same for 1
     // and for 32, but at least 16 turns a CTA, so that the last one is not half empty (2^24 amplitudes:
     // 127-141 us two random passes with 32 at a time, 94-110 with 4)
@@ -832,20 +851,25 @@ int launch_involution(float2 *psi, int nbits, const int *inv, cudaStream_t st, i
     bool any = false;
     for (int b = 0; b < nbits; b++) any |= inv[b] != b;
     if (!any) return 0;
-    // in-place tiles (no tile pairs) of at most 3 row bits, rows of >= 2^5 amplitudes: bulk copies
     PermGeom g;
-    int rc = build_geom(psi, nbits, inv, SYCSIM_PERM_TILE_SAME, g);
-    if (rc == 0 && g.nhh == 0 && g.q <= 3 && g.LB >= 5 && g.LB + g.q >= 8 && g.LB + g.q <= 12 && ((uintptr_t)psi & 15) == 0) {
+    const int rc = build_geom(psi, nbits, inv, SYCSIM_PERM_TILE, g);
+    if (rc == 0 && g.nhh == 0) {  // tiles that only permute in place gain from more work per CTA
+        PermGeom big;
+        if (build_geom(psi, nbits, inv, SYCSIM_PERM_TILE_SAME, big) == 0) g = big;
+    }
+    // long rows (see k_permute_tile_bulk): in place with at most 3 row bits, pairs without row bits, pairs
+    // of 2^11 amplitudes whose rows are 1 KiB and more
+    const bool bulk = g.nhh == 0 ? g.q <= 3 : (g.q == 0 || (g.LB + g.q == 11 && g.LB >= 7));
+    if (rc == 0 && bulk && g.LB >= 5 && g.LB + g.q >= 8 && g.LB + g.q <= (g.nhh ? 11 : 12) && ((uintptr_t)psi & 15) == 0) {
         const uint64_t tiles = 1ull << (nbits - g.LB - g.q);
         choose_lane_bits(g);
-        return launch_pdl(k_permute_tile_bulk, (unsigned)tiles, 256, sizeof(float2) << (g.LB + g.q), st, g, err) ==
-                       cudaSuccess
+        return launch_pdl(k_permute_tile_bulk, (unsigned)tiles, 256,
+                          (g.nhh ? 2 : 1) * (sizeof(float2) << (g.LB + g.q)), st, g, err) == cudaSuccess
                    ? 0
                    : -1;
     }
     const int tma = launch_permute_tma(psi, nbits, inv, st, err);
     if (tma <= 0) return tma;
-    rc = build_geom(psi, nbits, inv, SYCSIM_PERM_TILE, g);
     if (rc != 0) return rc;
     const int LB = g.LB, q = g.q;
     const uint64_t tiles = 1ull << (nbits - LB - q);
