@@ -46,6 +46,7 @@ struct MmaGeom {
     uint64_t n_mtiles;      // tiles of 16 groups: 2^(nbits - k - 4)
     int tpos[kMaxK];        // ascending target bits
     uint64_t moff[64];      // offset of member j
+    int early;              // the next kernel may start before this one ends (pdl_early)
 };
 
 __device__ __forceinline__ uint32_t to_tf32(float x)
@@ -129,6 +130,7 @@ __global__ void __launch_bounds__(256, mma_min_blocks(K)) k_apply_mma(const __gr
     constexpr int NC = NT < SYCSIM_MMA_NC ? NT : SYCSIM_MMA_NC;  // n-tiles per output chunk
     constexpr int FRAG_WORDS = KS * NT * 64;
     extern __shared__ uint32_t sb[];
+    if (g.early) pdl_launch_next();
     build_frag_tf32<K, kSplit>(block_mat_ptr(M), sb);
     pdl_wait();
 
@@ -136,7 +138,6 @@ __global__ void __launch_bounds__(256, mma_min_blocks(K)) k_apply_mma(const __gr
     const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     for (uint64_t mt = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; mt < g.n_mtiles;
          mt += nw) {
-        if (mt + nw >= g.n_mtiles) pdl_launch_next();  // this warp's last tile
         const uint64_t grp = mt * 16 + gid;
         float2 *p0 = g.psi + insert_zero_bits_t(grp, g.tpos, K);
         float2 *p1 = g.psi + insert_zero_bits_t(grp + 8, g.tpos, K);
@@ -246,6 +247,7 @@ __global__ void __launch_bounds__(256, mma_min_blocks(K)) k_apply_mma_f16x3(cons
     constexpr int NC = NT < SYCSIM_MMA_NC ? NT : SYCSIM_MMA_NC;
     constexpr int FRAG_WORDS = KS * NT * 64;
     extern __shared__ uint32_t sb[];
+    if (g.early) pdl_launch_next();
     build_frag_f16<K>(block_mat_ptr(M), sb);
     pdl_wait();
 
@@ -253,7 +255,6 @@ __global__ void __launch_bounds__(256, mma_min_blocks(K)) k_apply_mma_f16x3(cons
     const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
     for (uint64_t mt = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; mt < g.n_mtiles;
          mt += nw) {
-        if (mt + nw >= g.n_mtiles) pdl_launch_next();  // this warp's last tile
         const uint64_t grp = mt * 16 + gid;
         float2 *p0 = g.psi + insert_zero_bits_t(grp, g.tpos, K);
         float2 *p1 = g.psi + insert_zero_bits_t(grp + 8, g.tpos, K);
@@ -327,6 +328,7 @@ int launch_mma(float2 *psi, int nbits, const int *tpos, const BlockMat<K> &M, cu
     constexpr int D = 1 << K;
     MmaGeom g{};
     g.psi = psi;
+    g.early = pdl_early(nbits);
     g.n_mtiles = 1ull << (nbits - K - 4);
     for (int i = 0; i < K; i++) g.tpos[i] = tpos[i];
     for (int j = 0; j < D; j++) {

@@ -88,6 +88,7 @@ struct Tc5Geom {
     uint64_t roff[8];        // address offset of row bit j
     uint64_t moff[64];       // address offset of member m
     int *err;                // set to 1 if a wait timed out
+    int early;               // the next kernel may start at this one's last tiles (pdl_early)
     double *red;             // if set: this CTA's (sum p, sum p^2) of the results at red[2 blockIdx.x]
 };
 
@@ -483,7 +484,7 @@ __global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tcgen05(const __grid_c
                 if (lane == 0) give_up();
                 break;
             }
-            if (tile + gridDim.x >= g.n_tiles) pdl_launch_next();  // this CTA's last tile
+            if (g.early && tile + gridDim.x >= g.n_tiles) pdl_launch_next();  // this CTA's last tile
             const uint64_t base = insert_zero_bits_g(tile * (kRows * R2), g.tpos, K);
             const uint32_t bar = smem_u32(&loaded[st]);
             if (lane == 0) {
@@ -836,7 +837,7 @@ __global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tc6a(const __grid_cons
                 if (lane == 0) give_up();
                 break;
             }
-            if (tile + gridDim.x >= g.n_tiles) pdl_launch_next();  // this CTA's last tile
+            if (g.early && tile + gridDim.x >= g.n_tiles) pdl_launch_next();  // this CTA's last tile
             const uint64_t base = insert_zero_bits_g(tile * kRows, g.tpos, 6);
             const uint32_t bar = smem_u32(&loaded[st]);
             if (lane == 0) mbar_expect_tx(bar, kTc6Stage);  // before any of the copies can complete
@@ -1029,6 +1030,7 @@ int launch_tc5(sim_t *h, float2 *psi, int nbits, const int *tpos, const BlockMat
 {
     Tc5Geom g{};
     g.psi = psi;
+    g.early = pdl_early(nbits);
     g.red = red;
     for (int i = 0; i < K; i++) g.tpos[i] = tpos[i];  // ascending
     g.err = h->d_errflag;

@@ -18,10 +18,15 @@ namespace sycsim {
 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
-// The next kernel of the stream may start, once every CTA of this one has got here or left.  The
-// persistent tensor-core kernels call it at a CTA's last tile (2 % faster on a 20-qubit plan than
-// at the start, where the next kernel's CTAs crowd the SMs that are still idle).
+// The next kernel of the stream may start, once every CTA of this one has got here or left.
 __device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+
+// Whether a tensor-core pass over 2^nbits amplitudes lets the next one start early (the tcgen05 kernels
+// at each CTA's last tile, 2 % faster on a 20-qubit plan than at the start, where the next kernel's
+// CTAs crowd the SMs that are still idle).  Measured on plans, early / not: 22 qubits 266 / 290 us, 24
+// qubits 849 / 869, 26 qubits 3.31 / 3.34 ms, 28 qubits 31.48 / 31.56; at 30 qubits, where a pass takes
+// 2.7 ms and nothing is gained, 60.8 / 58.5 ms.
+inline bool pdl_early(int nbits) { return nbits <= 28; }
 
 template <typename... P, typename... A>
 cudaError_t launch_pdl(void (*kern)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A &&...args)
