@@ -28,11 +28,12 @@
 //    corrections hi*lo + lo*hi through a second (their rounding is 2^-11 smaller), and commits
 //    them to the stage's mbarrier;
 //  * drainer warps 10-17 read both accumulators (tcgen05.ld 32x32b: warp w sees TMEM lanes
-//    32 (w % 4) ..), add them and undo the row's scale.  With a deep stage ring the amplitudes
-//    go back into the stage and the lanes of warp 10 store its runs with bulk copies; with the
-//    3-stage ring of 64 KiB tiles, or a target below bit 4, they are stored from registers (16
-//    consecutive rows cover 64-128 contiguous bytes), which frees the stage as soon as TMEM is
-//    read.  Blocks with two or more targets below bit 4 are left to the other kernels.
+//    32 (w % 4) ..), add them, undo the row's scale and store from registers (16 consecutive rows
+//    cover 64-128 contiguous bytes); the stage is free as soon as the MMAs have read it.  (Writing the
+//    results back into the stage and storing its runs with bulk copies, as 32 KiB tiles did, holds the
+//    stage longer: 2^30 amplitudes, k = 4 3.13-3.89 ms instead of 2.78, k = 5 with a target at bits 4-7
+//    3.06 instead of 2.66-2.70.)  Blocks with two or more targets below bit 4 are left to the other
+//    kernels.
 // K (input reals) is interleaved, column 2m + p is part p (Re, Im) of member m, so a row's
 // 16-byte chunk is four consecutive members; N likewise.  R^T (hi, lo; FP16, core-matrix layout)
 // is split from the FP32 matrix into shared memory once per CTA.  Two TMEM accumulator sets let
@@ -59,10 +60,6 @@
 
 namespace sycsim {
 namespace {
-
-#ifndef SYCSIM_TC6_ATMEM
-#define SYCSIM_TC6_ATMEM 1  // 6-qubit blocks: A operand in tensor memory (k_apply_tc6a)
-#endif
 
 #ifndef SYCSIM_TC5_RUN_LOG2_MAX
 #define SYCSIM_TC5_RUN_LOG2_MAX 8  // 2 KiB copies: measured fastest (1 KiB: -26%, 4 KiB: -9%)
@@ -235,14 +232,8 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_
 }
 
 // A tile is R2 sub-tiles of 128 groups (row bit 7 = sub-tile), one MMA M = 128 each.
-__device__ __forceinline__ void bulk_store(void *dst, uint32_t src, uint32_t bytes)
-{
-    asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;\n" ::"l"(dst), "r"(src), "r"(bytes)
-                 : "memory");
-}
-
 // Shared memory: S stages of one tile each (raw amplitudes, then A hi | A lo of each sub-tile in
-// place, then the results), then B hi | B lo (KS slices of N x 16 FP16 each).
+// place), then B hi | B lo (KS slices of N x 16 FP16 each).
 template <int K, int R2>
 struct Tc5Layout {
     static constexpr int D = 1 << K;
@@ -254,19 +245,14 @@ struct Tc5Layout {
     static constexpr int B_BYTES = KS * B_SLICE;
     static constexpr int SUB = kRows * D * 8;     // one sub-tile = 2 * A_BYTES
     static constexpr int STAGE = R2 * SUB;
-    // stages: K <= 5 within 200 KiB (at most 8); K = 6 (64 KiB tiles, 64 KiB of B hi/lo) fits 2
-    static constexpr int S = K == 6 ? 2 : ((200 * 1024) / STAGE < 8 ? (200 * 1024) / STAGE : 8);
+    // stages within 200 KiB, at most 8
+    static constexpr int S = (200 * 1024) / STAGE < 8 ? (200 * 1024) / STAGE : 8;
     static constexpr int SMEM = S * STAGE + 2 * B_BYTES;
     static constexpr int TMEM_SUB = 2 * N;        // main + corrections of one sub-tile
     static constexpr int TMEM_SET = R2 * TMEM_SUB;
     static constexpr int TMEM_COLS = 2 * TMEM_SET;  // two sets
     static_assert(SUB == 2 * A_BYTES, "A hi/lo fill a sub-tile");
-    static_assert(S >= (K == 6 ? 2 : 3), "stage ring too short");
-    static_assert(K < 6 || R2 == 1, "6-qubit blocks: one 128-group sub-tile (tensor memory)");
-    // results leave through the stage with bulk stores when the ring is deep enough to hold a
-    // stage until its store has read it; the 3-stage ring (64 KiB tiles) stores from registers so
-    // that a stage is free as soon as its accumulators are read (measured: +20% there, -8% at 6+)
-    static constexpr bool BULK_STORE = S >= 6;
+    static_assert(K <= 5 && S >= 3, "stage ring too short");
     static_assert(TMEM_COLS <= 512, "tensor memory");
 };
 
@@ -337,11 +323,8 @@ __device__ __forceinline__ void build_b(const float2 *m, uint8_t *bHi, uint8_t *
 //   converters: wait loaded[s], read the rows, combine the halves' maxima (barrier), write A and
 //     the row scales in place, arrive full[s];
 //   MMA thread: wait full[s] and tmem_free of tile i - 2, multiply, commit to mma_done[s];
-//   drainers: wait mma_done[s] and full[s], take the row scales and the tile base into registers;
-//     storing from registers, arrive drained[s] right then (the MMAs have read the stage), read
-//     TMEM, arrive tmem_free and store; with bulk stores, read TMEM, arrive tmem_free, write the
-//     results into stage s, barrier, and warp 10 stores the runs and, once the store of tile
-//     i - 1 has read its stage, arrives drained for it.
+//   drainers: wait mma_done[s] and full[s], take the row scales and the tile base into registers,
+//     arrive drained[s] right then (the MMAs have read the stage), read TMEM, arrive tmem_free, store.
 // A stage is reloaded only after every drainer has passed its waits for it and taken what it
 // needs, and a TMEM set reused only after its read, so no barrier can run a phase ahead of a
 // waiter that still has to see the previous phase.
@@ -350,7 +333,6 @@ __global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tcgen05(const __grid_c
                                                                   const __grid_constant__ BlockMat<K> M)
 {
     using L = Tc5Layout<K, R2>;
-    constexpr bool BULK = L::BULK_STORE && !LOWT;  // results back through the stage
     constexpr int D = L::D, KS = L::KS, N = L::N, S = L::S, H = D / 2;  // H members per thread
     extern __shared__ __align__(1024) uint8_t sm[];
     uint8_t *bHi = sm + S * L::STAGE, *bLo = bHi + L::B_BYTES;
@@ -372,7 +354,7 @@ __global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tcgen05(const __grid_c
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(&full[st])), "r"(kConv) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;\n" ::"r"(smem_u32(&mma_done[st])) : "memory");
             asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(smem_u32(&drained[st])),
-                         "r"(BULK ? 1 : kDrain)
+                         "r"(kDrain)
                          : "memory");
         }
         for (int st = 0; st < 2; ++st)
@@ -541,16 +523,10 @@ __global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tcgen05(const __grid_c
         const int q = warp & 3;                        // TMEM lane quarter this warp may read
         const int half = (warp - kMmaWarp - 1) >> 2;   // warps 10-13: members 0..H-1; 14-17: H..D-1
         const int row = 32 * q + (tid & 31);
-        const bool store_warp = warp == kMmaWarp + 1;  // bulk stores: its lanes store a run each
-        const int lane = tid & 31;
-        uint32_t rx = 0;  // staging index of this row
         uint64_t ro = 0;  // address offset of this row within the tile (16 consecutive rows: 128 B)
 #pragma unroll
         for (int j = 0; j < 7; ++j)
-            if ((row >> j) & 1) {
-                rx |= g.ridx[j];
-                ro += g.roff[j];
-            }
+            if ((row >> j) & 1) ro += g.roff[j];
         double r1 = 0.0, r2 = 0.0;  // fused reduction (g.red)
         uint32_t i = 0;
         for (uint64_t tile = blockIdx.x; tile < g.n_tiles; tile += gridDim.x, ++i) {
@@ -562,44 +538,14 @@ __global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tcgen05(const __grid_c
                 break;
             }
             asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-            uint8_t *stage = sm + st * L::STAGE;
             float2 *const dst = g.psi + tile_base[st] + ro;
             float inv[R2];
 #pragma unroll
             for (int u = 0; u < R2; ++u) inv[u] = row_inv[st][u][row];
-            // storing from registers, the stage is dead once the MMAs have read it (mma_done): with
-            // its row scales and base in registers, release it now so the next tile's copies start
-            // while this one is drained
-            if constexpr (!BULK) mbar_arrive(smem_u32(&drained[st]));
-            if constexpr (K == 6) {
-                // 64 output reals per thread: read, add, unscale and store 16 columns at a time
-                // (registers), releasing the tensor memory and the stage after the last read
-                const uint32_t lane_base = tmem + (i & 1) * L::TMEM_SET + ((uint32_t)(32 * q) << 16) + half * (N / 2);
-#pragma unroll
-                for (int c0 = 0; c0 < N / 2; c0 += 16) {
-                    float a[16], b[16];
-                    tmem_ld16(lane_base + c0, a);
-                    tmem_ld16(lane_base + N + c0, b);
-                    asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
-                    if (c0 == N / 2 - 16) {
-                        asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-                        mbar_arrive(smem_u32(&tmem_free[i & 1]));
-                    }
-                    float t1 = 0.f, t2 = 0.f;
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        const float2 v =
-                            make_float2((a[2 * j] + b[2 * j]) * inv[0], (a[2 * j + 1] + b[2 * j + 1]) * inv[0]);
-                        const float p = fmaf(v.x, v.x, v.y * v.y);
-                        t1 += p;
-                        t2 = fmaf(p, p, t2);
-                        __stcs(dst + g.moff[H * half + c0 / 2 + j], v);
-                    }
-                    r1 += t1;
-                    r2 += t2;
-                }
-                continue;
-            }
+            // results are stored from registers, so the stage is dead once the MMAs have read it
+            // (mma_done): with its row scales and base in registers, release it now so the next tile's
+            // copies start while this one is drained
+            mbar_arrive(smem_u32(&drained[st]));
 #pragma unroll
             for (int u = 0; u < R2; ++u) {
                 const uint32_t lane_base =
@@ -626,34 +572,11 @@ __global__ void __launch_bounds__(kThreadsTc5, 1) k_apply_tcgen05(const __grid_c
                 }
                 r1 += t1;
                 r2 += t2;
-                if constexpr (BULK) {
-                    const uint32_t rxu = u ? rx | g.ridx[7] : rx;
+                float2 *const du = u ? dst + g.roff[7] : dst;
 #pragma unroll
-                    for (int j = 0; j < H; ++j)
-                        *reinterpret_cast<float2 *>(stage + 8 * (g.midx[H * half + j] | rxu)) = o[j];
-                } else {
-                    float2 *const du = u ? dst + g.roff[7] : dst;
-#pragma unroll
-                    for (int j = 0; j < H; ++j) __stcs(du + g.moff[H * half + j], o[j]);
-                }
-            }
-            if constexpr (BULK) {
-                asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // the bulk store reads it
-                bar_sync(2, kDrain);  // the whole tile is back in the stage
-                if (store_warp) {
-                    float2 *const tb = g.psi + tile_base[st];
-                    const uint32_t src = smem_u32(stage);
-                    for (int c = lane; c < n_runs; c += 32) bulk_store(tb + g.off_run[c], src + c * run_bytes, run_bytes);
-                    asm volatile("cp.async.bulk.commit_group;\n" ::: "memory");
-                    if (i > 0) {
-                        asm volatile("cp.async.bulk.wait_group.read 1;\n" ::: "memory");  // tile i - 1 read out
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(smem_u32(&drained[(i - 1) % S]));
-                    }
-                }
+                for (int j = 0; j < H; ++j) __stcs(du + g.moff[H * half + j], o[j]);
             }
         }
-        if (BULK && store_warp) asm volatile("cp.async.bulk.wait_group 0;\n" ::: "memory");
         if (g.red) drain_partials(r1, r2, tid - (kConv + 64), red_part, g.red);
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
@@ -1039,13 +962,8 @@ int launch_tc5(sim_t *h, float2 *psi, int nbits, const int *tpos, const BlockMat
     if (g.nlow > (K >= 5 ? 1 : 0)) return -2;  // not eligible (see tcgen05_eligible)
     if constexpr (K == 6) {  // 128-group tiles only: two 256-column accumulator sets fill the TMEM
         if (tile_geometry<K>(nbits, tpos, 7, g) < 0) return -1;
-#if SYCSIM_TC6_ATMEM
         if (g.nlow > 0) return launch_tc6a<true, BF>(g, M, nbits, st, grid_out);
         return launch_tc6a<false, BF>(g, M, nbits, st, grid_out);
-#else
-        if (g.nlow > 0) return launch_tc5_kr<K, 1, true, BF>(g, M, nbits, st, grid_out);
-        return launch_tc5_kr<K, 1, false, BF>(g, M, nbits, st, grid_out);
-#endif
     } else {
         // 128-group tiles when their runs reach 2 KiB (bit 7 is a target, or a target lies below
         // it); otherwise 256-group tiles, whose 8th row bit is bit 7, so that every bulk copy
