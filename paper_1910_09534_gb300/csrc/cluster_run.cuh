@@ -25,6 +25,28 @@ namespace sycsim {
 constexpr int kClThreads = 256;  // 512: 1.3-1.9 times the time at 10-18 qubits (dearer barriers)
 constexpr int kClMaxK = 5;
 
+// CTAs of the cluster for a kernel of kClThreads threads on the current device: 16 (beyond the portable
+// 8) where the device can place such a cluster, else 8.
+template <typename Kern>
+int cluster_ctas(Kern kern)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = 16;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(16);
+    cfg.blockDim = dim3(kClThreads);
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0)
+        return 16;
+    cudaGetLastError();  // not an error of the caller: the narrower cluster is used
+    return 8;
+}
+
 struct ClBlock {
     int k;
     int tpos[kMaxK];   // ascending physical target bits

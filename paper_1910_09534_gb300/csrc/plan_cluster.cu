@@ -33,8 +33,7 @@ __global__ void __launch_bounds__(kClThreads, 1) k_plan_cluster(float2 *psi, int
 
 }  // namespace
 
-// CTAs of the cluster on the current device: 16 (beyond the portable 8) where the device can place
-// such a cluster, else 8.
+// CTAs of the cluster on the current device, looked up once per device
 static int plan_ctas()
 {
     static std::atomic<uint64_t> wide{0}, known{0};  // bit d: device d < 64
@@ -42,21 +41,7 @@ static int plan_ctas()
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 8;
     const uint64_t bit = 1ull << dev;
     if (!(known.load(std::memory_order_acquire) & bit)) {
-        cudaLaunchAttribute attr{};
-        attr.id = cudaLaunchAttributeClusterDimension;
-        attr.val.clusterDim.x = 16;
-        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(16);
-        cfg.blockDim = dim3(kClThreads);
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        int n = 0;
-        if (cudaFuncSetAttribute(k_plan_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-            cudaOccupancyMaxActiveClusters(&n, k_plan_cluster, &cfg) == cudaSuccess && n > 0)
-            wide.fetch_or(bit, std::memory_order_acq_rel);
-        else
-            cudaGetLastError();  // not an error of this call: the narrower cluster is used
+        if (cluster_ctas(k_plan_cluster) == 16) wide.fetch_or(bit, std::memory_order_acq_rel);
         known.fetch_or(bit, std::memory_order_acq_rel);
     }
     return wide.load(std::memory_order_acquire) & bit ? 16 : 8;

@@ -57,58 +57,63 @@ struct PackedJob {
 };
 
 constexpr int kPackMaxK = kClMaxK;
-constexpr int kPackCtas = 8;  // CTAs of the cluster that runs one packed circuit
+constexpr int kPackMaxCtas = 16;  // CTAs of the cluster that runs one packed circuit: 16 or 8 (manage_workers)
 
 struct PackShared {
     ClShared run;
     double red[2][kClThreads / 32];
-    double part[2][kPackCtas];  // the leader's: each CTA's sums
+    double part[2][kPackMaxCtas];  // the leader's: the sums of each 16th of the state
 };
 
 // One whole small circuit on one cluster: reset to |0...0>, every block (cluster_run.cuh), then
 // (sum p, sum p^2) into out[0..1].  Measured one CTA to a circuit before: 18 qubits, 12 cycles 5.4
-// ms, with the other SMs idle unless many circuits were waiting.
+// ms, with the other SMs idle unless many circuits were waiting; on 8 CTAs 1.38 ms, on 16 0.95 (from
+// submission to result).
 __device__ __forceinline__ void run_circuit_cluster(const PackedJob &J, PackShared &sh, double *out)
 {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
-    const uint32_t rank = cl.block_rank();
-    const uint64_t amps = 1ull << J.n, step = (uint64_t)kPackCtas * kClThreads;
+    const uint32_t rank = cl.block_rank(), ncta = cl.num_blocks();
+    const uint64_t amps = 1ull << J.n, step = (uint64_t)ncta * kClThreads;
     const uint64_t first = (uint64_t)rank * kClThreads + threadIdx.x;
     for (uint64_t i = first; i < amps; i += step) J.psi[i] = make_float2(i == 0 ? 1.f : 0.f, 0.f);
     if (J.nblocks == 0) cl.sync();
     cl_run_blocks(J.psi, J.n, J.blocks, J.mats, J.nblocks, sh.run);
-    double s1 = 0.0, s2 = 0.0;
-    for (uint64_t i = first; i < amps; i += step) {
-        const float2 v = __ldcg(J.psi + i);
-        const double p = (double)v.x * v.x + (double)v.y * v.y;
-        s1 += p;
-        s2 += p * p;
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-        s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-    }
+    // the sums in 16 parts, whatever the width of the cluster: the result does not depend on it
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (lane == 0) {
-        sh.red[0][warp] = s1;
-        sh.red[1][warp] = s2;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double a = 0.0, c = 0.0;
-        for (int w = 0; w < kClThreads / 32; ++w) {
-            a += sh.red[0][w];
-            c += sh.red[1][w];
+    for (uint32_t part = rank; part < kPackMaxCtas; part += ncta) {
+        double s1 = 0.0, s2 = 0.0;
+        for (uint64_t i = (uint64_t)part * kClThreads + threadIdx.x; i < amps; i += kPackMaxCtas * kClThreads) {
+            const float2 v = __ldcg(J.psi + i);
+            const double p = (double)v.x * v.x + (double)v.y * v.y;
+            s1 += p;
+            s2 += p * p;
         }
-        PackShared *lead = cl.map_shared_rank(&sh, 0);
-        lead->part[0][rank] = a;
-        lead->part[1][rank] = c;
+        for (int o = 16; o > 0; o >>= 1) {
+            s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+            s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+        }
+        if (lane == 0) {
+            sh.red[0][warp] = s1;
+            sh.red[1][warp] = s2;
+        }
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double a = 0.0, c = 0.0;
+            for (int w = 0; w < kClThreads / 32; ++w) {
+                a += sh.red[0][w];
+                c += sh.red[1][w];
+            }
+            PackShared *lead = cl.map_shared_rank(&sh, 0);
+            lead->part[0][part] = a;
+            lead->part[1][part] = c;
+        }
+        __syncthreads();
     }
     cl.sync();
-    if (rank == 0 && threadIdx.x == 0) {  // in the order of the CTAs
+    if (rank == 0 && threadIdx.x == 0) {  // in the order of the parts
         double a = 0.0, c = 0.0;
-        for (int r = 0; r < kPackCtas; ++r) {
+        for (int r = 0; r < kPackMaxCtas; ++r) {
             a += sh.part[0][r];
             c += sh.part[1][r];
         }
@@ -149,7 +154,7 @@ __device__ __forceinline__ uint32_t ld_acquire_sys(const uint32_t *p)
 // next one; the cluster leaves once no job has been published for kWorkerIdleNs.  Jobs published while
 // the kernel runs are picked up without a new launch.  The only wait for the host is on its published
 // count, bounded by the idle time; the cluster's barriers wait for CTAs that are resident together.
-__global__ void __cluster_dims__(kPackCtas, 1, 1) __launch_bounds__(kClThreads, 2)
+__global__ void __launch_bounds__(kClThreads, 2)
     k_packed_worker(const uint32_t *published, QSlot *ring, uint32_t *head)
 {
     namespace cg = cooperative_groups;
@@ -178,7 +183,7 @@ __global__ void __cluster_dims__(kPackCtas, 1, 1) __launch_bounds__(kClThreads, 
             }
             PackedJob mine{};
             if (got != 0xffffffffu) mine = ring[got % kQueueCap].job;
-            for (int r = 0; r < kPackCtas; ++r) {
+            for (uint32_t r = 0; r < cl.num_blocks(); ++r) {
                 *cl.map_shared_rank(&job, r) = got;
                 *cl.map_shared_rank(&J, r) = mine;
             }
@@ -305,6 +310,7 @@ struct srv_s {
     uint64_t next_index = 0, published = 0, retired = 0;
     cudaStream_t wst[2] = {nullptr, nullptr};
     cudaEvent_t wev[2] = {nullptr, nullptr};
+    int max_ctas = 8;  // widest cluster of the workers: 16 where the device can place one
     int wclusters[2] = {0, 0};  // clusters of a worker still running (0: none)
     int sms = 0;
     double *h_results = nullptr;  // pinned ring of result pairs for unpacked requests
@@ -611,9 +617,27 @@ void manage_workers(srv_t *s, uint64_t not_done, bool *progressed)
     if (not_done <= (uint64_t)running) return;
     for (int w = 0; w < 2; w++)
         if (!s->wclusters[w]) {
-            const int clusters = (int)std::min<uint64_t>(not_done - running, (uint64_t)(2 * s->sms / kPackCtas));
-            k_packed_worker<<<clusters * kPackCtas, kClThreads, 0, s->wst[w]>>>(s->d_ctl, s->d_ring, s->d_head);
-            if (cudaGetLastError() != cudaSuccess || cudaEventRecord(s->wev[w], s->wst[w]) != cudaSuccess) return;
+            // Clusters of 16 finish a circuit sooner (16 of 18 qubits in 8.6 -> 4.8 ms, one in 1.41 -> 0.96;
+            // at 12 qubits no difference), but wait longer for 16 free SMs of one group beside the large
+            // lane's kernels, which then gets the portable 8.
+            int ctas = s->max_ctas;
+            for (auto &r : s->slot_req)
+                if (r) ctas = 8;
+            const int clusters = (int)std::min<uint64_t>(not_done - running, (uint64_t)(2 * s->sms / ctas));
+            cudaLaunchAttribute attr{};
+            attr.id = cudaLaunchAttributeClusterDimension;
+            attr.val.clusterDim.x = ctas;
+            attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+            cudaLaunchConfig_t cfg{};
+            cfg.gridDim = dim3(clusters * ctas);
+            cfg.blockDim = dim3(kClThreads);
+            cfg.stream = s->wst[w];
+            cfg.attrs = &attr;
+            cfg.numAttrs = 1;
+            if (cudaLaunchKernelEx(&cfg, k_packed_worker, (const uint32_t *)s->d_ctl, s->d_ring, s->d_head) !=
+                    cudaSuccess ||
+                cudaEventRecord(s->wev[w], s->wst[w]) != cudaSuccess)
+                return;
             s->wclusters[w] = clusters;
             *progressed = true;
             return;
@@ -948,6 +972,7 @@ int srv_create(const srv_opts *opts, srv_t **out)
                cudaHostGetDevicePointer(reinterpret_cast<void **>(&s->d_ctl), s->ctl, 0) == cudaSuccess &&
                cudaMalloc(reinterpret_cast<void **>(&s->d_head), sizeof(uint32_t)) == cudaSuccess &&
                cudaMemset(s->d_head, 0, sizeof(uint32_t)) == cudaSuccess;
+    s->max_ctas = cluster_ctas(k_packed_worker);
     for (int w = 0; w < 2 && qok; w++)
         qok = cudaStreamCreateWithFlags(&s->wst[w], cudaStreamNonBlocking) == cudaSuccess &&
               cudaEventCreateWithFlags(&s->wev[w], cudaEventDisableTiming) == cudaSuccess;
