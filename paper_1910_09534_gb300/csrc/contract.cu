@@ -486,7 +486,12 @@ __global__ void __launch_bounds__(kCtThreads, 1) k_contract_tcgen05(CtArgs g, co
             ct_tile(tile, g.tiles_x, g.tiles_y, tx, ty);
             float2 *dst = g.psi + ct_dep((uint64_t)tx << 7, o.xbit, g.n1) + ct_dep((uint64_t)ty << 7, o.ybit, g.n2) +
                           xoff[row];
-#pragma unroll 1
+            // The accumulator into registers (128 a thread) and released: the next tile's MMAs wait for
+            // the 256 KiB read, not for the stores.  The stores took 0.2-0.35 of a tile of 4-16 k-steps:
+            // 14 + 13 qubits, 256 entanglement values 550 -> 495-520 us, 14 + 14 and 64 532 -> 453,
+            // 14 + 14 and 16 (bound by the stores) 403 -> 392.
+            float2 v[64];
+#pragma unroll
             for (int c = 0; c < 64; c += 16) {
                 const int y0 = half * 64 + c;
                 float xr[16], xi[16], yr[16], yi[16];
@@ -497,10 +502,12 @@ __global__ void __launch_bounds__(kCtThreads, 1) k_contract_tcgen05(CtArgs g, co
                 asm volatile("tcgen05.wait::ld.sync.aligned;\n" ::: "memory");
 #pragma unroll
                 for (int j = 0; j < 16; ++j)
-                    __stcs(dst + yoff[y0 + j], make_float2((xr[j] - yi[j]) * inv, (xi[j] + yr[j]) * inv));
+                    v[c + j] = make_float2((xr[j] - yi[j]) * inv, (xi[j] + yr[j]) * inv);
             }
             asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
             ct_arrive(ct_smem(&acc_empty));
+#pragma unroll
+            for (int j = 0; j < 64; ++j) __stcs(dst + yoff[half * 64 + j], v[j]);
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
