@@ -8,8 +8,8 @@
 // where P places x's bits on the side-0 qubits and y's on the side-1 qubits in the output
 // handle's current physical layout.
 // Two kernels compute it:
-//  * k_contract_fp32 (CUDA cores): 64 x 64 output tiles, 4 x 4 per thread, FP32 products and
-//    sums, operands staged through shared memory 16 entanglement values at a time;
+//  * k_contract_fp32 (CUDA cores): 64 x 64 output tiles, 2 x 8 per thread, FP32 products and
+//    sums, operands staged through shared memory up to 16 entanglement values at a time;
 //  * k_contract_tcgen05 (5th-generation tensor cores): 128 x 128 output tiles as two real GEMMs
 //    of M = 128 (x) x N = 256 (Re y | Im y) x K = 16 (entanglement values) per step,
 //    X = [Re T1] . [Re T2 | Im T2] and Y = [Im T1] . [Re T2 | Im T2] in tensor memory, so that
@@ -39,7 +39,10 @@ using namespace sycsim;
 
 namespace {
 
-constexpr int kFx = 64, kFy = 64, kFk = 16;  // FP32 kernel: tile x, tile y, entanglement chunk
+constexpr int kFrx = 2, kFry = 8;               // FP32 kernel: x's and y's of a thread
+constexpr int kFx = 32 * kFrx, kFy = 8 * kFry;  // its tile: lane = x, warp = y
+constexpr int kFocc = 2;                        // its CTAs on an SM
+constexpr int kFk = 16;                         // entanglement values staged at a time
 
 // Where psi lands: bit i of x (side-0 qubit i, increasing qubit order) adds xbit[i] to the
 // physical index, bit j of y adds ybit[j] (powers of two from the output handle's layout).
@@ -47,6 +50,19 @@ struct CtOut {
     uint64_t xbit[kMaxQubits];
     uint64_t ybit[kMaxQubits];
 };
+
+const LaunchCfg &ct_cfg()
+{
+    static const LaunchCfg cfg = [] {
+        LaunchCfg c;
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess) return c;
+        if (cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return c;
+        c.ok = true;
+        return c;
+    }();
+    return cfg;
+}
 
 __device__ __forceinline__ uint64_t ct_dep(uint64_t v, const uint64_t *bit, int nb)
 {
@@ -56,72 +72,127 @@ __device__ __forceinline__ uint64_t ct_dep(uint64_t v, const uint64_t *bit, int 
     return o;
 }
 
-// t1 (t2): 2^n1 (2^n2) columns of each entanglement row, rows ld1 (ld2) amplitudes apart.
-__global__ void __launch_bounds__(256) k_contract_fp32(const float2 *__restrict__ t1, const float2 *__restrict__ t2,
-                                                       float2 *__restrict__ psi, int n1, int n2, uint64_t n_e,
-                                                       uint64_t ld1, uint64_t ld2, const __grid_constant__ CtOut o)
+__device__ __forceinline__ void ct_copy8(void *dst, const void *src)
 {
-    __shared__ __align__(16) float2 sa[kFk][kFx];
-    __shared__ __align__(16) float2 sb[kFk][kFy];
-    __shared__ uint64_t xoff[kFx], yoff[kFy];
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+
+// t1 (t2): 2^n1 (2^n2) columns of each entanglement row, rows ld1 (ld2) amplitudes apart.
+// Bound by the stores at 1 and 4 entanglement values, by the FMA rate from 16 on.  Persistent CTAs:
+// the operands of the next tile or chunk arrive (cp.async) while this one is multiplied and stored;
+// only as many entanglement values are multiplied as there are; a warp stores 32 consecutive x.  A CTA
+// a tile, always 16 values and 4 x 4 results a thread in 8-byte stores 32 bytes apart took, 14 + 14
+// qubits, 4 / 16 / 64 values: 1306 / 1372 / 3325 us; this 510 / 965 / 3196 (2^31 bytes of results take
+// 321, the FMAs 116 / 464 / 1856 at the nominal rate).  13 + 8 qubits, 4 values: 17.0 -> 8.8.  4 x 8 a
+// thread is 3-5 % faster at 28 qubits and 20-50 % slower at 16-21; 2 x 4 and 4 x 4 are slower.
+__global__ void __launch_bounds__(256, kFocc)
+    k_contract_fp32(const float2 *__restrict__ t1, const float2 *__restrict__ t2, float2 *__restrict__ psi, int n1,
+                    int n2, uint64_t n_e, uint64_t ld1, uint64_t ld2, const __grid_constant__ CtOut o)
+{
+    __shared__ __align__(16) float2 sa[2][kFk][kFx];
+    __shared__ __align__(16) float2 sb[2][kFk][kFy];
+    __shared__ uint64_t yoff[kFy];  // offsets of y's low bits, within a tile
     const uint64_t X = 1ull << n1, Y = 1ull << n2;
-    const uint64_t tiles_x = (X + kFx - 1) / kFx;
-    const uint64_t x0 = (blockIdx.x % tiles_x) * kFx, y0 = (blockIdx.x / tiles_x) * kFy;
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    if (tid < kFx)
-        xoff[tid] = ct_dep(x0 + tid, o.xbit, n1);
-    else if (tid < kFx + kFy)
-        yoff[tid - kFx] = ct_dep(y0 + tid - kFx, o.ybit, n2);
-    float2 acc[4][4];  // [y][x]
+    const uint64_t tiles_x = (X + kFx - 1) / kFx, tiles = tiles_x * ((Y + kFy - 1) / kFy);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (tid < kFy) yoff[tid] = ct_dep(tid, o.ybit, min(n2, 7));
+    uint64_t xoff[kFrx];  // the same of this thread's x's
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
+    for (int i = 0; i < kFrx; ++i) xoff[i] = ct_dep(lane + 32 * i, o.xbit, min(n1, 7));
+
+    auto load = [&](int buf, uint64_t tile, uint64_t e0) {
+        const uint64_t x0 = (tile % tiles_x) * kFx, y0 = (tile / tiles_x) * kFy;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) acc[j][i] = make_float2(0.f, 0.f);
-    for (uint64_t e0 = 0; e0 < n_e; e0 += kFk) {
-#pragma unroll
-        for (int r = 0; r < (kFk * kFx) / 256; ++r) {
+        for (int r = 0; r < kFk * kFx / 256; ++r) {
             const int idx = tid + 256 * r, k = idx / kFx, c = idx % kFx;
-            const uint64_t e = e0 + k;
-            sa[k][c] = (e < n_e && x0 + c < X) ? t1[x0 + c + e * ld1] : make_float2(0.f, 0.f);
-            sb[k][c] = (e < n_e && y0 + c < Y) ? t2[y0 + c + e * ld2] : make_float2(0.f, 0.f);
+            if (e0 + k < n_e && x0 + c < X) ct_copy8(&sa[buf][k][c], t1 + x0 + c + (e0 + k) * ld1);
         }
+#pragma unroll
+        for (int r = 0; r < kFk * kFy / 256; ++r) {
+            const int idx = tid + 256 * r, k = idx / kFy, c = idx % kFy;
+            if (e0 + k < n_e && y0 + c < Y) ct_copy8(&sb[buf][k][c], t2 + y0 + c + (e0 + k) * ld2);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    };
+
+    float2 acc[kFry][kFrx];
+    uint64_t tile = blockIdx.x, e0 = 0;
+    load(0, tile, 0);  // the grid is no larger than the tiles
+    for (int buf = 0; tile < tiles; buf ^= 1) {
+        uint64_t next_tile = tile, next_e = e0 + kFk;
+        if (next_e >= n_e) {
+            next_tile += gridDim.x;
+            next_e = 0;
+        }
+        if (next_tile < tiles) {
+            load(buf ^ 1, next_tile, next_e);
+            asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        } else
+            asm volatile("cp.async.wait_group 0;\n" ::: "memory");
         __syncthreads();
+        if (e0 == 0) {
 #pragma unroll
-        for (int k = 0; k < kFk; ++k) {
-            float2 a[4], b[4];
+            for (int j = 0; j < kFry; ++j)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) a[i] = sa[k][4 * tx + i];
+                for (int i = 0; i < kFrx; ++i) acc[j][i] = make_float2(0.f, 0.f);
+        }
+        const int kn = n_e < kFk ? (int)n_e : kFk;
+#pragma unroll 4
+        for (int k = 0; k < kn; ++k) {
+            float2 a[kFrx], b[kFry];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) b[j] = sb[k][4 * ty + j];
+            for (int i = 0; i < kFrx; ++i) a[i] = sa[buf][k][lane + 32 * i];
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
+            for (int j = 0; j < kFry; j += 2) {
+                const float4 v = *reinterpret_cast<const float4 *>(&sb[buf][k][kFry * warp + j]);
+                b[j] = make_float2(v.x, v.y);
+                b[j + 1] = make_float2(v.z, v.w);
+            }
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
+            for (int j = 0; j < kFry; ++j)
+#pragma unroll
+                for (int i = 0; i < kFrx; ++i) {
                     acc[j][i].x = fmaf(a[i].x, b[j].x, fmaf(-a[i].y, b[j].y, acc[j][i].x));
                     acc[j][i].y = fmaf(a[i].x, b[j].y, fmaf(a[i].y, b[j].x, acc[j][i].y));
                 }
         }
-        __syncthreads();
-    }
+        __syncthreads();  // the buffer is free for the load of the step after the next
+        if (next_e == 0) {
+            // the tile's base from one bit a lane; x0 and y0 have no low bits
+            const uint64_t x0 = (tile % tiles_x) * kFx, y0 = (tile / tiles_x) * kFy;
+            uint64_t base = 0;
+            for (int i = lane; i < max(n1, n2); i += 32) {
+                if (i < n1 && (x0 >> i & 1)) base += o.xbit[i];
+                if (i < n2 && (y0 >> i & 1)) base += o.ybit[i];
+            }
+            base = (uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)base) |
+                   (uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(base >> 32)) << 32;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        const uint64_t y = y0 + 4 * ty + j;
-        if (y >= Y) continue;
+            for (int j = 0; j < kFry; ++j) {
+                const int y = kFry * warp + j;
+                if (y0 + y >= Y) break;
+                const uint64_t row = base + yoff[y];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const uint64_t x = x0 + 4 * tx + i;
-            if (x < X) psi[xoff[4 * tx + i] + yoff[4 * ty + j]] = acc[j][i];
+                for (int i = 0; i < kFrx; ++i)
+                    if (x0 + lane + 32 * i < X) psi[row + xoff[i]] = acc[j][i];
+            }
         }
+        tile = next_tile;
+        e0 = next_e;
     }
 }
 
 int launch_contract_fp32(const float2 *t1, const float2 *t2, float2 *psi, int n1, int n2, int e_bits, uint64_t ld1,
                          uint64_t ld2, const CtOut &o, cudaStream_t st)
 {
+    const LaunchCfg &cfg = ct_cfg();
+    if (!cfg.ok) return -1;
     const uint64_t X = 1ull << n1, Y = 1ull << n2;
-    const uint64_t blocks = ((X + kFx - 1) / kFx) * ((Y + kFy - 1) / kFy);
-    if (blocks > 0x7fffffffull) return -1;
-    k_contract_fp32<<<(unsigned)blocks, 256, 0, st>>>(t1, t2, psi, n1, n2, 1ull << e_bits, ld1, ld2, o);
+    const uint64_t tiles = ((X + kFx - 1) / kFx) * ((Y + kFy - 1) / kFy);
+    if (tiles > 0x7fffffffull) return -1;
+    const unsigned grid = (unsigned)std::min<uint64_t>(tiles, (uint64_t)kFocc * cfg.sms);
+    k_contract_fp32<<<grid, 256, 0, st>>>(t1, t2, psi, n1, n2, 1ull << e_bits, ld1, ld2, o);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
@@ -523,19 +594,6 @@ size_t tcgen05_scratch_bytes(int n1, int n2, int e_bits)
 {
     const uint64_t ks = ((1ull << e_bits) + 15) / 16;
     return (size_t)((1ull << n1) / 128) * ks * kCtSlab + (size_t)((1ull << n2) / 128) * ks * kCtSlab + 256;
-}
-
-const LaunchCfg &ct_cfg()
-{
-    static const LaunchCfg cfg = [] {
-        LaunchCfg c;
-        int dev = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess) return c;
-        if (cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return c;
-        c.ok = true;
-        return c;
-    }();
-    return cfg;
 }
 
 // Scales and operand images of both (whole) tensors, on st, into the scratch (the output
