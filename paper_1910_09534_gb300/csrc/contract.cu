@@ -34,6 +34,7 @@
 #include <cstring>
 
 #include "internal.h"
+#include "pdl.cuh"
 
 using namespace sycsim;
 
@@ -340,14 +341,20 @@ __device__ __forceinline__ void ct_tile(uint64_t i, uint32_t tiles_x, uint32_t t
     tx = r / gh;
 }
 
-// Largest |Re|, |Im| of n amplitudes into *out (a float's bits; non-negative floats order as
-// unsigned integers).  *out must be 0 before the launch.
-// The tensor is read as pairs of amplitudes (16 bytes), four pairs in flight per thread.
-__global__ void __launch_bounds__(256) k_absmax(const float4 *__restrict__ t, uint64_t n4, unsigned *out)
+// Largest |Re|, |Im| of each tensor's amplitudes into out[0], out[1] (a float's bits; non-negative
+// floats order as unsigned integers), which must be 0 before the launch.  The first blocks1 CTAs read
+// tensor 1, the others tensor 2, as pairs of amplitudes (16 bytes), four pairs in flight per thread.
+__global__ void __launch_bounds__(256) k_absmax(const float4 *__restrict__ t1, uint64_t n1, unsigned blocks1,
+                                                const float4 *__restrict__ t2, uint64_t n2, unsigned *out)
 {
+    pdl_launch_next();
+    const bool second = blockIdx.x >= blocks1;
+    const float4 *__restrict__ t = second ? t2 : t1;
+    const uint64_t n4 = second ? n2 : n1;
+    if (second) ++out;
     float m = 0.f;
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+    const uint64_t stride = (uint64_t)(second ? gridDim.x - blocks1 : blocks1) * blockDim.x;
+    uint64_t i = (blockIdx.x - (second ? blocks1 : 0)) * (uint64_t)blockDim.x + threadIdx.x;
     for (; i + 3 * stride < n4; i += 4 * stride) {
         float4 v[4];
 #pragma unroll
@@ -382,21 +389,27 @@ __device__ __forceinline__ void ct_split(float v, uint16_t &h, uint16_t &l)
     }
 }
 
-// Operand image of one tensor T[e][c] (c < 2^nside contiguous, e < n_e; e >= n_e reads as 0).
+// Operand images of the tensors T[e][c] (c < 2^n1 or 2^n2 contiguous, e < n_e; e >= n_e reads as 0).
+// The first 2^n1 / 128 * ks CTAs write tensor 1's, the others tensor 2's.
 // Thread = (tile, k-step, row r < 128, K half kh): 8 entanglement values of column c = 128 tile + r.
 // role 0 (A, tensor 1): slabs Re hi | Re lo | Im hi | Im lo, 128 rows x 16 each (4 KiB).
 // role 1 (B, tensor 2): slabs hi | lo, 256 rows x 16 each (8 KiB): row r = Re, row 128 + r = Im.
 template <bool BF>
-__global__ void __launch_bounds__(256) k_contract_image(const float2 *__restrict__ t, int nside, uint64_t n_e,
-                                                        uint32_t ks, const float *amax, uint8_t *img, int role)
+__global__ void __launch_bounds__(256) k_contract_image(const float2 *__restrict__ t1, int n1,
+                                                        const float2 *__restrict__ t2, int n2, uint64_t n_e,
+                                                        uint32_t ks, const float *amax, uint8_t *img1, uint8_t *img2)
 {
-    const uint64_t C = 1ull << nside;
-    const uint64_t gid = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-    if (gid >= (C / 128) * ks * 256) return;
-    const int r = (int)(gid & 127), kh = (int)((gid >> 7) & 1);
-    const uint64_t ts = gid >> 8;  // tile * ks + k-step
+    pdl_launch_next();
+    const uint64_t blocks1 = ((1ull << n1) / 128) * ks;
+    const int role = blockIdx.x >= blocks1;
+    const float2 *__restrict__ t = role ? t2 : t1;
+    uint8_t *img = role ? img2 : img1;
+    const uint64_t C = 1ull << (role ? n2 : n1);
+    const uint64_t ts = blockIdx.x - (role ? blocks1 : 0);  // tile * ks + k-step
+    const int r = (int)(threadIdx.x & 127), kh = (int)(threadIdx.x >> 7);
     const uint64_t tile = ts / ks, step = ts % ks;
-    const float sc = ldexpf(1.f, ct_shift(*amax));
+    pdl_wait();  // the maxima
+    const float sc = ldexpf(1.f, ct_shift(__ldcg(amax + role)));
     __align__(16) uint16_t rh[8], rl[8], ih[8], il[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
@@ -452,6 +465,7 @@ __global__ void __launch_bounds__(kCtThreads, 1) k_contract_tcgen05(CtArgs g, co
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
     const uint32_t tmem = tmem_base;
+    pdl_wait();
     volatile int *ab = &abort_flag;
     auto give_up = [&]() {
         *ab = 1;
@@ -559,8 +573,9 @@ __global__ void __launch_bounds__(kCtThreads, 1) k_contract_tcgen05(CtArgs g, co
                           xoff[row];
             // The accumulator into registers (128 a thread) and released: the next tile's MMAs wait for
             // the 256 KiB read, not for the stores.  The stores took 0.2-0.35 of a tile of 4-16 k-steps:
-            // 14 + 13 qubits, 256 entanglement values 550 -> 495-520 us, 14 + 14 and 64 532 -> 453,
-            // 14 + 14 and 16 (bound by the stores) 403 -> 392.
+            // 14 + 13 qubits, 256 entanglement values 550-585 -> 495-570 us (power-limited), 14 + 14 and
+            // 64 532 -> 453, 14 + 14 and 16 (bound by the stores) 403 -> 392; 14 + 14 and 1024, where the
+            // power limit decides, no difference.
             float2 v[64];
 #pragma unroll
             for (int c = 0; c < 64; c += 16) {
@@ -587,7 +602,9 @@ __global__ void __launch_bounds__(kCtThreads, 1) k_contract_tcgen05(CtArgs g, co
     if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
 }
 
-// Images, then the GEMM, all on st.  The scratch (images + maxima) belongs to the output handle
+// Maxima, images, then the GEMM, all on st, one launch each for both tensors, each resident before the
+// one ahead ends (as a launch a tensor, in turn: 8 + 9 qubits, 64 entanglement values 26 us a call, now
+// 13; 16 without the early start of the GEMM; 14 + 14 and 64 487 -> 475).  The scratch (images + maxima) belongs to the output handle
 // and is kept between calls: allocating it per call from the stream-ordered pool re-mapped it
 // every time the pool trimmed at a synchronisation, on the host's critical path.
 size_t tcgen05_scratch_bytes(int n1, int n2, int e_bits)
@@ -621,14 +638,15 @@ int prepare_tcgen05(sim_t *h, const float2 *t1, const float2 *t2, int n1, int n2
     if (cudaMemsetAsync(amax, 0, 2 * sizeof(float), st) != cudaSuccess) return -1;
     // X, Y >= 128: whole pairs of amplitudes; tensor states start 256-byte aligned
     const uint64_t n4a = X * n_e / 2, n4b = Y * n_e / 2;
-    const unsigned blocks = (unsigned)std::min<uint64_t>(8ull * cfg.sms, (n4a + 255) / 256);
-    k_absmax<<<blocks, 256, 0, st>>>(reinterpret_cast<const float4 *>(t1), n4a, reinterpret_cast<unsigned *>(amax));
+    const unsigned blocks1 = (unsigned)std::min<uint64_t>(8ull * cfg.sms, (n4a + 255) / 256);
     const unsigned blocks2 = (unsigned)std::min<uint64_t>(8ull * cfg.sms, (n4b + 255) / 256);
-    k_absmax<<<blocks2, 256, 0, st>>>(reinterpret_cast<const float4 *>(t2), n4b, reinterpret_cast<unsigned *>(amax + 1));
-    auto image = bf16 ? k_contract_image<true> : k_contract_image<false>;
-    image<<<(unsigned)((X / 128) * ks), 256, 0, st>>>(t1, n1, n_e, ks, amax, scratch, 0);
-    image<<<(unsigned)((Y / 128) * ks), 256, 0, st>>>(t2, n2, n_e, ks, amax + 1, scratch + a_bytes, 1);
-    h->launches += 4;
+    k_absmax<<<blocks1 + blocks2, 256, 0, st>>>(reinterpret_cast<const float4 *>(t1), n4a, blocks1,
+                                                reinterpret_cast<const float4 *>(t2), n4b,
+                                                reinterpret_cast<unsigned *>(amax));
+    if (launch_pdl(bf16 ? k_contract_image<true> : k_contract_image<false>, (unsigned)((X / 128 + Y / 128) * ks), 256, 0,
+                   st, t1, n1, t2, n2, n_e, ks, (const float *)amax, scratch, scratch + a_bytes) != cudaSuccess)
+        return -1;
+    h->launches += 2;
     *aimg = scratch;
     *bimg = scratch + a_bytes;
     *amax_out = amax;
@@ -660,9 +678,10 @@ int launch_gemm_tcgen05(sim_t *h, const uint8_t *aimg, const uint8_t *bimg, cons
     g.bf16 = bf16 ? 1 : 0;
     const uint64_t grid = std::min<uint64_t>((uint64_t)g.tiles_x * g.tiles_y, (uint64_t)cfg.sms);
     const int ps = prof_begin(h, SIM_PROF_CONTRACT, 8.0 * (double)X * (double)Y * (double)n_e, st);
-    k_contract_tcgen05<<<(unsigned)grid, kCtThreads, kCtStages * kCtStage, st>>>(g, o);
+    const cudaError_t e =
+        launch_pdl(k_contract_tcgen05, (unsigned)grid, kCtThreads, (size_t)kCtStages * kCtStage, st, g, o);
     prof_end(h, ps, st);
-    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+    return e == cudaSuccess && cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
 }  // namespace
