@@ -369,14 +369,14 @@ def serving_run(count: int, device: int, rate_hz: float = 0.0, precision: str = 
            f"Poisson at {rate_hz:g} circuits/s (last arrival at {arrivals[-1]:.2f} s)")
     if fp32:
         arith = ("fp32 on CUDA cores (k_max 5 up to 24 qubits, 4 above, in a chosen layout above 20 "
-                 "qubits; circuits of <= 20 qubits packed one per CTA, k_max 5)")
+                 "qubits; circuits of <= 20 qubits packed one per cluster, k_max 5)")
         front = ("circuits of >= 26 qubits (from 22 where the autotuner measured it faster) whose first "
                  "2 crossings of the chosen bipartition leave >= 10% of the gates in front run them as "
                  "two tensors and one FP32 contraction on CUDA cores; the one-at-a-time path runs every "
                  "circuit plainly")
     else:
         arith = ("fp16x3_tmem (k_max 6 in a chosen layout above 20 qubits; circuits of <= 20 "
-                 "qubits packed one per CTA in FP32, k_max 5)")
+                 "qubits packed one per cluster in FP32, k_max 5)")
         front = ("circuits of >= 26 qubits whose first 5 crossings of the chosen bipartition leave >= 30% "
                  "of the gates in front run them as two tensors and one tcgen05 contraction; the "
                  "one-at-a-time path runs every circuit plainly")

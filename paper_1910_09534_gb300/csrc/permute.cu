@@ -8,9 +8,11 @@
 //  * transpositions between two bits >= LB swap whole tiles (tile tau <-> tile sigma(tau));
 //  * transpositions with one bit < LB make the other bit a "row" bit of the tile;
 //  * transpositions inside [0, LB) act within the tile.
-// A CTA loads a tile pair (2^(LB+q) amplitudes each, rows of 2^LB contiguous amplitudes) with
-// 16-byte loads, permutes it in shared memory and writes it back with coalesced 16-byte stores.  Tiles that
-// nothing moves are skipped, so a single high-bit swap touches half of the state.
+// A tile (or tile pair) of 2^(LB+q) amplitudes, rows of 2^LB contiguous amplitudes, is brought into
+// shared memory, permuted there and written back.  Tiles that nothing moves are skipped, so a single
+// high-bit swap touches half of the state.  Three kernels, chosen in launch_involution: a tensor-map
+// pipeline (k_permute_tma), a bulk copy a row where rows are long (k_permute_tile_bulk), 16-byte loads
+// and stores for the small states and the geometries left (k_permute_pass).
 #include <cuda.h>
 #include <cuda_runtime.h>
 
@@ -265,7 +267,7 @@ __global__ void __launch_bounds__(256) k_permute_tile_bulk(PermGeom g, int *err)
 // transpositions) or, without any, one tile of twice the size.
 //  * warp 0, producer: its lanes look at up to 32 tiles at a time (the partner's base, whether anything
 //    moves); the tiles that do are loaded into the stage ring, a copy a lane (bytes counted on an mbarrier);
-//  * warps 2-17, swappers, four groups of 128 threads, a stage to each in turn: 16 amplitudes a
+//  * warps 2-9, swappers, two groups of 128 threads, a stage to each in turn: 16 amplitudes a
 //    thread, read where the in-tile involution sig puts them from, a barrier among the group, written
 //    to their places.  The maps are XOR-linear: a thread part computed once, an iteration part from
 //    the parameters;

@@ -584,7 +584,9 @@ namespace {
 
 // Estimated time of one fused pass over 2^30 amplitudes (ms) on the kernel a block of k targets at
 // physical bits tpos takes, from CUDA-event timings of each kernel path on GB300; the layout search
-// only compares sums of these.
+// only compares sums of these.  The entries for FP32 blocks of 4-6 qubits and tcgen05 blocks of 4 and 5
+// stem from earlier forms of those kernels (k = 5 in FP32 takes 5.7 ms now with any targets): a plan's
+// layout, and with it the last bits of its results, stays what it was.
 double pass_ms(int k, const int *tpos, int precision)
 {
     int low4 = 0, low5 = 0;
