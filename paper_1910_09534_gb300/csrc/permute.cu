@@ -279,8 +279,8 @@ __global__ void __launch_bounds__(256) k_permute_tile_bulk(PermGeom g, int *err)
 // 737 -> 673, 3 high pairs 587 -> 584; random permutations (two passes) of 2^29 3.2-4.5 -> 2.70-2.93 ms,
 // of 2^24 127-141 -> 85-94 us.  The kernel before, one CTA a tile pair and 4 amplitudes a thread, was
 // issue-bound (76 %) on setting up its maps.
-// Every wait is bounded by %globaltimer: on a timeout the kernel records the failure, every role
-// leaves, and the CTA waits (again bounded) for its own copies.
+// Every wait is bounded by %globaltimer, from when the kernels before have ended: on a timeout the
+// kernel records the failure, every role leaves, and the producer waits (again bounded) for its copies.
 constexpr int kPtRing = 98304;                    // bytes of stages (64 KiB: 10-20 % slower); a stage is one tile or a tile pair
 constexpr int kPtMaxStages = 16;
 constexpr int kPtGroups = 2;                      // swapper groups, a stage to each in turn
@@ -365,6 +365,7 @@ __global__ void __launch_bounds__(kPtThreads, 2) k_permute_tma(const __grid_cons
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     __syncthreads();
+    pdl_wait();  // every role: the waits' time limits count from here, not from an early start
     volatile int *ab = &abort_flag;
     auto give_up = [&]() {
         *ab = 1;
@@ -398,7 +399,6 @@ __global__ void __launch_bounds__(kPtThreads, 2) k_permute_tma(const __grid_cons
 
     if (warp == 0) {
         // ---------------- producer ----------------
-        pdl_wait();
         uint32_t it = 0;
         bool stop = false;
         for (uint64_t c0 = (uint64_t)blockIdx.x * g.per; c0 < g.n_tiles && !stop; c0 += (uint64_t)gridDim.x * g.per) {
@@ -448,15 +448,14 @@ __global__ void __launch_bounds__(kPtThreads, 2) k_permute_tma(const __grid_cons
                 ntile_of[e % S] = 0;
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(perm_smem(&full[e % S])) : "memory");
             }
-            if (marks < (uint32_t)kPtGroups) {
-                // given up: no copy may still be writing a stage when the CTA leaves.  (Otherwise the
-                // storer has waited for every one of them, and the end marks have moved barriers on.)
-                give_up();
-                for (uint32_t j = it + marks > S ? it + marks - S : 0; j < it; ++j) {
-                    const uint64_t t0 = perm_now_ns();
-                    while (!perm_try(perm_smem(&full[j % S]), (j / S) & 1, 20000) &&
-                           perm_now_ns() - t0 <= kPtWaitNs) {
-                    }
+            if (marks < (uint32_t)kPtGroups) give_up();
+            // No copy may still be writing a stage when the CTA leaves, whichever role gave up and when
+            // (the storer and the swappers, which otherwise wait for every copy, may already be gone).
+            // The barriers of items older than these have been moved on by later copies or end marks,
+            // which waited until those items had been stored.
+            for (uint32_t j = it + marks > S ? it + marks - S : 0; j < it; ++j) {
+                const uint64_t t0 = perm_now_ns();
+                while (!perm_try(perm_smem(&full[j % S]), (j / S) & 1, 20000) && perm_now_ns() - t0 <= kPtWaitNs) {
                 }
             }
         }
