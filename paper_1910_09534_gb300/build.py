@@ -32,7 +32,7 @@ def nvcc() -> str:
 
 
 def _headers_mtime() -> float:
-    paths = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".h")]
+    paths = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
     paths.append(os.path.join(INCLUDE, "sycsim.h"))
     return max(os.path.getmtime(p) for p in paths)
 
