@@ -14,6 +14,12 @@
 
 #include <utility>
 
+// The runtime call that launches a kernel in clusters, which a device may refuse: a test compiles
+// one that refuses in its place.
+#ifndef SYCSIM_CLUSTER_LAUNCH
+#define SYCSIM_CLUSTER_LAUNCH cudaLaunchKernelEx
+#endif
+
 namespace sycsim {
 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }

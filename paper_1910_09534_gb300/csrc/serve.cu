@@ -40,6 +40,7 @@
 
 #include "cluster_run.cuh"
 #include "internal.h"
+#include "pdl.cuh"
 
 namespace sycsim {
 namespace {
@@ -239,6 +240,7 @@ struct Req {
     bool contracted = false;
     Clock::time_point t_submit, t_done;
     int status = 1;  // 1 pending, 0 ok, < 0 error
+    std::string why;  // of an error, if known
     double norm = 0.0, s2 = 0.0;
     int bypassed = 0;
     std::shared_ptr<GraphEntry> graph;  // repeated circuit: replay this entry's graph
@@ -305,13 +307,14 @@ struct srv_s {
     // the packed jobs' queue (see k_packed_worker): ring entries in mapped pinned memory, the
     // published count beside them, the claim counter in device memory, up to two workers in flight
     QSlot *ring = nullptr, *d_ring = nullptr;
-    uint32_t *ctl = nullptr, *d_ctl = nullptr;  // ctl[0]: published count
+    uint32_t *ctl = nullptr, *d_ctl = nullptr;  // ctl[0]: published count; ctl[16]: source of a new claim count
     uint32_t *d_head = nullptr;
     uint64_t next_index = 0, published = 0, retired = 0;
     cudaStream_t wst[2] = {nullptr, nullptr};
     cudaEvent_t wev[2] = {nullptr, nullptr};
     int max_ctas = 8;  // widest cluster of the workers: 16 where the device can place one
     int wclusters[2] = {0, 0};  // clusters of a worker still running (0: none)
+    bool no_workers = false;    // the claim counter could not be moved on: no worker may start any more
     int sms = 0;
     double *h_results = nullptr;  // pinned ring of result pairs for unpacked requests
     std::thread worker;
@@ -605,6 +608,32 @@ int copy_out_packed(Batch &B)
     return rc;
 }
 
+// With no worker running, what is published and not done has not been claimed: fail those units, the
+// reason kept for their waiters, and set the claim counter past them for workers to come (scheduler
+// thread, lock held).
+void fail_published(srv_t *s, cudaError_t e)
+{
+    if (!s->no_workers) {
+        s->ctl[16] = (uint32_t)s->published;
+        if (cudaMemcpyAsync(s->d_head, s->ctl + 16, sizeof(uint32_t), cudaMemcpyHostToDevice, s->wst[0]) != cudaSuccess ||
+            cudaStreamSynchronize(s->wst[0]) != cudaSuccess)
+            s->no_workers = true;  // a worker would claim jobs whose memory is given back here
+    }
+    for (auto &B : s->batches) {
+        if (B.state != Batch::Running) continue;
+        cudaFreeAsync(B.d_mem, B.st);
+        B.d_mem = nullptr;
+        for (auto &r : B.jobs) {
+            r->why = std::string("worker launch: ") + cudaGetErrorString(e);
+            finish(s, r, SIM_E_CUDA, 0.0, 0.0);
+        }
+        s->retired += B.jobs.size();
+        B.jobs.clear();
+        B.state = Batch::Free;
+    }
+    cudaGetLastError();
+}
+
 // Jobs published and not yet seen done; launch a worker when they outnumber the clusters of the
 // workers still running (scheduler thread, lock held).
 void manage_workers(srv_t *s, uint64_t not_done, bool *progressed)
@@ -615,37 +644,45 @@ void manage_workers(srv_t *s, uint64_t not_done, bool *progressed)
         running += s->wclusters[w];
     }
     if (not_done <= (uint64_t)running) return;
-    for (int w = 0; w < 2; w++)
-        if (!s->wclusters[w]) {
-            // Clusters of 16 finish a circuit sooner (16 of 18 qubits in 8.6 -> 4.8 ms, one in 1.41 -> 0.96;
-            // at 12 qubits no difference), but wait longer for 16 free SMs of one group beside the large
-            // lane's kernels: 8 then.  300 circuits of 16-30 qubits at once, 16 always / by this rule / 8 always:
-            // 152 circuits/s each; p50 from arrival 420 / 430 / 455 ms, inside the server 210-250 / 190 / 130.
-            int ctas = s->max_ctas;
-            for (auto &r : s->slot_req)
-                if (r) ctas = 8;
-            const int clusters = (int)std::min<uint64_t>(not_done - running, (uint64_t)(2 * s->sms / ctas));
-            cudaLaunchAttribute attr{};
-            attr.id = cudaLaunchAttributeClusterDimension;
-            attr.val.clusterDim.x = ctas;
-            attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
-            cudaLaunchConfig_t cfg{};
-            cfg.gridDim = dim3(clusters * ctas);
-            cfg.blockDim = dim3(kClThreads);
-            cfg.stream = s->wst[w];
-            cfg.attrs = &attr;
-            cfg.numAttrs = 1;
-            if (cudaLaunchKernelEx(&cfg, k_packed_worker, (const uint32_t *)s->d_ctl, s->d_ring, s->d_head) !=
-                cudaSuccess) {
-                cudaGetLastError();
-                s->max_ctas = 8;  // tried again on the scheduler's next turn
-                return;
-            }
-            if (cudaEventRecord(s->wev[w], s->wst[w]) != cudaSuccess) return;
-            s->wclusters[w] = clusters;
-            *progressed = true;
-            return;
-        }
+    int w = 0;
+    while (w < 2 && s->wclusters[w]) ++w;
+    if (w == 2) return;
+    // Clusters of 16 finish a circuit sooner (16 of 18 qubits in 8.6 -> 4.8 ms, one in 1.41 -> 0.96;
+    // at 12 qubits no difference), but wait longer for 16 free SMs of one group beside the large
+    // lane's kernels: 8 then.  300 circuits of 16-30 qubits at once, 16 always / by this rule / 8 always:
+    // 152 circuits/s each; p50 from arrival 420 / 430 / 455 ms, inside the server 210-250 / 190 / 130.
+    int ctas = s->max_ctas;
+    for (auto &r : s->slot_req)
+        if (r) ctas = 8;
+    cudaError_t e = cudaErrorUnknown;
+    int clusters = 0;
+    while (!s->no_workers) {
+        clusters = (int)std::min<uint64_t>(not_done - running, (uint64_t)(2 * s->sms / ctas));
+        cudaLaunchAttribute attr{};
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = ctas;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(clusters * ctas);
+        cfg.blockDim = dim3(kClThreads);
+        cfg.stream = s->wst[w];
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        e = SYCSIM_CLUSTER_LAUNCH(&cfg, k_packed_worker, (const uint32_t *)s->d_ctl, s->d_ring, s->d_head);
+        if (e == cudaSuccess || ctas <= 8) break;
+        cudaGetLastError();
+        ctas = s->max_ctas = 8;  // the wider one was refused
+    }
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        if (running > 0) return;  // the workers there are go through the jobs
+        fail_published(s, e);
+    } else if (cudaEventRecord(s->wev[w], s->wst[w]) == cudaSuccess) {
+        s->wclusters[w] = clusters;
+    } else {
+        cudaStreamSynchronize(s->wst[w]);  // no event to ask: the worker leaves when it runs out of jobs
+    }
+    *progressed = true;
 }
 
 // Replay a repeated circuit's graph on its entry's handle (scheduler thread, lock held): reset,
@@ -1254,7 +1291,8 @@ int srv_wait(srv_t *s, uint64_t ticket, int timeout_ms, double *norm, double *su
     if (r->ev) cudaEventDestroy(r->ev);
     r->ev = nullptr;
     s->reqs.erase(it);
-    if (r->status != SIM_OK) return srv_fail(s, r->status, "srv_wait: request failed");
+    if (r->status != SIM_OK)
+        return srv_fail(s, r->status, "srv_wait: request failed%s%s", r->why.empty() ? "" : ": ", r->why.c_str());
     if (norm) *norm = r->norm;
     if (sum_p2_scaled) *sum_p2_scaled = std::ldexp(r->s2, r->n);
     if (latency_ms) *latency_ms = std::chrono::duration<double, std::milli>(r->t_done - r->t_submit).count();
