@@ -284,7 +284,8 @@ int launch_apply_fp32(sim_t *h, float2 *psi, int nbits, int k, const int *tpos,
 
 // ---- plan_cluster.cu: a whole plan on a small state in a few launches (FP32) ----
 bool plan_cluster_eligible(int n, int nblocks, int max_k);
-// block i: k[i] targets tpos[i] (ascending physical bits), matrix mats[i]; *launches: kernels launched
+// block i: k[i] targets tpos[i] (ascending physical bits), matrix mats[i]; *launches: kernels launched.
+// Returns how many blocks are enqueued, in order: fewer than nblocks if the device refuses a cluster
 int launch_plan_cluster(float2 *psi, int n, int nblocks, const int *k, const int *const *tpos,
                         const float2 *const *mats, cudaStream_t st, int *launches);
 

@@ -68,7 +68,7 @@ cudaError_t launch_cluster(void (*kern)(P...), unsigned grid, unsigned cluster, 
     cfg.stream = st;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+    return SYCSIM_CLUSTER_LAUNCH(&cfg, kern, std::forward<A>(args)...);
 }
 
 }  // namespace sycsim

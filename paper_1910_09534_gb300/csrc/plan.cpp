@@ -932,8 +932,10 @@ int sim_apply_plan(sim_t *h, const sim_plan_t *p)
         total += (pb.bytes + 255) & ~size_t(255);
         max_k = std::max(max_k, pb.k);
     }
+    size_t first = 0;  // blocks before this one are enqueued
     if (p->precision == SIM_FP32 && plan_cluster_eligible(h->n, (int)nb, max_k)) {
-        // a small state: its blocks are applied by one cluster, many a launch
+        // a small state: its blocks are applied by one cluster, many a launch (no operands to stage:
+        // max_k <= 5); where the device refuses the cluster, by the launches below
         std::vector<int> ks(nb);
         std::vector<const int *> tp(nb);
         std::vector<const float2 *> ms(nb);
@@ -944,13 +946,10 @@ int sim_apply_plan(sim_t *h, const sim_plan_t *p)
         }
         const int ps = prof_begin(h, SIM_PROF_APPLY, 16.0 * std::ldexp((double)nb, h->n), h->stream);
         int launches = 0;
-        const int rc = launch_plan_cluster(h->d_state, h->n, (int)nb, ks.data(), tp.data(), ms.data(), h->stream,
-                                           &launches);
+        first = (size_t)launch_plan_cluster(h->d_state, h->n, (int)nb, ks.data(), tp.data(), ms.data(), h->stream,
+                                            &launches);
         prof_end(h, ps, h->stream);
-        h->launches += launches > 1 ? launches - 1 : 0;  // prof_begin counted one
-        h->red_blocks = 0;
-        return rc == 0 ? SIM_OK
-                       : fail(h, SIM_E_CUDA, "sim_apply_plan: launch failed: %s", cudaGetErrorString(cudaGetLastError()));
+        h->launches += launches - 1;  // prof_begin counted one
     }
     char *d_ops = nullptr;
     int slot = -1;
@@ -988,7 +987,7 @@ int sim_apply_plan(sim_t *h, const sim_plan_t *p)
     // own and was never handed out: nobody else can write it in between)
     const bool fuse = h->own_state && !h->state_exposed;
     int red_grid = 0;
-    for (size_t i = 0; i < nb; i++) {
+    for (size_t i = first; i < nb; i++) {
         const Prep &pb = prep[i];
         const bool last = i + 1 == nb;
         const int ps = prof_begin(h, SIM_PROF_APPLY, pass_bytes, h->stream);

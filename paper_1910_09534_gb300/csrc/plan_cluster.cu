@@ -64,7 +64,7 @@ int launch_plan_cluster(float2 *psi, int n, int nblocks, const int *k, const int
 {
     static thread_local PlanTable t;
     *launches = 0;
-    const int ctas = plan_ctas();
+    int ctas = plan_ctas();
     for (int i = 0; i < nblocks;) {
         int c = 0;
         uint32_t off = 0;
@@ -76,11 +76,19 @@ int launch_plan_cluster(float2 *psi, int n, int nblocks, const int *k, const int
             std::memcpy(t.mats + off, mats[i], sizeof(float2) << (2 * k[i]));
             off += 1u << (2 * k[i]);
         }
-        if (launch_cluster(k_plan_cluster, ctas, ctas, kClThreads, 0, st, psi, n, c, t) != cudaSuccess)
-            return -1;
+        cudaError_t e = launch_cluster(k_plan_cluster, ctas, ctas, kClThreads, 0, st, psi, n, c, t);
+        if (e != cudaSuccess && ctas > 8) {  // the occupancy query's answer does not bind the launch
+            cudaGetLastError();
+            ctas = 8;
+            e = launch_cluster(k_plan_cluster, ctas, ctas, kClThreads, 0, st, psi, n, c, t);
+        }
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return i - c;
+        }
         ++*launches;
     }
-    return 0;
+    return nblocks;
 }
 
 }  // namespace sycsim

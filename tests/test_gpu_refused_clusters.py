@@ -2,7 +2,8 @@
 
 Packed serving goes on with clusters of 8 where wider ones are refused, with the same bits; where those
 are refused too, the requests end with an error that names the reason, other circuits are served
-still, and the server can be destroyed.
+still, and the server can be destroyed.  Plans go on with clusters of 8, and where those are refused,
+at the first launch or a later one, with one launch a block: the same bits.
 """
 import os
 import subprocess
@@ -75,3 +76,25 @@ def test_packed_serving_reports_a_refused_launch(refusing_lib, after):
     assert all("worker launch: too many resources" in x for x in out.splitlines() if x.startswith("error"))
     if after == 0:
         assert out.count("error") == 5
+
+
+PLAN = """
+for n, kmax in ((6, 3), (12, 4), (14, 5), (16, 5)):
+    c = si.sycamore_circuit(si.near_square_grid(n), 8, seed=n)
+    p = pkg.sim_plan_create(n, pkg.gates_array(c), kmax=kmax)
+    h = pkg.sim_create(n)
+    pkg.sim_apply_plan(h, p)
+    out = pkg.sim_amplitudes(h)
+    pkg.sim_sync(h)
+    print(n, hashlib.sha256(out.tobytes()).hexdigest(), abs(pkg.sim_reduce(h)[0] - 1) < 1e-5)
+    pkg.sim_destroy(h)
+    pkg.sim_plan_destroy(p)
+"""
+
+
+def test_plans_go_on_where_clusters_are_refused(refusing_lib):
+    want = run(refusing_lib, PLAN, 16)
+    assert want.count("True") == 4
+    assert run(refusing_lib, PLAN, 8) == want
+    for after in (0, 1, 2, 3):
+        assert run(refusing_lib, PLAN, 0, after) == want
