@@ -69,7 +69,6 @@ __device__ __forceinline__ uint64_t insert_zero_bits_p(uint64_t x, const int *po
 __global__ void __launch_bounds__(256) k_permute_pass(PermGeom g)
 {
     extern __shared__ float2 sm[];
-    pdl_launch_next();
     pdl_wait();
     const uint64_t baseA = insert_zero_bits_p((uint64_t)blockIdx.x << g.LB, g.rowpos, g.q);
     uint64_t baseB = baseA;
@@ -152,6 +151,9 @@ __device__ __forceinline__ uint64_t perm_now_ns()
 // amplitudes in place with 0-3 row bits 606-630 / 660-685, with 4, 5 (rows of 256-512 bytes) 727, 737 /
 // 670-690; tile pairs with no row bits, 2^30 1225 / 1322, 2^28 575 / 590; pairs of 2^11 with rows of 1 KiB 687
 // / 740, of 2^10 809 / 690, with shorter rows 973-1286 / 690-711.
+// It lets no kernel start early, nor does k_permute_pass: a CTA a tile, most of which only find that
+// nothing moves, and each paid for the trigger (bits 26 and 27 of 2^28 amplitudes: 497 us, without 400; of
+// 2^24 21.9, 17.6).
 // The only wait (the copies' mbarrier) is bounded by %globaltimer: on a timeout the CTA records the
 // failure, writes nothing back and waits (again bounded) for its copies before leaving.
 __global__ void __launch_bounds__(256) k_permute_tile_bulk(PermGeom g, int *err)
@@ -160,7 +162,6 @@ __global__ void __launch_bounds__(256) k_permute_tile_bulk(PermGeom g, int *err)
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t p_it[64], sig_it[64];  // the iteration part of p, and its image under sig
     __shared__ int ok;
-    pdl_launch_next();
     const int nloc = g.LB + g.q, T = 1 << nloc;
     const uint32_t row_bytes = 8u << g.LB;
     const uint64_t base = insert_zero_bits_p((uint64_t)blockIdx.x << g.LB, g.rowpos, g.q);

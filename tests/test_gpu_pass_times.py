@@ -1,0 +1,61 @@
+"""GPU: passes that an early start of the next kernel once slowed down, held against other work of the
+same run: a device copy or fill of the same bytes, or the same blocks on half of the state.  Each
+bound lies between the two times measured with and without the fault, named beside it."""
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def pkg():
+    from paper_1910_09534_gb300 import build
+    build.build()
+    import paper_1910_09534_gb300 as p
+    return p
+
+
+@pytest.fixture(scope="module")
+def stream():
+    import torch
+    return torch.cuda.Stream()
+
+
+def us(stream, call, reps):
+    """Microseconds a call, back to back on the stream: the best of 7 runs."""
+    import torch
+    with torch.cuda.stream(stream):
+        call()
+        best = float("inf")
+        for _ in range(7):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda.synchronize()
+            a.record(stream)
+            for _ in range(reps):
+                call()
+            b.record(stream)
+            b.synchronize()
+            best = min(best, a.elapsed_time(b) * 1e3 / reps)
+    return best
+
+
+def handle(pkg, stream, n):
+    import torch
+    buf = torch.zeros(2 << n, dtype=torch.float32, device="cuda")
+    torch.cuda.synchronize()
+    h = pkg.sim_create(n, stream=stream.cuda_stream, ext_state=buf.data_ptr(), ext_bytes=8 << n)
+    pkg.sim_sync(h)
+    return h, buf
+
+
+def test_swap_of_two_high_bits(pkg, stream):
+    # half of 2^28 amplitudes move: 1.25 times a copy of that half, 1.55 with the trigger in every CTA
+    n = 28
+    h, buf = handle(pkg, stream, n)
+    half = len(buf) // 2
+    perms = [list(range(n - 2)) + [n - 1, n - 2], list(range(n))]  # there and back
+    try:
+        t = us(stream, lambda: [pkg.sim_permute(h, p) for p in perms], 5) / 2
+        copy = us(stream, lambda: buf[:half].copy_(buf[half:]), 10)
+        assert t < 1.4 * copy, (t, copy)
+    finally:
+        pkg.sim_destroy(h)
