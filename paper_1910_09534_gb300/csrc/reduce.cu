@@ -144,9 +144,11 @@ __global__ void k_gather_region(float2 *base, uint64_t lo, uint64_t hi, float2 *
 }
 
 // |phys> into a state of 2 n4 amplitudes: zeros and the one, in one launch and one write of the state.
+// Bound by the writes.  Four 16-byte stores a thread and as many CTAs as that takes: 278 us for 2^28
+// amplitudes (a memset 284; 8 CTAs an SM looping over the state 325), 552 for 2^29 (557; 649), 18.4 for
+// 2^24 (24; 21).  No trigger for the next launch: it would cost each of these short CTAs.
 __global__ void __launch_bounds__(256) k_reset(float4 *psi4, uint64_t n4, uint64_t phys)
 {
-    pdl_launch_next();
     pdl_wait();
     const uint64_t one = phys >> 1;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (uint64_t)gridDim.x * blockDim.x) {
@@ -276,8 +278,7 @@ int launch_reset(float2 *psi, uint64_t amps, uint64_t phys, cudaStream_t st)
 {
     if (phys >= amps) return -1;
     const uint64_t n4 = amps / 2;
-    const uint64_t need = (n4 + 1023) / 1024;  // four 16-byte stores a thread, up to 8 CTAs an SM
-    const unsigned grid = (unsigned)(need < 152 * 8 ? need : 152 * 8);
+    const unsigned grid = (unsigned)((n4 + 1023) / 1024);
     return launch_pdl(k_reset, grid, 256, 0, st, reinterpret_cast<float4 *>(psi), n4, phys) == cudaSuccess ? 0 : -1;
 }
 

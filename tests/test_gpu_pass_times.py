@@ -59,3 +59,15 @@ def test_swap_of_two_high_bits(pkg, stream):
         assert t < 1.4 * copy, (t, copy)
     finally:
         pkg.sim_destroy(h)
+
+
+@pytest.mark.parametrize("n", [26, 28])
+def test_reset(pkg, stream, n):
+    # every amplitude written once: 0.98-1.00 times a fill of the same memory, 1.12-1.15 with too few CTAs
+    h, buf = handle(pkg, stream, n)
+    try:
+        t = us(stream, lambda: pkg.sim_reset(h), 10)
+        fill = us(stream, lambda: buf.zero_(), 10)
+        assert t < 1.07 * fill, (t, fill)
+    finally:
+        pkg.sim_destroy(h)
