@@ -24,6 +24,9 @@
 // The matrix (FP32, complex64) is a kernel parameter for k <= 5: up to k = 4 (2 KiB) the FMAs read it
 // straight from the constant bank; k = 5, 6 (8, 32 KiB, more than the constant cache keeps) are
 // copied to shared memory once per CTA, k = 6 from device memory.
+//
+// Early starts: reg and direct do not trigger the next launch, rtile does at its last tile (pdl.cuh has
+// the figures; rtile on 18-19 qubits, trigger at the start / at the last tile: 76, 115 / 62, 96 us a replay).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -159,7 +162,6 @@ template <int K>
 __global__ void __launch_bounds__(256, 4) k_apply_direct(DirectGeom g, MatP<K> M)
 {
     constexpr int D = 1 << K;
-    pdl_launch_next();
     const uint64_t gi = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (gi >= g.n_groups) return;
     pdl_wait();
@@ -180,7 +182,7 @@ __global__ void __launch_bounds__(tiled_threads(K), tiled_min_blocks(K)) k_apply
     extern __shared__ float2 smem[];
     float2 *tile = smem;
     float2 *msm = smem + ((size_t)D << g.F);
-    pdl_launch_next();
+    if constexpr (K <= 4) pdl_launch_next();  // one or two CTAs; K = 5 took 5 % longer with it
     if constexpr (kSmemMat) stage_matrix<K>(msm, M.p);
 
     const uint32_t tid = threadIdx.x;
@@ -361,7 +363,6 @@ __global__ void __launch_bounds__(256, reg_min_blocks(K)) k_apply_reg(RegGeom g,
 {
     constexpr int D = 1 << K;
     __shared__ float2 xch[kLow ? 8 * 32 * D : 1];
-    pdl_launch_next();
     pdl_wait();
     const int lane = threadIdx.x & 31;
     const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
@@ -521,7 +522,6 @@ __global__ void __launch_bounds__(rtile_threads(K), rtile_min_blocks(K))
     __shared__ uint64_t ioff[NI];
     __shared__ uint32_t isw[NI];
     const int tid = threadIdx.x, lane = tid & 31, rg = tid >> 5;
-    pdl_launch_next();
     {
         const float2 *src;
         if constexpr (K == 6) {
@@ -578,7 +578,10 @@ __global__ void __launch_bounds__(rtile_threads(K), rtile_min_blocks(K))
     for (uint64_t t = blockIdx.x; t < g.n_tiles; t += gridDim.x, buf ^= 1) {
         cp_async_wait_all();
         __syncthreads();  // the tile is here; the other buffer's results have been read out
-        if (t + gridDim.x < g.n_tiles) fetch(t + gridDim.x, buf ^ 1);
+        if (t + gridDim.x < g.n_tiles)
+            fetch(t + gridDim.x, buf ^ 1);
+        else
+            pdl_launch_next();
         uint8_t *sb = sm + buf * T * 8;
         float2 y[RT][2];
 #pragma unroll

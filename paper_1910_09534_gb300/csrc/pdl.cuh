@@ -24,7 +24,14 @@ namespace sycsim {
 
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
-// The next kernel of the stream may start, once every CTA of this one has got here or left.
+// The next kernel of the stream may start, once every CTA of this one has got here or left.  A kernel
+// of which several CTAs fit on an SM had better not call it, or at its last tile: the next one's CTAs
+// are put where there is room, several on the SMs that are idle or done first, and share those while
+// others stand empty.  Without it the next launch still reaches the SMs while this kernel drains.
+// Replays of plans of FP32 blocks, us, launched the ordinary way / trigger at the start / at the last tile
+// / none: 4 qubits a block on 19 qubits (128 CTAs a pass) 90 / 134 / 84 / 82, on 20 137 / 171 / 164 / 125,
+// on 22 349 / 370 / 368 / 340; 3 qubits on 18 76 / 98 / 82 / 62, on 20 166 / 148 / 149 / 146.  A kernel of very
+// many short CTAs pays for the instruction itself (permute.cu).
 __device__ __forceinline__ void pdl_launch_next() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 
 // Whether a tensor-core pass over 2^nbits amplitudes lets the next one start early (the tcgen05 kernels

@@ -71,3 +71,24 @@ def test_reset(pkg, stream, n):
         assert t < 1.07 * fill, (t, fill)
     finally:
         pkg.sim_destroy(h)
+
+
+@pytest.mark.parametrize("kmax, n", [(3, 18), (4, 19)])
+def test_fp32_blocks_below_one_wave(pkg, stream, kmax, n):
+    # the same blocks on n - 1 and n qubits, both less than one CTA an SM: 1.1 times the time, 1.4-1.5
+    # where the passes crowd on the SMs that the pass before has left idle
+    import syc_inputs as si
+    gates = pkg.gates_array(si.sycamore_circuit(si.near_square_grid(n - 1), 12, seed=n))
+    t = []
+    for m in (n - 1, n):
+        h, buf = handle(pkg, stream, m)
+        p = pkg.sim_plan_create(m, gates, kmax=kmax)
+        try:
+            pkg.sim_reset(h)
+            g = pkg.sim_graph_create(h, p)
+            t.append(us(stream, lambda: pkg.sim_graph_launch(h, g), 20))
+            pkg.sim_graph_destroy(g)
+        finally:
+            pkg.sim_plan_destroy(p)
+            pkg.sim_destroy(h)
+    assert t[1] < 1.28 * t[0], t
