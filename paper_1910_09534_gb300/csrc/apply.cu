@@ -6,7 +6,7 @@
 // Each group is replaced by M times itself.  One pass reads and writes every amplitude
 // once: 16 bytes per amplitude of HBM traffic, 8 * 2^k - 2 real flops per amplitude.
 //
-// Four kernels:
+// Five kernels:
 //  * reg (default for k <= 4, n >= k + 5) -- see the comment above k_apply_reg: persistent warps,
 //    register-resident groups, an exchange through the warp's own shared memory for targets
 //    below bit 5.
@@ -15,7 +15,8 @@
 //  * direct -- every target >= 5: thread = group; the 32 threads of a warp take 32
 //    consecutive groups, so each member load/store is one contiguous 256-byte run.
 //    Amplitudes go straight to registers; no shared memory.  Used for k <= 3.
-//  * tiled -- the smallest states: a CTA stages a tile of 2^(F+k) amplitudes (2^h rows of
+//  * cta -- k = 5 on at most 10 qubits: one CTA, several threads to a group's rows.
+//  * tiled -- the smallest states otherwise: a CTA stages a tile of 2^(F+k) amplitudes (2^h rows of
 //    2^m contiguous amplitudes, the rows indexed by the h targets >= m) through shared
 //    memory with coalesced loads, each of its 2^F threads applies M to one group, and
 //    the tile is written back.  An XOR swizzle maps the low target bits onto free bits
@@ -34,6 +35,7 @@
 #include <cstring>
 #include <type_traits>
 
+#include "cluster_run.cuh"
 #include "internal.h"
 #include "pdl.cuh"
 
@@ -155,8 +157,8 @@ __device__ __forceinline__ void stage_matrix(float2 *sm, const float2 *gm)
 }
 
 // Occupancy targets (CTAs per SM) that bound the register count of each width.
-constexpr int tiled_threads(int k) { return k <= 4 ? 256 : (k == 5 ? 128 : 64); }
-constexpr int tiled_min_blocks(int k) { return k <= 3 ? 4 : (k <= 5 ? 2 : 4); }
+constexpr int tiled_threads(int k) { return k <= 4 ? 256 : 64; }
+constexpr int tiled_min_blocks(int k) { return k == 4 ? 2 : 4; }
 
 template <int K>
 __global__ void __launch_bounds__(256, 4) k_apply_direct(DirectGeom g, MatP<K> M)
@@ -182,7 +184,7 @@ __global__ void __launch_bounds__(tiled_threads(K), tiled_min_blocks(K)) k_apply
     extern __shared__ float2 smem[];
     float2 *tile = smem;
     float2 *msm = smem + ((size_t)D << g.F);
-    if constexpr (K <= 4) pdl_launch_next();  // one or two CTAs; K = 5 took 5 % longer with it
+    pdl_launch_next();
     if constexpr (kSmemMat) stage_matrix<K>(msm, M.p);
 
     const uint32_t tid = threadIdx.x;
@@ -227,8 +229,8 @@ __global__ void __launch_bounds__(tiled_threads(K), tiled_min_blocks(K)) k_apply
 }
 
 // Threads per CTA (log2) of the tiled kernel for width k.
-int tiled_F(int k) { return k <= 4 ? 8 : (k == 5 ? 7 : 6); }
-static_assert(tiled_threads(4) == 256 && tiled_threads(5) == 128 && tiled_threads(6) == 64, "F");
+int tiled_F(int k) { return k <= 4 ? 8 : 6; }
+static_assert(tiled_threads(4) == 256 && tiled_threads(6) == 64, "F");
 
 template <typename Kern>
 cudaError_t ensure_smem(Kern kern, size_t bytes)
@@ -317,6 +319,45 @@ int launch_tiled(float2 *psi, int nbits, const int *tpos, const MatSrc &M, cudaS
     auto kern = k_apply_tiled<K, MatSrc>;
     if (ensure_smem(kern, smem) != cudaSuccess) return -1;
     return launch_pdl(kern, (unsigned)tiles, 1u << g.F, smem, st, g, M) == cudaSuccess ? 0 : -1;
+}
+
+// ---------------------------------------------------------------------------------------
+// k = 5 on 5 to 10 qubits: at most 32 groups, one CTA.  Bound by one chain of FMAs: a thread a group is
+// 4096 of them on one warp, with 8 KiB of constants that miss the cache; eight threads a group take 512
+// each (cl_apply), the matrix read from shared memory.  Sums in the order of the other kernels.
+// Replays of 10-qubit plans, 12 cycles: 73 us by the register kernel, 97 by the tiled one, 27 by this; 7
+// qubits 49, 68, 14.
+// ---------------------------------------------------------------------------------------
+struct CtaGeom {
+    float2 *psi;
+    uint32_t groups;
+    int tpos[kMaxK];
+    uint32_t moff[32];
+};
+
+__global__ void __launch_bounds__(kClThreads) k_apply_cta5(const __grid_constant__ CtaGeom g,
+                                                           const __grid_constant__ MatP<5> M)
+{
+    __shared__ __align__(16) float2 m[1024];
+    pdl_launch_next();  // one CTA: there is room for the next pass to fetch its matrix meanwhile
+    const float2 *src = M.m;
+    asm volatile("" : "+l"(src));  // ordinary loads, not constants (32 addresses a warp)
+    for (int i = threadIdx.x; i < 1024; i += kClThreads) m[i] = src[i];
+    __syncthreads();
+    pdl_wait();
+    cl_apply<5>(g.psi, 0, g.groups, g.tpos, m, g.moff);
+}
+
+int launch_cta5(float2 *psi, int nbits, const int *tpos, const MatP<5> &M, cudaStream_t st)
+{
+    CtaGeom g{};
+    g.psi = psi;
+    g.groups = 1u << (nbits - 5);
+    std::copy(tpos, tpos + 5, g.tpos);
+    for (int j = 0; j < 32; j++)
+        for (int b = 0; b < 5; b++)
+            if ((j >> b) & 1) g.moff[j] += 1u << tpos[b];
+    return launch_pdl(k_apply_cta5, 1, kClThreads, 0, st, g, M) == cudaSuccess ? 0 : -1;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -730,10 +771,10 @@ int launch_param(float2 *psi, int nbits, const int *tpos, const float2 *mat, cud
     }
     if constexpr (K <= 4) {
         if (nbits >= K + 5) return launch_reg<K>(psi, nbits, tpos, M, st);
+        return launch_tiled<K, MatP<K>>(psi, nbits, tpos, M, st);
     } else {
-        if (nbits >= K + kRtF) return launch_rtile<K>(psi, nbits, tpos, M, st);
+        return nbits >= K + kRtF ? launch_rtile<K>(psi, nbits, tpos, M, st) : launch_cta5(psi, nbits, tpos, M, st);
     }
-    return launch_tiled<K, MatP<K>>(psi, nbits, tpos, M, st);
 }
 
 }  // namespace

@@ -59,3 +59,11 @@ def test_every_set_of_low_targets(pkg, oracle_mod, n, k):
             high = list(range(n - 1, n - 1 - (k - j), -1))
             targets = high + list(reversed(low))
             check(pkg, oracle_mod, n, targets, seed=100 * j + sum(low))
+
+
+@pytest.mark.parametrize("n", [5, 6, 7, 8, 9, 10])
+def test_five_qubits_of_a_small_state(pkg, oracle_mod, n):
+    # one CTA: from one group, all rows of which eight threads share, to 32 groups
+    rng = np.random.default_rng(n)
+    for seed in range(3):
+        check(pkg, oracle_mod, n, [int(q) for q in rng.permutation(n)[:5]], seed=10 * n + seed)

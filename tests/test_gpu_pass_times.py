@@ -92,3 +92,23 @@ def test_fp32_blocks_below_one_wave(pkg, stream, kmax, n):
             pkg.sim_plan_destroy(p)
             pkg.sim_destroy(h)
     assert t[1] < 1.28 * t[0], t
+
+
+def test_five_qubit_blocks_below_the_smallest_tile(pkg, stream):
+    # the same blocks on 10 qubits, one CTA, and on 11, one tile: less than the time, 2 times with one
+    # thread to a group
+    import syc_inputs as si
+    gates = pkg.gates_array(si.sycamore_circuit(si.near_square_grid(10), 12, seed=5))
+    t = []
+    for m in (10, 11):
+        h, buf = handle(pkg, stream, m)
+        p = pkg.sim_plan_create(m, gates, kmax=5)
+        try:
+            pkg.sim_reset(h)
+            g = pkg.sim_graph_create(h, p)
+            t.append(us(stream, lambda: pkg.sim_graph_launch(h, g), 20))
+            pkg.sim_graph_destroy(g)
+        finally:
+            pkg.sim_plan_destroy(p)
+            pkg.sim_destroy(h)
+    assert t[0] < 1.4 * t[1], t
