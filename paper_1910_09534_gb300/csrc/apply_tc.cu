@@ -328,7 +328,6 @@ int launch_mma(float2 *psi, int nbits, const int *tpos, const BlockMat<K> &M, cu
     constexpr int D = 1 << K;
     MmaGeom g{};
     g.psi = psi;
-    g.early = pdl_early(nbits);
     g.n_mtiles = 1ull << (nbits - K - 4);
     for (int i = 0; i < K; i++) g.tpos[i] = tpos[i];
     for (int j = 0; j < D; j++) {
@@ -351,7 +350,12 @@ int launch_mma(float2 *psi, int nbits, const int *tpos, const BlockMat<K> &M, cu
     }();
     if (!cfg.ok) return -1;
     const uint64_t need = (g.n_mtiles + 7) / 8;
-    const uint64_t grid = std::min<uint64_t>(need, (uint64_t)cfg.sms * cfg.occ);
+    const uint64_t most = (uint64_t)cfg.sms * cfg.occ, grid = std::min<uint64_t>(need, most);
+    // With room left on the SMs, where several CTAs fit on one (k = 4, 5), the next pass's CTAs crowd
+    // (pdl.cuh): early only with half of the SMs idle or all of the room taken.  Replays of 3xFP16 plans, k =
+    // 5, early / not: 18 qubits (64 CTAs) 60 / 70 us, 19 100 / 76, 20 125 / 106, 21 (all taken) 165 / 174, 24
+    // 864 / 874; k = 6, one CTA an SM, 19 qubits 98 / 112, 20 117 / 127.
+    g.early = pdl_early(nbits) && (cfg.occ == 1 || 2 * grid <= (uint64_t)cfg.sms || grid == most);
     return launch_pdl(kern, (unsigned)grid, 256, kBytes, st, g, M) == cudaSuccess ? 0 : -1;
 }
 
