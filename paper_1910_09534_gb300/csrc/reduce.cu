@@ -25,10 +25,12 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
+// Bound by reading the state.  No trigger for the next launch, whose CTAs would crowd (pdl.cuh): back to
+// back, ordinary launches / with it / without, 2^20 amplitudes 14.4 / 11.2 / 6.6 us, 2^24 28.8 / 31.2 /
+// 24.8, 2^26 86.4 / 86.1 / 82.6.
 __global__ void __launch_bounds__(kReduceThreads) k_reduce_partials(const float4 *psi4, uint64_t n4,
                                                                     double *partials)
 {
-    pdl_launch_next();
     pdl_wait();
     double s1 = 0.0, s2 = 0.0;
     const uint64_t stride = (uint64_t)gridDim.x * kReduceThreads * kReduceUnroll;

@@ -113,3 +113,18 @@ def test_five_qubit_blocks_below_the_smallest_tile(pkg, stream):
             pkg.sim_plan_destroy(p)
             pkg.sim_destroy(h)
     assert t[0] < 1.4 * t[1], t
+
+
+def test_reduction_of_an_l2_sized_state(pkg, stream):
+    # reading 2^24 amplitudes takes 1.35 times as long as writing them, 1.7 where the next call's CTAs crowd
+    import torch
+    n = 24
+    h, buf = handle(pkg, stream, n)
+    out = torch.zeros(3, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+    try:
+        reset = us(stream, lambda: pkg.sim_reset(h), 40)
+        t = us(stream, lambda: pkg.sim_reduce_noalloc(buf.data_ptr(), 1 << n, out.data_ptr(), stream.cuda_stream), 40)
+        assert t < 1.5 * reset, (t, reset)
+    finally:
+        pkg.sim_destroy(h)
