@@ -15,8 +15,8 @@
 //  * direct -- every target >= 5: thread = group; the 32 threads of a warp take 32
 //    consecutive groups, so each member load/store is one contiguous 256-byte run.
 //    Amplitudes go straight to registers; no shared memory.  Used for k <= 3.
-//  * cta -- k = 5 on at most 10 qubits: one CTA, several threads to a group's rows.
-//  * tiled -- the smallest states otherwise: a CTA stages a tile of 2^(F+k) amplitudes (2^h rows of
+//  * cta -- k = 5, 6 on fewer qubits than that: one CTA, several threads to a group's rows.
+//  * tiled -- k <= 4 on fewer than k + 5 qubits: a CTA stages a tile of 2^(F+k) amplitudes (2^h rows of
 //    2^m contiguous amplitudes, the rows indexed by the h targets >= m) through shared
 //    memory with coalesced loads, each of its 2^F threads applies M to one group, and
 //    the tile is written back.  An XOR swizzle maps the low target bits onto free bits
@@ -69,8 +69,8 @@ struct TiledGeom {
     int hpos[kMaxK];     // high target bits (ascending, >= m)
     int nsw;             // swizzle pairs: bit sw_src[i] of a tile position is XORed into bit sw_dst[i]
     int sw_src[4], sw_dst[4];
-    uint32_t soff[64];   // tile-local offset of member j
-    uint64_t rowoff[64]; // global offset of tile row r
+    uint32_t soff[16];   // tile-local offset of member j (k <= 4)
+    uint64_t rowoff[16]; // global offset of tile row r
 };
 
 __device__ __forceinline__ uint64_t insert_zero_bits(uint64_t x, const int *pos, int cnt)
@@ -121,12 +121,12 @@ __device__ __forceinline__ uint32_t swizzle(uint32_t p, const TiledGeom &g)
 
 // y = M x for one group; rows are produced RB at a time (RB independent FMA chains per
 // real/imag part) and handed to `st(row, value)`.
-template <int K, bool kUnrollRows, typename MatAt, typename Store>
+template <int K, typename MatAt, typename Store>
 __device__ __forceinline__ void apply_group(const float2 (&x)[1 << K], MatAt M, Store st)
 {
     constexpr int D = 1 << K;
     constexpr int RB = D >= 4 ? 4 : D;
-#pragma unroll(kUnrollRows ? D / RB : 1)
+#pragma unroll
     for (int r0 = 0; r0 < D; r0 += RB) {
         float yr[RB], yi[RB];
 #pragma unroll
@@ -147,17 +147,7 @@ __device__ __forceinline__ void apply_group(const float2 (&x)[1 << K], MatAt M, 
     }
 }
 
-// Copy a 2^K x 2^K matrix from global memory to shared memory (all threads).
-template <int K>
-__device__ __forceinline__ void stage_matrix(float2 *sm, const float2 *gm)
-{
-    constexpr int N = (1 << K) * (1 << K);
-    for (int i = threadIdx.x; i < N; i += blockDim.x) sm[i] = gm[i];
-    __syncthreads();
-}
-
-// Occupancy targets (CTAs per SM) that bound the register count of each width.
-constexpr int tiled_threads(int k) { return k <= 4 ? 256 : 64; }
+// Occupancy target (CTAs per SM) that bounds the register count of each width.
 constexpr int tiled_min_blocks(int k) { return k == 4 ? 2 : 4; }
 
 template <int K>
@@ -172,20 +162,16 @@ __global__ void __launch_bounds__(256, 4) k_apply_direct(DirectGeom g, MatP<K> M
 #pragma unroll
     for (int j = 0; j < D; ++j) x[j] = __ldcs(p + g.moff[j]);
     float2 *const q = opaque(p);
-    apply_group<K, true>(x, [&](int r, int c) { return M.m[r * D + c]; },
+    apply_group<K>(x, [&](int r, int c) { return M.m[r * D + c]; },
                          [&](int r, float2 y) { __stcs(q + g.moff[r], y); });
 }
 
-template <int K, typename MatSrc>
-__global__ void __launch_bounds__(tiled_threads(K), tiled_min_blocks(K)) k_apply_tiled(TiledGeom g, MatSrc M)
+template <int K>
+__global__ void __launch_bounds__(256, tiled_min_blocks(K)) k_apply_tiled(TiledGeom g, MatP<K> M)
 {
     constexpr int D = 1 << K;
-    constexpr bool kSmemMat = std::is_same<MatSrc, MatPtr>::value;
-    extern __shared__ float2 smem[];
-    float2 *tile = smem;
-    float2 *msm = smem + ((size_t)D << g.F);
+    extern __shared__ float2 tile[];
     pdl_launch_next();
-    if constexpr (kSmemMat) stage_matrix<K>(msm, M.p);
 
     const uint32_t tid = threadIdx.x;
     const int F = g.F;
@@ -211,10 +197,7 @@ __global__ void __launch_bounds__(tiled_threads(K), tiled_min_blocks(K)) k_apply
 #pragma unroll
     for (int j = 0; j < D; ++j) x[j] = tile[sb ^ g.soff[j]];
     auto st = [&](int r, float2 y) { tile[sb ^ g.soff[r]] = y; };
-    if constexpr (kSmemMat)
-        apply_group<K, false>(x, [&](int r, int c) { return msm[r * D + c]; }, st);
-    else
-        apply_group<K, true>(x, [&](int r, int c) { return M.m[r * D + c]; }, st);
+    apply_group<K>(x, [&](int r, int c) { return M.m[r * D + c]; }, st);
     __syncthreads();
 
     // store
@@ -228,9 +211,7 @@ __global__ void __launch_bounds__(tiled_threads(K), tiled_min_blocks(K)) k_apply
     }
 }
 
-// Threads per CTA (log2) of the tiled kernel for width k.
-int tiled_F(int k) { return k <= 4 ? 8 : 6; }
-static_assert(tiled_threads(4) == 256 && tiled_threads(6) == 64, "F");
+constexpr int kTiledF = 8;  // most threads per CTA (log2) of the tiled kernel
 
 template <typename Kern>
 cudaError_t ensure_smem(Kern kern, size_t bytes)
@@ -257,15 +238,13 @@ int launch_direct(float2 *psi, int nbits, const int *tpos, const MatP<K> &M, cud
     return launch_pdl(k_apply_direct<K>, (unsigned)blocks, 256, 0, st, g, M) == cudaSuccess ? 0 : -1;
 }
 
-template <int K, typename MatSrc>
-int launch_tiled(float2 *psi, int nbits, const int *tpos, const MatSrc &M, cudaStream_t st)
+template <int K>
+int launch_tiled(float2 *psi, int nbits, const int *tpos, const MatP<K> &M, cudaStream_t st)
 {
     constexpr int D = 1 << K;
-    constexpr bool kSmemMat = std::is_same<MatSrc, MatPtr>::value;
-    const size_t mat_bytes = kSmemMat ? sizeof(float2) * D * D : 0;
     TiledGeom g{};
     g.psi = psi;
-    g.F = std::min(tiled_F(K), nbits - K);
+    g.F = std::min(kTiledF, nbits - K);
     int m = g.F;
     for (;;) {  // m = F + #(targets below m)
         int below = 0;
@@ -315,49 +294,58 @@ int launch_tiled(float2 *psi, int nbits, const int *tpos, const MatSrc &M, cudaS
         g.rowoff[r] = o;
     }
     const uint64_t tiles = 1ull << (nbits - g.F - K);
-    const size_t smem = (sizeof(float2) << (g.F + K)) + mat_bytes;
-    auto kern = k_apply_tiled<K, MatSrc>;
+    const size_t smem = sizeof(float2) << (g.F + K);
+    auto kern = k_apply_tiled<K>;
     if (ensure_smem(kern, smem) != cudaSuccess) return -1;
     return launch_pdl(kern, (unsigned)tiles, 1u << g.F, smem, st, g, M) == cudaSuccess ? 0 : -1;
 }
 
 // ---------------------------------------------------------------------------------------
-// k = 5 on 5 to 10 qubits: at most 32 groups, one CTA.  Bound by one chain of FMAs: a thread a group is
-// 4096 of them on one warp, with 8 KiB of constants that miss the cache; eight threads a group take 512
-// each (cl_apply), the matrix read from shared memory.  Sums in the order of the other kernels.
-// Replays of 10-qubit plans, 12 cycles: 73 us by the register kernel, 97 by the tiled one, 27 by this; 7
-// qubits 49, 68, 14.
+// k = 5, 6 on fewer qubits than a tile of k_apply_rtile (n < k + 6): at most 32 groups, one CTA.  Bound by
+// one chain of FMAs: a thread a group is 4^(k+1) of them on one warp; 2^k / 4 threads a group (8 where
+// 32 groups of 64 leave no more) take four rows each (cl_apply), the matrix read from shared memory.
+// Sums in the order of the other kernels.  Replays of plans of 5-qubit blocks, 12 cycles: on 10 qubits 73 us
+// by the register kernel, 97 by the tiled one, 27 by this; on 7 qubits 49, 68, 14.  One 6-qubit block, its
+// upload included: 6 qubits 251 -> 15 us, 8 qubits 126 -> 16, 10 and 11 qubits 74, 64 -> 25.
 // ---------------------------------------------------------------------------------------
+template <int K>
 struct CtaGeom {
     float2 *psi;
     uint32_t groups;
     int tpos[kMaxK];
-    uint32_t moff[32];
+    uint32_t moff[1 << K];
 };
 
-__global__ void __launch_bounds__(kClThreads) k_apply_cta5(const __grid_constant__ CtaGeom g,
-                                                           const __grid_constant__ MatP<5> M)
+template <int K, typename MatSrc>
+__global__ void __launch_bounds__(kClThreads) k_apply_cta(const __grid_constant__ CtaGeom<K> g,
+                                                          const __grid_constant__ MatSrc mat)
 {
-    __shared__ __align__(16) float2 m[1024];
+    __shared__ __align__(16) float2 m[1 << (2 * K)];
     pdl_launch_next();  // one CTA: there is room for the next pass to fetch its matrix meanwhile
-    const float2 *src = M.m;
-    asm volatile("" : "+l"(src));  // ordinary loads, not constants (32 addresses a warp)
-    for (int i = threadIdx.x; i < 1024; i += kClThreads) m[i] = src[i];
+    const float2 *src;
+    if constexpr (K == 6) {
+        src = mat.p;
+    } else {
+        src = mat.m;
+        asm volatile("" : "+l"(src));  // ordinary loads, not constants (32 addresses a warp)
+    }
+    for (int i = threadIdx.x; i < 1 << (2 * K); i += kClThreads) m[i] = src[i];
     __syncthreads();
     pdl_wait();
-    cl_apply<5>(g.psi, 0, g.groups, g.tpos, m, g.moff);
+    cl_apply<K>(g.psi, 0, g.groups, g.tpos, m, g.moff);
 }
 
-int launch_cta5(float2 *psi, int nbits, const int *tpos, const MatP<5> &M, cudaStream_t st)
+template <int K, typename MatSrc>
+int launch_cta(float2 *psi, int nbits, const int *tpos, const MatSrc &M, cudaStream_t st)
 {
-    CtaGeom g{};
+    CtaGeom<K> g{};
     g.psi = psi;
-    g.groups = 1u << (nbits - 5);
-    std::copy(tpos, tpos + 5, g.tpos);
-    for (int j = 0; j < 32; j++)
-        for (int b = 0; b < 5; b++)
+    g.groups = 1u << (nbits - K);
+    std::copy(tpos, tpos + K, g.tpos);
+    for (int j = 0; j < (1 << K); j++)
+        for (int b = 0; b < K; b++)
             if ((j >> b) & 1) g.moff[j] += 1u << tpos[b];
-    return launch_pdl(k_apply_cta5, 1, kClThreads, 0, st, g, M) == cudaSuccess ? 0 : -1;
+    return launch_pdl(k_apply_cta<K, MatSrc>, 1, kClThreads, 0, st, g, M) == cudaSuccess ? 0 : -1;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -436,14 +424,14 @@ __global__ void __launch_bounds__(256, reg_min_blocks(K)) k_apply_reg(RegGeom g,
             __syncwarp();
 #pragma unroll
             for (int j = 0; j < D; ++j) x[j] = *reinterpret_cast<const float2 *>(my + (br ^ g.cr[j]));
-            apply_group<K, true>(x, MatAt,
+            apply_group<K>(x, MatAt,
                                  [&](int r, float2 v) { *reinterpret_cast<float2 *>(my + (br ^ g.cr[r])) = v; });
             __syncwarp();
 #pragma unroll
             for (int j = 0; j < D; ++j)
                 __stcs(q + g.xoff[j], *reinterpret_cast<const float2 *>(my + (bw ^ g.cw[j])));
         } else {
-            apply_group<K, true>(x, MatAt, [&](int r, float2 v) { __stcs(q + g.xoff[r], v); });
+            apply_group<K>(x, MatAt, [&](int r, float2 v) { __stcs(q + g.xoff[r], v); });
         }
         if (wn < g.n_wtiles) {
             const float2 *pn = tile_ptr(wn);
@@ -771,9 +759,9 @@ int launch_param(float2 *psi, int nbits, const int *tpos, const float2 *mat, cud
     }
     if constexpr (K <= 4) {
         if (nbits >= K + 5) return launch_reg<K>(psi, nbits, tpos, M, st);
-        return launch_tiled<K, MatP<K>>(psi, nbits, tpos, M, st);
+        return launch_tiled<K>(psi, nbits, tpos, M, st);
     } else {
-        return nbits >= K + kRtF ? launch_rtile<K>(psi, nbits, tpos, M, st) : launch_cta5(psi, nbits, tpos, M, st);
+        return nbits >= K + kRtF ? launch_rtile<K>(psi, nbits, tpos, M, st) : launch_cta<K>(psi, nbits, tpos, M, st);
     }
 }
 
@@ -790,7 +778,7 @@ int launch_apply_fp32(sim_t *, float2 *psi, int nbits, int k, const int *tpos, c
     case 5: return launch_param<5>(psi, nbits, tpos, mat, st);
     case 6:
         if (nbits >= 6 + kRtF) return launch_rtile<6>(psi, nbits, tpos, MatPtr{mat6_dev}, st);
-        return launch_tiled<6, MatPtr>(psi, nbits, tpos, MatPtr{mat6_dev}, st);
+        return launch_cta<6>(psi, nbits, tpos, MatPtr{mat6_dev}, st);
     default: return -1;
     }
 }

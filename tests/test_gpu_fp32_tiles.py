@@ -61,9 +61,9 @@ def test_every_set_of_low_targets(pkg, oracle_mod, n, k):
             check(pkg, oracle_mod, n, targets, seed=100 * j + sum(low))
 
 
-@pytest.mark.parametrize("n", [5, 6, 7, 8, 9, 10])
-def test_five_qubits_of_a_small_state(pkg, oracle_mod, n):
-    # one CTA: from one group, all rows of which eight threads share, to 32 groups
+@pytest.mark.parametrize("k,n", [(k, n) for k in (5, 6) for n in range(k, k + 6)])
+def test_wide_blocks_of_a_small_state(pkg, oracle_mod, k, n):
+    # one CTA: from one group, whose rows 8 or 16 threads share, to 32 groups
     rng = np.random.default_rng(n)
     for seed in range(3):
-        check(pkg, oracle_mod, n, [int(q) for q in rng.permutation(n)[:5]], seed=10 * n + seed)
+        check(pkg, oracle_mod, n, [int(q) for q in rng.permutation(n)[:k]], seed=10 * n + seed)

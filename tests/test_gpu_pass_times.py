@@ -95,15 +95,17 @@ def test_blocks_below_one_wave(pkg, stream, precision, kmax, n, bound):
     assert t[1] < bound * t[0], t
 
 
-def test_five_qubit_blocks_below_the_smallest_tile(pkg, stream):
-    # the same blocks on 10 qubits, one CTA, and on 11, one tile: less than the time, 2 times with one
-    # thread to a group
+@pytest.mark.parametrize("kmax", [5, 6])
+def test_wide_blocks_below_the_smallest_tile(pkg, stream, kmax):
+    # the same blocks on the most qubits that one CTA takes, and on one more, one tile: less than the time,
+    # 2-3 times with one thread to a group
     import syc_inputs as si
-    gates = pkg.gates_array(si.sycamore_circuit(si.near_square_grid(10), 12, seed=5))
+    n = kmax + 5
+    gates = pkg.gates_array(si.sycamore_circuit(si.near_square_grid(n), 12, seed=5))
     t = []
-    for m in (10, 11):
+    for m in (n, n + 1):
         h, buf = handle(pkg, stream, m)
-        p = pkg.sim_plan_create(m, gates, kmax=5)
+        p = pkg.sim_plan_create(m, gates, kmax=kmax)
         try:
             pkg.sim_reset(h)
             g = pkg.sim_graph_create(h, p)
