@@ -47,15 +47,16 @@ static int plan_ctas()
     return wide.load(std::memory_order_acquire) & bit ? 16 : 8;
 }
 
-// Where one cluster is faster than a launch per block on all SMs.  Measured (12 cycles, us a plan,
-// cluster of 16 / of 8 / separate launches from a CUDA graph): k_max 4: 12 qubits 23 / 25 / 45, 14
-// qubits 39 / 41 / 63, 15 qubits 48 / 67 / 76, 16 qubits 60 / 101 / 74, 17 qubits 121 / 215 / 89; k_max
-// 5, whose separate kernel is slow to start: 14 qubits 50 / 68 / 158, 16 qubits 87 / 131 / 230, 17 qubits
-// 138 / 246 / 230, 18 qubits 280 / 524 / 259.
+// Where one cluster is faster than a launch per block on all SMs.  Measured (20 cycles, us a plan, cluster
+// of 16 / of 8 / separate launches): k_max 4: 12 qubits 37 / 39 / 59, 14 qubits 58 / 66 / 76, 15 qubits 81 /
+// 105 / 90, 16 qubits 88 / 150 / 82; k_max 5, whose separate blocks several threads a group share: 12
+// qubits 45 / 50 / 65, 13 qubits 51 / 67 / 52, 14 qubits 73 / 83 / 65; k_max 3: 13 qubits 57 / 63 / 65,
+// 14 qubits 74 / 81 / 76 and a plan alone on the device 87 / 95 / 85; k_max 2: 13 qubits 133 / 139 / 149,
+// 14 qubits 158 / 181 / 169, 15 qubits 205 / 284 / 189.
 bool plan_cluster_eligible(int n, int nblocks, int max_k)
 {
     if (nblocks < 2 || max_k > kClMaxK) return false;
-    const int top = max_k == 5 ? 17 : 16;
+    const int top = max_k == 4 ? 15 : 13;
     return n <= top - 1 || (n <= top && plan_ctas() == 16);
 }
 

@@ -79,8 +79,8 @@ def test_packed_serving_reports_a_refused_launch(refusing_lib, after):
 
 
 PLAN = """
-for n, kmax in ((6, 3), (12, 4), (14, 5), (16, 5)):
-    c = si.sycamore_circuit(si.near_square_grid(n), 8, seed=n)
+for n, kmax in ((6, 3), (12, 4), (13, 5), (15, 4)):
+    c = si.sycamore_circuit(si.near_square_grid(n), 20, seed=n)
     p = pkg.sim_plan_create(n, pkg.gates_array(c), kmax=kmax)
     h = pkg.sim_create(n)
     pkg.sim_apply_plan(h, p)
