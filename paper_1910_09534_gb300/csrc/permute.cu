@@ -151,17 +151,19 @@ __device__ __forceinline__ uint64_t perm_now_ns()
 // amplitudes in place with 0-3 row bits 606-630 / 660-685, with 4, 5 (rows of 256-512 bytes) 727, 737 /
 // 670-690; tile pairs with no row bits, 2^30 1225 / 1322, 2^28 575 / 590; pairs of 2^11 with rows of 1 KiB 687
 // / 740, of 2^10 809 / 690, with shorter rows 973-1286 / 690-711.
-// It lets no kernel start early, nor does k_permute_pass: a CTA a tile, most of which only find that
-// nothing moves, and each paid for the trigger (bits 26 and 27 of 2^28 amplitudes: 497 us, without 400; of
-// 2^24 21.9, 17.6).
+// A CTA a tile, most of which may only find that nothing moves, and each pays for the trigger of the next
+// launch: a swap of the two highest of 28 bits (2^18 CTAs) 497 us with it, 400 without, of 24 bits (2^14)
+// 21.9, 17.6, of 22 bits (2^12) 8.7, 8.8; random permutations of 21-22 bits 1-3 % faster with it.
 // The only wait (the copies' mbarrier) is bounded by %globaltimer: on a timeout the CTA records the
 // failure, writes nothing back and waits (again bounded) for its copies before leaving.
+constexpr unsigned kPermEarlyCtas = 4096;
 __global__ void __launch_bounds__(256) k_permute_tile_bulk(PermGeom g, int *err)
 {
     extern __shared__ __align__(128) float2 tile[];
     __shared__ __align__(8) uint64_t bar;
     __shared__ uint32_t p_it[64], sig_it[64];  // the iteration part of p, and its image under sig
     __shared__ int ok;
+    if (gridDim.x <= kPermEarlyCtas) pdl_launch_next();
     const int nloc = g.LB + g.q, T = 1 << nloc;
     const uint32_t row_bytes = 8u << g.LB;
     const uint64_t base = insert_zero_bits_p((uint64_t)blockIdx.x << g.LB, g.rowpos, g.q);
@@ -281,7 +283,7 @@ __global__ void __launch_bounds__(256) k_permute_tile_bulk(PermGeom g, int *err)
 // of 2^24 127-141 -> 85-94 us.  The kernel before, one CTA a tile pair and 4 amplitudes a thread, was
 // issue-bound (76 %) on setting up its maps.
 // Every wait is bounded by %globaltimer, from when the kernels before have ended: on a timeout the
-// kernel records the failure, every role leaves, and the producer waits (again bounded) for its copies.
+// kernel records the failure, every role leaves, and the CTA waits (again bounded) for its own copies.
 constexpr int kPtRing = 98304;                    // bytes of stages (64 KiB: 10-20 % slower); a stage is one tile or a tile pair
 constexpr int kPtMaxStages = 16;
 constexpr int kPtGroups = 2;                      // swapper groups, a stage to each in turn
@@ -366,7 +368,6 @@ __global__ void __launch_bounds__(kPtThreads, 2) k_permute_tma(const __grid_cons
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
     }
     __syncthreads();
-    pdl_wait();  // every role: the waits' time limits count from here, not from an early start
     volatile int *ab = &abort_flag;
     auto give_up = [&]() {
         *ab = 1;
@@ -398,8 +399,12 @@ __global__ void __launch_bounds__(kPtThreads, 2) k_permute_tma(const __grid_cons
                          : "memory");
     };
 
+    uint32_t issued = 0, marked = 0;  // thread 0: items loaded, end marks behind them
     if (warp == 0) {
         // ---------------- producer ----------------
+        // Every role waits for the work before first, each after its own set-up, so that its waits' time
+        // limits do not count from an early start.
+        pdl_wait();
         uint32_t it = 0;
         bool stop = false;
         for (uint64_t c0 = (uint64_t)blockIdx.x * g.per; c0 < g.n_tiles && !stop; c0 += (uint64_t)gridDim.x * g.per) {
@@ -450,18 +455,12 @@ __global__ void __launch_bounds__(kPtThreads, 2) k_permute_tma(const __grid_cons
                 asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(perm_smem(&full[e % S])) : "memory");
             }
             if (marks < (uint32_t)kPtGroups) give_up();
-            // No copy may still be writing a stage when the CTA leaves, whichever role gave up and when
-            // (the storer and the swappers, which otherwise wait for every copy, may already be gone).
-            // The barriers of items older than these have been moved on by later copies or end marks,
-            // which waited until those items had been stored.
-            for (uint32_t j = it + marks > S ? it + marks - S : 0; j < it; ++j) {
-                const uint64_t t0 = perm_now_ns();
-                while (!perm_try(perm_smem(&full[j % S]), (j / S) & 1, 20000) && perm_now_ns() - t0 <= kPtWaitNs) {
-                }
-            }
+            issued = it;
+            marked = marks;
         }
     } else if (warp == 1) {
         // ---------------- storer ----------------
+        pdl_wait();
         uint32_t it = 0;
         for (;; ++it) {
             const uint32_t st = it % S;
@@ -497,6 +496,7 @@ __global__ void __launch_bounds__(kPtThreads, 2) k_permute_tma(const __grid_cons
                 pt ^= g.tp[j];
                 qt ^= g.tq[j];
             }
+        pdl_wait();
         // a group takes the items congruent to its number, the last of them an end mark
         for (uint32_t it = grp;; it += kPtGroups) {
             const uint32_t st = it % S;
@@ -522,6 +522,16 @@ __global__ void __launch_bounds__(kPtThreads, 2) k_permute_tma(const __grid_cons
             if ((tid & 31) == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];\n" ::"r"(perm_smem(&swapped[st])) : "memory");
         }
     }
+    // No copy may still be writing a stage when the CTA leaves.  The storer has waited for every one, unless
+    // a role gave up: then those whose barriers have not moved on (by later copies or end marks, which
+    // waited until the older items were stored) are waited for here, after the last role.
+    __syncthreads();
+    if (tid == 0 && *ab)
+        for (uint32_t j = issued + marked > S ? issued + marked - S : 0; j < issued; ++j) {
+            const uint64_t t0 = perm_now_ns();
+            while (!perm_try(perm_smem(&full[j % S]), (j / S) & 1, 20000) && perm_now_ns() - t0 <= kPtWaitNs) {
+            }
+        }
 }
 
 // One involution pass; inv[b] = partner of bit b (inv[b] == b: fixed).
