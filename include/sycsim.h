@@ -308,8 +308,11 @@ int sim_apply_plan(sim_t *h, const sim_plan_t *p);
 /* ---- CUDA graphs (not in the paper) ----------------------------------------
  * Capture the block launches of a plan on h once and replay them.  For a plan run many times
  * (the same circuit from several initial states, repeated runs) a replay skips the per-block host
- * work -- matrix rounding, operand staging, the launch itself -- which dominates below ~2^20
- * amplitudes.  The 6-qubit blocks' matrices are uploaded once into device memory that the graph
+ * work -- matrix rounding, operand staging, the launch itself: 12-25 % of a run of 6-qubit blocks on
+ * 2^12 to 2^20 amplitudes, 10-30 % of one of 2-qubit blocks, less than 10 % of the others.  A graph
+ * holds one launch a block: FP32 plans of 4- and 5-qubit blocks on up to 13-15 qubits run faster
+ * through sim_apply_plan, which gives one cluster of CTAs many blocks a launch (12 qubits, k_max 4:
+ * 23 us, its replay 37).  The 6-qubit blocks' matrices are uploaded once into device memory that the graph
  * owns (narrower blocks carry theirs in the captured launches).  A graph is bound to h (its state
  * buffer, stream and layout): sim_graph_launch refuses with SIM_E_INVAL on another handle or
  * once h's layout has changed (sim_permute), and a graph must be destroyed before its handle.
@@ -320,7 +323,7 @@ int sim_apply_plan(sim_t *h, const sim_plan_t *p);
  * GB300 depends on which physical bits a block targets: in SIM_FP16X3_TMEM, 5- and 6-qubit blocks
  * with two or more targets below bit 4 (and 4-qubit blocks with one) leave the tcgen05 kernel for
  * a slower one, and tcgen05 blocks with no target below bit 8 move their tiles in 1 KiB pieces
- * instead of 2 KiB; in SIM_FP32 targets below bit 5 cost register exchanges.  sim_plan_layout
+ * instead of 2 KiB; in SIM_FP32 targets below bit 5 are exchanged between lanes.  sim_plan_layout
  * searches layouts (pairwise swaps from 4 seeded starts) for the smallest sum over the
  * plan's blocks of a per-pass time estimate (measured per kernel path on 2^30 amplitudes; other
  * precisions: every layout costs the same and the identity is returned), and writes perm[q] = the

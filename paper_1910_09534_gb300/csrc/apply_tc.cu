@@ -361,14 +361,15 @@ int launch_mma(float2 *psi, int nbits, const int *tpos, const BlockMat<K> &M, cu
 
 }  // namespace
 
-// Measured on GB300 (n = 30): for k = 4 the CUDA-core FP32 kernel is faster than every
-// tensor-core mode (2.8 ms vs >= 3.6 ms per pass), for k >= 5 the tensor cores win (3xFP16 k = 5:
-// 3.3 ms vs 7.0 ms).  Any target set works: groups map to amplitude offsets by bit insertion.
+// Measured on GB300 (n = 30, ms a pass): for k >= 5 the tensor cores win (3xFP16 k = 5 2.8-3.3, CUDA-core
+// FP32 5.7; k = 6 4.5-5.1, 10.6).  k = 4 stays on CUDA cores in these modes (2.81 with every target at bit 5
+// and above, 3.18-3.20 otherwise): the tensor-core kernels took 3.6 and more when the rule was made
+// (3xFP16 with a low target: below).  Any target set works: groups map to amplitude offsets by bit insertion.
 bool tc_eligible(int nbits, int k, const int *) { return k >= 5 && k <= 6 && nbits >= k + 4; }
 
 // In SIM_FP16X3_TMEM mode the blocks the tcgen05 kernel leaves (targets in the low bits) come
 // here for k = 4 too: measured on 2^30 amplitudes, targets {0,1,2,3}: 2.73 ms (CUDA-core FP32
-// 4.27 ms), {0,2,6,8}: 2.59 ms (3.57), {1,6,7,12}: 2.60 ms (3.24).
+// 3.18 ms), {0,2,6,8}: 2.60 ms (3.19), {1,6,7,12}: 2.61 ms (3.20).
 bool tc_eligible_low4(int nbits, int k) { return k == 4 && nbits >= k + 4; }
 
 int launch_apply_tc(float2 *psi, int nbits, int k, const int *tpos, const float2 *mat, const float2 *mat6_dev,

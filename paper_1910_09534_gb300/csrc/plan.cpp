@@ -584,9 +584,11 @@ namespace {
 
 // Estimated time of one fused pass over 2^30 amplitudes (ms) on the kernel a block of k targets at
 // physical bits tpos takes, from CUDA-event timings of each kernel path on GB300; the layout search
-// only compares sums of these.  The entries for FP32 blocks of 4-6 qubits and tcgen05 blocks of 4 and 5
-// stem from earlier forms of those kernels (k = 5 in FP32 takes 5.7 ms now with any targets): a plan's
-// layout, and with it the last bits of its results, stays what it was.
+// only compares sums of these.  The entries for FP32 blocks and tcgen05 blocks of 4 and 5 qubits stem
+// from earlier forms of those kernels, and the layouts have not been searched again with the costs of
+// the present ones: FP32 k <= 3 2.43-2.53 with every target at bit 5 and above, else 2.58-2.81, k = 4 2.81 and
+// 3.18-3.20, k = 5 5.7, k = 6 10.6 whatever the targets; tcgen05 k = 4 2.88, k = 5 2.64-2.70; mma.sync 3xFP16
+// k = 4 2.60-2.73, k = 5 2.76-3.26.
 double pass_ms(int k, const int *tpos, int precision)
 {
     int low4 = 0, low5 = 0;
@@ -607,8 +609,8 @@ double pass_ms(int k, const int *tpos, int precision)
         return 2.45;
     }
     if (precision == SIM_FP32) {
-        // register kernel: each target below bit 5 costs warp exchanges (k = 4: 2.79 ms with none,
-        // 3.3 mixed, 4.3 all low); k >= 5 is FP32-ALU bound whatever the targets
+        // register kernel: targets below bit 5 are exchanged between lanes (as shuffles, which these
+        // costs are of: k = 4 2.79 ms with none, 3.3 mixed, 4.3 all low); k >= 5 is FP32-ALU bound
         if (k >= 5) return 6.9;
         if (k == 4) return low5 == 0 ? 2.79 : (low5 >= 4 ? 4.29 : 3.30);
         return low5 == 0 ? 2.45 : 2.90;

@@ -15,9 +15,9 @@
 //    running workers have fewer clusters than jobs waiting), and a worker leaves after 200 us without
 //    new work, so small circuits that arrive while others run start without a new launch;
 //  * runs larger circuits on one of several slot streams with stream-ordered allocation, so
-//    circuits of different sizes overlap on the device; their blocks are enqueued a few at a
-//    time, as far as the slot's matrix-staging ring has free slots, so the scheduler never
-//    waits on device progress;
+//    circuits of different sizes overlap on the device; their blocks are enqueued in one turn, up
+//    to the first 6-qubit block whose matrix finds no free slot in the staging ring (narrower
+//    blocks carry theirs in the launch), so the scheduler never waits on device progress;
 //  * detects completion by polling events, frees memory and budget, and wakes waiters.
 // Results (norm, 2^n sum p^2, XEB; optionally all amplitudes into the caller's buffer) and
 // latencies (submit -> completion seen) are recorded; srv_stats reports p50/p99 and circuits/s.
@@ -866,7 +866,7 @@ void scheduler(srv_t *s)
             if (!first_blocked) first_blocked = r;
             ++it;
         }
-        // stream-path requests: enqueue what the staging rings allow
+        // stream-path requests: enqueue what the staging rings of 6-qubit matrices allow
         for (size_t i = 0; i < s->slots.size(); i++) {
             auto r = s->slot_req[i];
             if (!r || r->launched) continue;
