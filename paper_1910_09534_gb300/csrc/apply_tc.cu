@@ -323,7 +323,7 @@ template <int K, bool kSplit>
 constexpr size_t mma_bytes() { return sizeof(uint32_t) * (kSplit ? 2 : 1) * ((1 << K) / 4) * ((1 << K) / 4) * 64; }
 
 template <int K, size_t kBytes, void (*kern)(const MmaGeom, const BlockMat<K>)>
-int launch_mma(float2 *psi, int nbits, const int *tpos, const BlockMat<K> &M, cudaStream_t st)
+int launch_mma(float2 *psi, int nbits, const int *tpos, const BlockMat<K> &M, int precision, cudaStream_t st)
 {
     constexpr int D = 1 << K;
     MmaGeom g{};
@@ -354,8 +354,10 @@ int launch_mma(float2 *psi, int nbits, const int *tpos, const BlockMat<K> &M, cu
     // With room left on the SMs, where several CTAs fit on one (k = 4, 5), the next pass's CTAs crowd
     // (pdl.cuh): early only with half of the SMs idle or all of the room taken.  Replays of 3xFP16 plans, k =
     // 5, early / not: 18 qubits (64 CTAs) 60 / 70 us, 19 100 / 76, 20 125 / 106, 21 (all taken) 165 / 174, 24
-    // 864 / 874; k = 6, one CTA an SM, 19 qubits 98 / 112, 20 117 / 127.
-    g.early = pdl_early(nbits) && (cfg.occ == 1 || 2 * grid <= (uint64_t)cfg.sms || grid == most);
+    // 864 / 874; k = 6, one CTA an SM, 19 qubits 98 / 112, 20 117 / 127.  In the tcgen05 modes the next pass
+    // is mostly one of those kernels, of which one CTA fills an SM: always early (reset and plan, 14
+    // cycles, k_max 6, 19 qubits 119 / 124, 20 146 / 148).
+    g.early = pdl_early(nbits) && (tmem_mode(precision) || cfg.occ == 1 || 2 * grid <= (uint64_t)cfg.sms || grid == most);
     return launch_pdl(kern, (unsigned)grid, 256, kBytes, st, g, M) == cudaSuccess ? 0 : -1;
 }
 
@@ -378,10 +380,10 @@ int launch_apply_tc(float2 *psi, int nbits, int k, const int *tpos, const float2
     auto go = [&](auto kc) {
         constexpr int K = decltype(kc)::value;
         const BlockMat<K> M = block_mat<K>(mat, mat6_dev);
-        if (f16x3_mode(precision)) return launch_mma<K, f16x3_bytes<K>(), k_apply_mma_f16x3<K>>(psi, nbits, tpos, M, st);
+        if (f16x3_mode(precision)) return launch_mma<K, f16x3_bytes<K>(), k_apply_mma_f16x3<K>>(psi, nbits, tpos, M, precision, st);
         if (precision == SIM_TF32X3)
-            return launch_mma<K, mma_bytes<K, true>(), k_apply_mma<K, true>>(psi, nbits, tpos, M, st);
-        return launch_mma<K, mma_bytes<K, false>(), k_apply_mma<K, false>>(psi, nbits, tpos, M, st);
+            return launch_mma<K, mma_bytes<K, true>(), k_apply_mma<K, true>>(psi, nbits, tpos, M, precision, st);
+        return launch_mma<K, mma_bytes<K, false>(), k_apply_mma<K, false>>(psi, nbits, tpos, M, precision, st);
     };
     switch (k) {
     case 4: return go(std::integral_constant<int, 4>{});

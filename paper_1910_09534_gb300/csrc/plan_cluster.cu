@@ -51,12 +51,12 @@ static int plan_ctas()
 // of 16 / of 8 / separate launches): k_max 4: 12 qubits 37 / 39 / 59, 14 qubits 58 / 66 / 76, 15 qubits 81 /
 // 105 / 90, 16 qubits 88 / 150 / 82; k_max 5, whose separate kernel keeps up with one tile a CTA: 12
 // qubits 45 / 50 / 65, 13 qubits 51 / 67 / 52, 14 qubits 73 / 83 / 65; k_max 3: 13 qubits 57 / 63 / 65,
-// 14 qubits 74 / 81 / 76 and a plan alone on the device 87 / 95 / 85; k_max 2: 13 qubits 133 / 139 / 149,
-// 14 qubits 158 / 181 / 169, 15 qubits 205 / 284 / 189.
+// 14 qubits 74 / 81 / 76, 15 qubits 90 / 129 / 83; k_max 2: 13 qubits 133 / 139 / 149, 14 qubits 158 / 181 /
+// 169, 15 qubits 205 / 284 / 189.
 bool plan_cluster_eligible(int n, int nblocks, int max_k)
 {
     if (nblocks < 2 || max_k > kClMaxK) return false;
-    const int top = max_k == 4 ? 15 : 13;
+    const int top = max_k == 4 ? 15 : (max_k == 5 ? 13 : 14);
     return n <= top - 1 || (n <= top && plan_ctas() == 16);
 }
 

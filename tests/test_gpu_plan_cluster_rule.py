@@ -15,7 +15,7 @@ def pkg():
     return p
 
 
-@pytest.mark.parametrize("kmax,n,cluster", [(2, 12, True), (2, 14, False), (3, 12, True), (3, 14, False), (4, 14, True),
+@pytest.mark.parametrize("kmax,n,cluster", [(2, 13, True), (2, 15, False), (3, 13, True), (3, 15, False), (4, 14, True),
                                             (4, 16, False), (5, 12, True), (5, 14, False), (5, 17, False),
                                             (6, 12, False)])
 def test_launches_of_a_plan(pkg, kmax, n, cluster):
