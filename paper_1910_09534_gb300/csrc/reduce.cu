@@ -148,9 +148,14 @@ __global__ void k_gather_region(float2 *base, uint64_t lo, uint64_t hi, float2 *
 // |phys> into a state of 2 n4 amplitudes: zeros and the one, in one launch and one write of the state.
 // Bound by the writes.  Four 16-byte stores a thread and as many CTAs as that takes: 278 us for 2^28
 // amplitudes (a memset 284; 8 CTAs an SM looping over the state 325), 552 for 2^29 (557; 649), 18.4 for
-// 2^24 (24; 21).  No trigger for the next launch: it would cost each of these short CTAs.
+// 2^24 (24; 21).  The next launch is triggered only from half of the SMs at most (2^17 amplitudes), where a
+// tensor-core pass sets up meanwhile: reset and a 3xFP16 plan of 5-qubit blocks, 20 cycles, on 13 qubits
+// 65.6 us, 67.0 without, on 15 92.3, 93.1; on more SMs the next pass's CTAs crowd (pdl.cuh): reset and an
+// FP32 plan, 14 cycles, k_max 5, on 19 qubits 115, 94 without.
+constexpr unsigned kResetEarlyCtas = 76;
 __global__ void __launch_bounds__(256) k_reset(float4 *psi4, uint64_t n4, uint64_t phys)
 {
+    if (gridDim.x <= kResetEarlyCtas) pdl_launch_next();
     pdl_wait();
     const uint64_t one = phys >> 1;
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (uint64_t)gridDim.x * blockDim.x) {
